@@ -53,12 +53,15 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
     bdir.mkdir(parents=True, exist_ok=True)
     headers = list(CSRC.glob("*.cuh")) + [ROOT / "include" / "cwthf.h"]
     srcs = sources()
-    objs = [bdir / (s.stem + ".o") for s in srcs]
+    # the FFT sources hold no checked indices (every index there comes from loop
+    # bounds): the checked library links the plain objects
+    objs = [(BUILD if s.stem.startswith("fft") else bdir) / (s.stem + ".o") for s in srcs]
     extra = (["-Xptxas", "-v"] if ptxas_info else []) + (["-DCWTHF_CHECKED"] if checked else [])
 
     def compile_one(pair):
         src, obj = pair
-        if not force and not ptxas_info and not _stale(obj, [src, *headers]):
+        shared = checked and obj.parent == BUILD
+        if (not force or shared) and not ptxas_info and not _stale(obj, [src, *headers]):
             return ""
         cmd = [nvcc(), *flags(extra), "-c", str(src), "-o", str(obj)]
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -66,10 +69,12 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
             raise RuntimeError(f"nvcc failed for {src.name}:\n{r.stderr}")
         return r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 4)) as ex:
-        logs = list(ex.map(compile_one, zip(srcs, objs)))
+    # the longest compilations first
+    jobs = sorted(zip(srcs, objs), key=lambda j: not j[0].stem.startswith("fft_"))
+    with cf.ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 4)) as ex:
+        logs = list(ex.map(compile_one, jobs))
     if verbose or ptxas_info:
-        for s, log in zip(srcs, logs):
+        for (s, _), log in zip(jobs, logs):
             if log:
                 print(f"--- {s.name}\n{log}")
     if force or _stale(out, objs):
@@ -83,9 +88,8 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
 
 
 def build_all(force: bool = False) -> list[Path]:
-    """The library and its checked variant, compiled side by side."""
-    with cf.ThreadPoolExecutor(max_workers=2) as ex:
-        return list(ex.map(lambda c: build(force=force, checked=c), (False, True)))
+    """The library, then its checked variant (which shares the FFT objects)."""
+    return [build(force=force), build(force=force, checked=True)]
 
 
 if __name__ == "__main__":
