@@ -287,8 +287,7 @@ def algorithmic_bytes(name, u):
         "k_fft_x_fwd": 8 * cells + 8 * half,      # int64 grid in, half spectrum out
         "k_fft_yz": 2 * 8 * half,                 # half spectrum in and out
         "k_fft_x_inv": 8 * half + 4 * cells,      # half spectrum in, fp32 CWT out
-        "k_seg_parent": 4 * cells,                # CWT in
-        "k_seg_chase": 4 * cells,                 # labels out
+        "k_seg_tile": 8 * cells,                  # CWT in, labels out
         "k_halo_sums": 12 * npart + 4 * npart,    # positions (as binned records), label gather
         "k_finalize": 4 * npart * u["scales"],    # halo ids out, every scale
     }

@@ -7,12 +7,9 @@
 // C > cwt_min is a seed; the label of a cell is the seed its parent chain
 // reaches, or -1 when the chain ends at a maximum that is not a seed.
 //
-// k_seg_parent finds every cell's parent and writes it as a one-byte code
-// (the offset along each axis, a maximum flag, a seed flag): each thread keeps
-// a column of rows in registers and walks along z, so the 27-cell search needs
-// no shared memory and no barrier.  k_seg_chase loads a tile's codes into
-// shared memory as parent pointers and resolves every chain that stays inside
-// the tile.  A chain that leaves the tile is written as a flagged pointer
+// k_seg_tile finds the parents of a tile's cells and keeps them as pointers in
+// shared memory, resolves every chain that stays inside the tile, and writes
+// the labels.  A chain that leaves the tile is written as a flagged pointer
 // (-2 - g) to the first cell g outside; the global pass then replaces flagged
 // pointers by the label of their target (bounded walks, then, only if a chain
 // outlived them, pointer-doubling rounds in one cooperative launch; hitting the
@@ -20,424 +17,330 @@
 // depend on update order: every update moves a pointer further along the
 // (unique) chain.
 #include <cuda/atomic>
-#include <type_traits>
 
 #include "internal.cuh"
 
 namespace cwthf {
 namespace {
 
-// Chain tiles: 64 x 16 x 16 cells, one warp per row of 64 columns, each lane
-// owning two adjacent columns (one 2-byte code load, one 8-byte pointer and
-// label store per cell pair).  Shared parent pointers use the local index
-// (lz * 16 + ly) * 64 + lx, so local coordinates come back with shifts and
-// masks.  A tile row's flagged cells go out as 32 masks: word 2 lz + p holds
-// plane lz's columns of parity p (bit = lane).
+// Chain tiles: 64 x 16 x 16 cells.  A warp owns kSegRows rows of 64 columns in
+// every plane, each lane two adjacent columns.  A tile row's flagged cells go
+// out as 32 masks: word 2 lz + p holds plane lz's columns of parity p (bit =
+// lane).
 constexpr int kChTX = 64, kChTY = 16, kChTZ = 16;
-constexpr int kChThreads = 32 * kChTY;  // 512
-constexpr int kPX = 64, kPXBits = 6;
-constexpr int kPlaneL = kPX * kChTY, kPlaneBits = 10;
-constexpr int kLocal = kPlaneL * kChTZ;  // 16384 entries
-constexpr int kRowWords = 2 * kChTZ;     // flagged-cell masks per tile row (32)
-static_assert(kChTX == kPX && kPlaneL == (1 << kPlaneBits) && kRowWords == 32, "local index layout");
+constexpr int kRowWords = 2 * kChTZ;  // flagged-cell masks per tile row (32)
+constexpr int kSegRows = 2, kSegThreads = 32 * (kChTY / kSegRows);  // 256
+static_assert(kRowWords == 32 && kChTX == 64, "mask layout");
+// Shared-memory pointers: the 16-bit byte offset of the target's own entry, in
+// a box with one cell of halo on each side (rows padded to 68 entries, so that
+// a lane's column pair is 4-byte aligned); a root points at itself.  One more
+// entry stands for "no seed".
+constexpr int kSRow = 2 * (kChTX + 4), kSPlane = kSRow * (kChTY + 2);  // bytes
+constexpr int kSNone = kSPlane * (kChTZ + 2), kSBytes = kSNone + 8;
+static_assert(kSBytes < 65536 && kSRow == 136 && kSPlane == 2448, "16-bit offsets; quotients below");
 // A flagged pointer (a chain still to be followed) to cell g is stored as
 // -2 - g, apart from -1 (no seed) and the final labels (seed cells, >= 0).
 __device__ __forceinline__ bool is_flagged(int32_t v) { return v <= -2; }
 __device__ __forceinline__ int32_t flag_target(int32_t v) { return -2 - v; }
-constexpr int kJumpRoundsInTile = 16;  // in-place jumping rounds (each at least doubles the distance): 2^14 >= cells of a tile
+constexpr int kJumpRoundsInTile = 16;  // in-place jumping rounds (each triples the distance)
 // Seeds of one tile: at most one local maximum per 2 x 2 x 2 block of cells
 // (any two cells of such a block are neighbours).
 constexpr int kTileSeedCap = (kChTX / 2) * (kChTY / 2) * (kChTZ / 2);
-constexpr int32_t kLocalMask = 0xffff;  // local index bits of a shared-memory pointer
-constexpr int kCountShift = 16;         // a seed's in-tile cell count rides above them
+// pointers, the tile's seeds (offsets), their cell counts (16 bits each: a tile has 2^14 cells), rows
+constexpr int kSegLines = (kChTY + 2) * (kChTZ + 2);  // rows of the box, with their global indices
+constexpr int kSegSmem = kSBytes + 2 * kTileSeedCap + 2 * kTileSeedCap + 4 * kSegLines;
 
-// Parent codes: bits 0-1 / 2-3 / 4-5 the offset + 1 along x / y / z; a local
-// maximum has offsets (0, 0, 0); bit 6 marks a maximum that seeds a halo.
-constexpr uint8_t kCodeMax = 0x15, kCodeSeed = 0x40;
-
-// Parent-code blocks: a warp owns 30 columns (lanes 1-30; lanes 0 and 31 hold
-// the x-halo columns) x kParR rows (plus the two y-halo rows) x kParZ planes
-// (plus one halo plane at each end), streamed through a ring of kParStages
-// planes in shared memory.
-constexpr int kParR = 4, kParZ = 128, kParWarps = 4, kParStages = 6, kParBlocks = 6;
-constexpr int kParThreads = 32 * kParWarps;
+// o / kSRow for offsets o <= kSNone
+constexpr uint32_t kYMul = 30841;
+constexpr int kYShift = 22;
 
 __device__ __forceinline__ int wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-// Search codes of the three candidates (-1, 0, +1) along one axis: rank of
-// the wrapped coordinate (0 = smallest) times 4 plus the candidate's position.
-// The smallest code among the candidates holding the maximum is the winner
-// under the strict order; kNoMatch (only reached when the window holds no
-// comparable value, i.e. NaN input) decodes to the centre.
-constexpr int kNoMatch = 13;
-__device__ __forceinline__ void codes3(int m, int c, int p, int& km, int& kc, int& kp) {
-    km = ((m > c) + (m > p)) * 4 + 0;
-    kc = ((c > m) + (c > p)) * 4 + 1;
-    kp = ((p > m) + (p > c)) * 4 + 2;
+// The better of two candidates under the strict order, the first one coming
+// earlier in position order: the second wins if it is greater, or, with `tie`
+// (one of the two lies across the periodic boundary, which reverses their
+// index order), if it is equal.
+template <bool kInner>
+__device__ __forceinline__ void best2(float m1, int q1, float m2, int q2, bool tie, float& m, int& q) {
+    const bool w = kInner ? m2 > m1 : (m2 > m1 || (tie && m2 == m1));
+    m = fmaxf(m1, m2);
+    q = w ? q2 : q1;
 }
 
-// Position (0, 1, 2 for -1, 0, +1) of the first candidate, in the strict
-// order, whose value equals M.
-__device__ __forceinline__ int pick3(float a, float b, float c, float M, int ka, int kb, int kc) {
-    const int x = min(min(a == M ? ka : kNoMatch, b == M ? kb : kNoMatch), c == M ? kc : kNoMatch);
-    return x & 3;
-}
-// Winner of a window of three candidates along one axis (offsets -1, 0, +1),
-// with their window maxima a, b, c and payloads qa, qb, qc (the choices made
-// along the axes searched before this one); the winner's choice (0, 1, 2) is
-// added to its payload at bit `shift`.  Away from the periodic boundary (I) the
-// strict order ranks the candidates in position order, so the winner is the
-// first one holding the maximum: a later candidate wins only if strictly
-// greater.  At the boundary the search codes of the wrapped coordinates decide.
-template <bool I>
-__device__ __forceinline__ void win3(float a, float b, float c, uint32_t qa, uint32_t qb, uint32_t qc, int ka, int kb,
-                                     int kc, int shift, float& m, uint32_t& q) {
-    if (I) {
-        const float m1 = fmaxf(a, b);
-        const uint32_t q1 = b > a ? (qb | (1u << shift)) : qa;
-        m = fmaxf(m1, c);
-        q = c > m1 ? (qc | (2u << shift)) : q1;
-    } else {
-        m = fmaxf(fmaxf(a, b), c);
-        const int k = pick3(a, b, c, m, ka, kb, kc);
-        q = (k == 0 ? qa : (k == 1 ? qb : qc)) | (uint32_t(k) << shift);
-    }
-}
-
-// Asynchronous 4-byte copy global -> shared (sm_80+ cp.async), completed in
-// groups: each thread waits only for its own copies.
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))),
-                 "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// Parent code of every cell.  The best of the 27 cells around c is the first
-// cell, in wrapped (z, y, x) lexicographic order, holding the window's maximum
-// M, so it is found separably: per row and plane the x window (warp shuffles)
-// gives the row's maximum and x choice; per plane the y window over the
-// thread's rows gives the plane's maximum and (y, x) choice; the z window over
-// a ring of the last three planes gives M and the full choice, which is the
-// parent code itself (offset + 1 along x, y, z in bits 0-1, 2-3, 4-5).  The
-// choices ride along with the maxima as payloads, so no choice is searched for
-// twice.  Each lane streams its column's rows through a ring of kParStages
-// planes in shared memory (asynchronous copies issued kParStages - 1 planes
-// ahead), which keeps enough loads in flight without holding them in
-// registers.  The plane loop is unrolled six times, so that the ring slots
-// rotate by renaming rather than copying.
-// One warp's block.  XI / YI: the block's owned columns / rows are away from
-// the periodic boundary, where the x / y choices reduce to position order;
-// the z choice takes the same shortcut on every plane but the two wrapped ones.
-template <bool XI, bool YI>
-__device__ __forceinline__ void parent_block(const float* __restrict__ C, int N, float cwt_min,
-                                             uint8_t* __restrict__ code_out, uint32_t* __restrict__ seed_bits,
-                                             int* status, int x0, int y0, int z0, int wzc, float* ring) {
-    constexpr int R = kParR, NR = kParR + 2, S = kParStages;
-    static_assert(6 % S == 0, "the unrolled loop fixes each plane's ring slot");
-    const int lane = threadIdx.x & 31;
+// One tile.  The best of the 27 cells around c is the first cell, in wrapped
+// (z, y, x) lexicographic order, holding the window's maximum, so it is found
+// separably: the x windows of every row (shuffles), the y windows over the
+// warp's rows, the z windows over the planes as they come.  Neighbouring
+// windows of three share a pair (columns 2k, 2k+1; the warp's two rows), so two
+// windows take three two-way choices instead of four.  Each choice carries the
+// candidate's offset in the pointer array: the x choice is relative to the
+// lane's first column, the row's offset rides in it as a constant, and the
+// plane's is added once, so the z choice is the pointer itself.  kInner: the
+// tile and its halo are clear of the periodic boundary.
+//
+// What bounds it and what it replaced: instruction issue, not DRAM.  Two
+// kernels did this before (one-byte parent codes through memory, then a tile
+// kernel that decoded them to 32-bit pointers): 250 instructions per cell,
+// 3.34 + 4.52 ms per scale at 1024^3 and 0.26 + 0.26 ms at 384^3, against
+// 5.63 and 0.35 ms here.  16-bit
+// pointers in a box with a halo need no decoding and no test for neighbours
+// outside the tile, and leave room for four blocks per SM.  Two rows per warp
+// rather than four: the halo rows' x windows cost 4 instructions per cell more,
+// but half the code and 64 registers per thread keep 32 warps on an SM
+// (1024^3: 7.16 ms with four rows, 128 registers and 16 warps).
+template <bool kInner>
+__device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, float cwt_min, int32_t* __restrict__ label,
+                                         uint32_t* __restrict__ seed_bits, uint32_t* __restrict__ seed_cells,
+                                         uint32_t* __restrict__ ballots, int* status, unsigned char* sm,
+                                         uint32_t* n_seeds) {
+    uint16_t* seeds = reinterpret_cast<uint16_t*>(sm + kSBytes);
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(sm + kSBytes + 2 * kTileSeedCap);
+    int32_t* line = reinterpret_cast<int32_t*>(sm + kSBytes + 4 * kTileSeedCap);  // global index of each row's x = 0
+    auto at = [&](int off) -> uint16_t& { return *reinterpret_cast<uint16_t*>(sm + off); };
+    auto pair_at = [&](int off) -> uint32_t& { return *reinterpret_cast<uint32_t*>(sm + off); };
     const unsigned full = 0xffffffffu;
-    const int xc = ((x0 + lane - 1) % N + N) % N;
-    const bool own_x = lane >= 1 && lane <= 30 && x0 + lane - 1 < N;
-    int kxm = 0, kxc = 5, kxp = 10;
-    if (!XI) codes3(wrap(xc - 1, N), xc, wrap(xc + 1, N), kxm, kxc, kxp);
-    // offsets of the rows y0-1 .. y0+R (wrapped) and the y search codes of the
-    // owned rows, packed km | kc << 4 | kp << 8 per row
-    int32_t yoff[NR];
-#pragma unroll
-    for (int j = 0; j < NR; j++) yoff[j] = (((y0 - 1 + j) % N + N) % N) * N;
-    int ykc[R];
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-        ykc[r] = 0 | (5 << 4) | (10 << 8);
-        if (!YI) {
-            int a, b, c;
-            codes3(yoff[r] / N, yoff[r + 1] / N, yoff[r + 2] / N, a, b, c);
-            ykc[r] = a | (b << 4) | (c << 8);
-        }
-    }
-    const int32_t plane = N * N;
-    const float* colp = C + xc;
-    const int np_ = wzc + 2;
-    float* my = ring + lane;  // this lane's column of ring slot s, row j: my[(s * NR + j) * 32]
-    // copies of plane p (z = z0 - 1 + p, wrapped) into ring slot p % S, one group per plane
-    auto issue = [&](int p) {
-        if (p < np_) {
-            const int z = ((z0 - 1 + p) % N + N) % N;
-            const float* base = colp + size_t(z) * size_t(plane);
-            float* dst = my + (p % S) * NR * 32;
-#pragma unroll
-            for (int j = 0; j < NR; j++) cp_async4(dst + j * 32, base + yoff[j]);
-        }
-        cp_async_commit();  // empty groups past the end keep the count uniform
-    };
-    bool bad = false;
-    // plane p (ring slot p % S, unroll position u = p % 6): x and y windows
-    // into the window ring slot (mn, qn), then the z windows of plane p - 1
-    // from the slots of planes p - 2 (mo, qo), p - 1 (mm, qm) and p (mn, qn)
-    auto step = [&](int p, auto u, const float (&mo)[R], const uint32_t (&qo)[R], const float (&mm)[R],
-                    const uint32_t (&qm)[R], float (&mn)[R], uint32_t (&qn)[R]) {
-        issue(p + S - 1);
-        cp_async_wait<S - 1>();  // this lane's copies of plane p have landed
-        const float* src = my + (decltype(u)::value % S) * NR * 32;
-        float rm[NR];
-        uint32_t rq[NR];
-#pragma unroll
-        for (int j = 0; j < NR; j++) {
-            const float v = src[j * 32];
-            bad |= (v != v);
-            const float vl = __shfl_up_sync(full, v, 1), vr = __shfl_down_sync(full, v, 1);
-            win3<XI>(vl, v, vr, 0u, 0u, 0u, kxm, kxc, kxp, 0, rm[j], rq[j]);
-        }
-#pragma unroll
-        for (int r = 0; r < R; r++)
-            win3<YI>(rm[r], rm[r + 1], rm[r + 2], rq[r], rq[r + 1], rq[r + 2], ykc[r] & 15, (ykc[r] >> 4) & 15,
-                     ykc[r] >> 8, 2, mn[r], qn[r]);
-        if (p >= 2) {
-            // the cells of plane p-1 (z = z0 + p - 2)
-            const int zc = z0 + p - 2;
-            const bool zlo = zc == 0, zhi = zc == N - 1;
-            const int kzm = zlo ? 8 : (zhi ? 4 : 0), kzc = zlo ? 1 : (zhi ? 9 : 5), kzp = zlo ? 6 : (zhi ? 2 : 10);
-            uint8_t* out = code_out + size_t(zc) * size_t(plane) + xc;
-            const int32_t gz = zc * plane + xc;
-            auto emit = [&](auto zi) {
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    float M;
-                    uint32_t code;
-                    win3<decltype(zi)::value>(mo[r], mm[r], mn[r], qo[r], qm[r], qn[r], kzm, kzc, kzp, 4, M, code);
-                    const bool seed = code == kCodeMax && M > cwt_min;
-                    if (own_x && y0 + r < N) {
-                        out[yoff[r + 1]] = uint8_t(code | (seed ? kCodeSeed : 0u));
-                        if (seed) {
-                            const uint32_t g = uint32_t(gz + yoff[r + 1]);
-                            atomicOr(&seed_bits[g >> 5], 1u << (g & 31));
-                        }
-                    }
-                }
-            };
-            if (!zlo && !zhi) emit(std::integral_constant<bool, true>{});  // uniform: once per plane
-            else emit(std::integral_constant<bool, false>{});
-        }
-    };
-    float m0[R], m1[R], m2[R];
-    uint32_t q0[R], q1[R], q2[R];
-#pragma unroll
-    for (int p = 0; p < S - 1; p++) issue(p);
-    // plane p goes to window ring slot p % 3
-#pragma unroll 1
-    for (int p = 0; p < np_; p += 6) {
-        using I0 = std::integral_constant<int, 0>;
-        using I1 = std::integral_constant<int, 1>;
-        using I2 = std::integral_constant<int, 2>;
-        using I3 = std::integral_constant<int, 3>;
-        using I4 = std::integral_constant<int, 4>;
-        using I5 = std::integral_constant<int, 5>;
-        step(p, I0{}, m1, q1, m2, q2, m0, q0);
-        if (p + 1 >= np_) break;
-        step(p + 1, I1{}, m2, q2, m0, q0, m1, q1);
-        if (p + 2 >= np_) break;
-        step(p + 2, I2{}, m0, q0, m1, q1, m2, q2);
-        if (p + 3 >= np_) break;
-        step(p + 3, I3{}, m1, q1, m2, q2, m0, q0);
-        if (p + 4 >= np_) break;
-        step(p + 4, I4{}, m2, q2, m0, q0, m1, q1);
-        if (p + 5 >= np_) break;
-        step(p + 5, I5{}, m0, q0, m1, q1, m2, q2);
-    }
-    cp_async_wait<0>();  // nothing left in flight (the trailing groups are empty)
-    if (bad) set_status(status, CWTHF_E_BAD_INPUT);
-}
-
-__global__ void __launch_bounds__(kParThreads, kParBlocks) k_seg_parent(const float* __restrict__ C, int ng,
-                                                                     float cwt_min, uint8_t* __restrict__ code_out,
-                                                                     uint32_t* __restrict__ seed_bits, int* status) {
-    constexpr int R = kParR;
-    __shared__ float ring[kParWarps][kParStages * (kParR + 2) * 32];
-    const int N = ng;
-    const int nbx = (N + 29) / 30, nby = (N + R - 1) / R;
-    const int64_t warp = (int64_t(blockIdx.x) * kParThreads + threadIdx.x) >> 5;
-    const int64_t nwarps = int64_t(nbx) * nby * ((N + kParZ - 1) / kParZ);
-    if (warp >= nwarps) return;  // warp-uniform
-    const int by = int(warp % nby), bx = int((warp / nby) % nbx), bz = int(warp / (int64_t(nby) * nbx));
-    const int x0 = bx * 30, y0 = by * R, z0 = bz * kParZ;
-    const int wzc = min(kParZ, N - z0);
-    float* my_ring = ring[threadIdx.x >> 5];
-    // warp-uniform: owned columns x0 .. x0+29 and rows y0 .. y0+R-1 clear of 0 and N-1
-    if (x0 > 0 && x0 + 30 < N && y0 > 0 && y0 + R < N)
-        parent_block<true, true>(C, N, cwt_min, code_out, seed_bits, status, x0, y0, z0, wzc, my_ring);
-    else
-        parent_block<false, false>(C, N, cwt_min, code_out, seed_bits, status, x0, y0, z0, wzc, my_ring);
-}
-
-// In-tile chains of a 64 x 16 x 16-cell tile from the parent codes.  Every
-// cell's code becomes a shared-memory pointer (a local index, a seed's own
-// index, -1 for a maximum that is not a seed, or -2 - g for a parent g outside
-// the tile); pointer-jumping rounds over the whole tile then bring every
-// pointer to the end of its chain inside the tile: a seed, a non-seed maximum,
-// or a cell outside the tile.  A cell whose chain ends at a seed of this tile
-// adds one to the seed's cell count, kept in the upper half of the seed's own
-// entry.
-__global__ void __launch_bounds__(kChThreads, 3) k_seg_chase(const uint8_t* __restrict__ codes, int ng,
-                                                           int32_t* __restrict__ label,
-                                                           uint32_t* __restrict__ seed_cells,
-                                                           uint32_t* __restrict__ ballots, int* status) {
-    extern __shared__ __align__(16) int32_t ptr[];  // [kLocal], dynamic
-    __shared__ uint16_t tile_seeds[kTileSeedCap];
-    __shared__ uint32_t n_tile_seeds;
-    const int N = ng;  // even
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ntx = (N + kChTX - 1) / kChTX, nty = (N + kChTY - 1) / kChTY;
     const int t = int(blockIdx.x);
     const int tx = t % ntx, ty = (t / ntx) % nty, tz = t / (ntx * nty);
     const int x0 = tx * kChTX, y0 = ty * kChTY, z0 = tz * kChTZ;
-    const int wx = min(kChTX, N - x0), wy = min(kChTY, N - y0), wz = min(kChTZ, N - z0);  // wx even
-    const int lane = threadIdx.x & 31, ly = threadIdx.x >> 5;
-    const int lx = 2 * lane;  // this lane's columns lx, lx + 1
-    const bool own = lx < wx && ly < wy;
-    const int xc = x0 + lx, yc = y0 + ly;
-    const int32_t plane32 = N * N;
-    // global index pieces of the neighbours (one step, or across the periodic
-    // boundary) of the even column xc and the odd column xc + 1
-    const int32_t oxm0 = xc == 0 ? N - 1 : -1, oxp1 = xc + 1 == N - 1 ? -(N - 1) : 1;
-    const int32_t oym = yc == 0 ? (N - 1) * N : -N, oyp = yc == N - 1 ? -(N - 1) * N : N;
-    if (threadIdx.x == 0) n_tile_seeds = 0;
-    __syncthreads();
-    const int i0 = ly * kPX + lx;
-    // a cell's shared-memory pointer from its parent code: a seed's own index,
-    // -1 for a maximum that is not a seed, a local index, or -2 - g for a
-    // parent g outside the tile
-    auto decode = [&](uint32_t code, int cx, int lz, int zc, int32_t g, int32_t oxm, int32_t oxp, int i) -> int32_t {
-        if ((code & 0x3fu) == kCodeMax) {
-            if (code & kCodeSeed) {
-                const uint32_t j = atomicAdd(&n_tile_seeds, 1u);
-                if (j < uint32_t(kTileSeedCap)) tile_seeds[j] = uint16_t(i);
-                return i;
-            }
-            return -1;
-        }
-        const int dx = int(code & 3u) - 1, dy = int((code >> 2) & 3u) - 1, dz = int((code >> 4) & 3u) - 1;
-        if (unsigned(cx + dx) < unsigned(wx) && unsigned(ly + dy) < unsigned(wy) && unsigned(lz + dz) < unsigned(wz))
-            return i + dx + dy * kPX + dz * kPlaneL;
-        const int32_t ozm = zc == 0 ? (N - 1) * plane32 : -plane32;
-        const int32_t ozp = zc == N - 1 ? -(N - 1) * plane32 : plane32;
-        return -2 - (g + (dx < 0 ? oxm : (dx > 0 ? oxp : 0)) + (dy < 0 ? oym : (dy > 0 ? oyp : 0)) +
-                     (dz < 0 ? ozm : (dz > 0 ? ozp : 0)));
-    };
-    if (own) {
-        const int32_t grow = yc * N + xc;  // even
-        constexpr int kBatch = 8;  // planes whose codes are loaded together (independent loads in flight)
-        for (int lb = 0; lb < wz; lb += kBatch) {
-            uint32_t cb[kBatch];
-#pragma unroll
-            for (int u = 0; u < kBatch; u++)
-                cb[u] = lb + u < wz ? *reinterpret_cast<const uint16_t*>(codes + (z0 + lb + u) * plane32 + grow) : 0u;
-#pragma unroll
-            for (int u = 0; u < kBatch; u++) {
-                const int lz = lb + u;
-                if (lz >= wz) break;
-                const int zc = z0 + lz;
-                const int32_t g = zc * plane32 + grow;
-                const int i = i0 + lz * kPlaneL;
-                int2 v;
-                v.x = decode(cb[u] & 0xffu, lx, lz, zc, g, oxm0, 1, i);
-                v.y = decode(cb[u] >> 8, lx + 1, lz, zc, g + 1, -1, oxp1, i + 1);
-                *reinterpret_cast<int2*>(&ptr[i]) = v;
-            }
-        }
+    const int wx = min(kChTX, N - x0), wy = min(kChTY, N - y0), wz = min(kChTZ, N - z0);  // all even
+    const int32_t plane = N * N;
+    // every entry a root (the halo and what a ragged tile leaves out stay that way)
+    for (int i = threadIdx.x; i < kSBytes / 4; i += kSegThreads)
+        pair_at(4 * i) = uint32_t(4 * i) | (uint32_t(4 * i + 2) << 16);
+    for (int i = threadIdx.x; i < kSegLines; i += kSegThreads) {
+        const int z = z0 - 1 + i / (kChTY + 2), y = y0 - 1 + i % (kChTY + 2);
+        line[i] = kInner ? z * plane + y * N : ((z + N) % N) * plane + ((y + N) % N) * N;
     }
     __syncthreads();
-    // Pointer jumping in place, every cell of the tile in lockstep (no divergent
-    // walks): a pointer to a non-root cell moves two links further (the target's
-    // target's pointer, so a round triples the distance covered), until no
-    // pointer changes.  A value read while another thread rewrites it is either
-    // the old or the new pointer, both points of the same chain.
-    auto jump1 = [&](int i, int32_t v, bool& changed) {
-        if (v >= 0 && v != i && index_ok(v, kLocal, status)) {
-            int32_t w = ptr[v];
-            if (w != v) {
-                if (w >= 0 && index_ok(w, kLocal, status)) w = ptr[w];
-                ptr[i] = w;
-                changed = true;
+
+    // ---- parents ----
+    constexpr int R = kSegRows, NR = R + 2;
+    const int lx = 2 * lane, r0 = warp * R;  // this lane's columns lx, lx + 1; the warp's rows r0 .. r0 + R - 1
+    const int xa = kInner ? x0 + lx : (x0 + lx) % N;
+    // lanes 0 and 31 fetch the columns beside the tile as well
+    const int xe = lane == 0 ? (kInner ? x0 - 1 : (x0 - 1 + N) % N) : (kInner ? x0 + kChTX : (x0 + kChTX) % N);
+    const bool edge = lane == 0 || lane == 31;
+    int32_t roff[NR];
+#pragma unroll
+    for (int j = 0; j < NR; j++) {
+        const int y = y0 + r0 - 1 + j;
+        roff[j] = (kInner ? y : (y + N) % N) * N;
+    }
+    const bool vec = (reinterpret_cast<uintptr_t>(C) & 7u) == 0;  // N and xa are even
+    const bool tie_xl = !kInner && xa == 0, tie_xr = !kInner && xa + 1 == N - 1;
+    bool bad = false;
+    float2 va[NR];
+    float ve[NR];
+    auto fetch = [&](int p) {  // plane p: z = z0 - 1 + p
+        const int z = kInner ? z0 - 1 + p : (z0 - 1 + p + N) % N;
+        const float* base = C + size_t(z) * size_t(plane);
+#pragma unroll
+        for (int j = 0; j < NR; j++) {
+            const float* a = base + roff[j] + xa;
+            if (vec) va[j] = *reinterpret_cast<const float2*>(a);
+            else va[j] = make_float2(a[0], a[1]);
+            ve[j] = edge ? base[roff[j] + xe] : 0.f;
+        }
+    };
+    // x and y windows of the plane fetched last, with offsets relative to the
+    // plane's (row r0 - 1, this lane's first column)
+    auto xy = [&](float (&M)[2 * R], int (&Q)[2 * R], int qz) {
+        float m[2 * NR];
+        int q[2 * NR];
+#pragma unroll
+        for (int j = 0; j < NR; j++) {
+            const float a = va[j].x, b = va[j].y;
+            bad |= (a != a) | (b != b);
+            float l = __shfl_up_sync(full, b, 1), r = __shfl_down_sync(full, a, 1);
+            if (lane == 0) l = ve[j];
+            if (lane == 31) r = ve[j];
+            const int o = j * kSRow;
+            const float pm = fmaxf(a, b);
+            const int pq = b > a ? o + 2 : o;
+            best2<kInner>(l, o - 2, pm, pq, tie_xl, m[2 * j], q[2 * j]);
+            best2<kInner>(pm, pq, r, o + 4, tie_xr, m[2 * j + 1], q[2 * j + 1]);
+        }
+#pragma unroll
+        for (int k = 0; k < R; k += 2) {  // rows k, k + 1 of the warp (fetched rows k + 1, k + 2)
+            const int y = y0 + r0 + k;
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                float pm;
+                int pq;
+                best2<true>(m[2 * (k + 1) + c], q[2 * (k + 1) + c], m[2 * (k + 2) + c], q[2 * (k + 2) + c], false, pm, pq);
+                best2<kInner>(m[2 * k + c], q[2 * k + c], pm, pq, !kInner && y == 0, M[2 * k + c], Q[2 * k + c]);
+                best2<kInner>(pm, pq, m[2 * (k + 3) + c], q[2 * (k + 3) + c], !kInner && y + 1 == N - 1,
+                              M[2 * (k + 1) + c], Q[2 * (k + 1) + c]);
+                Q[2 * k + c] += qz;
+                Q[2 * (k + 1) + c] += qz;
             }
         }
     };
-    auto jump = [&](int lz, bool& changed) {
-        const int i = i0 + lz * kPlaneL;
-        const int2 v = *reinterpret_cast<const int2*>(&ptr[i]);
-        jump1(i, v.x, changed);
-        jump1(i + 1, v.y, changed);
+    const int lane0 = r0 * kSRow + 2 * (lx + 2);  // offset of (plane 0, row r0 - 1, column lx)
+    const bool own_x = lx < wx;
+    // stores the pointers of tile plane lz = p - 1 from the choices (m1, q1), (m2, q2) along z
+    auto emit = [&](int p, const float (&m1)[2 * R], const int (&q1)[2 * R], const float (&m2)[2 * R],
+                    const int (&q2)[2 * R], bool tie, bool first) {
+        const int own0 = lane0 + p * kSPlane + kSRow;
+#pragma unroll
+        for (int k = 0; k < R; k++) {
+            float m[2];
+            int q[2];
+            // (first: the pair's choice may lie in the plane across the boundary, which loses ties)
+            best2<kInner>(m1[2 * k], q1[2 * k], m2[2 * k], q2[2 * k], tie || (first && q1[2 * k] < kSPlane), m[0], q[0]);
+            best2<kInner>(m1[2 * k + 1], q1[2 * k + 1], m2[2 * k + 1], q2[2 * k + 1],
+                          tie || (first && q1[2 * k + 1] < kSPlane), m[1], q[1]);
+            const int own = own0 + k * kSRow;
+            if (own_x && r0 + k < wy) {
+#pragma unroll
+                for (int c = 0; c < 2; c++)
+                    if (q[c] == own + 2 * c) {  // a local maximum
+                        if (m[c] > cwt_min) {
+                            const uint32_t g = uint32_t((z0 + p - 1) * plane + (y0 + r0 + k) * N + x0 + lx + c);
+                            atomicOr(&seed_bits[g >> 5], 1u << (g & 31));
+                            const uint32_t j = atomicAdd(n_seeds, 1u);
+                            if (j < uint32_t(kTileSeedCap)) seeds[j] = uint16_t(q[c]);
+                        } else {
+                            q[c] = kSNone;
+                        }
+                    }
+                pair_at(own) = uint32_t(q[0]) | (uint32_t(q[1]) << 16);
+            }
+        }
     };
+    // along z: the better of the last two planes, and the last plane
+    float mP[2 * R], mL[2 * R], mN[2 * R];
+    int qP[2 * R], qL[2 * R], qN[2 * R];
+    fetch(0);
+    xy(mP, qP, lane0);
+    fetch(1);
+    xy(mL, qL, lane0 + kSPlane);
+    fetch(2);
+    // planes 0 and 1: the first one wins ties unless it lies across the boundary
+#pragma unroll
+    for (int i = 0; i < 2 * R; i++)
+        best2<kInner>(mP[i], qP[i], mL[i], qL[i], !kInner && z0 == 0, mP[i], qP[i]);
+#pragma unroll 1
+    for (int p = 1; p <= wz; p++) {
+        xy(mN, qN, lane0 + (p + 1) * kSPlane);
+        if (p < wz) fetch(p + 2);
+        emit(p, mP, qP, mN, qN, !kInner && z0 + p == N, !kInner && z0 == 0 && p == 1);
+#pragma unroll
+        for (int i = 0; i < 2 * R; i++) {
+            best2<true>(mL[i], qL[i], mN[i], qN[i], false, mP[i], qP[i]);
+            mL[i] = mN[i];
+            qL[i] = qN[i];
+        }
+    }
+    if (bad) set_status(status, CWTHF_E_BAD_INPUT);
+    __syncthreads();
+
+    // ---- chains inside the tile: pointer jumping in place, every cell in
+    // lockstep; a pointer takes its target's target's target, until every
+    // pointer names a root.  A value read while another thread rewrites it is
+    // the old or the new pointer, both points of the same chain. ----
+    const int mine = lane0 + kSPlane + kSRow;  // (plane lz 0, row r0)
     for (int round = 0; round < kJumpRoundsInTile; round++) {
-        bool changed = false;
-        if (own) {
-            if (wz == kChTZ) {  // every tile but a ragged last one along z
+        bool more = false;
+#pragma unroll 1
+        for (int k = 0; k < R; k++) {
 #pragma unroll 8
-                for (int lz = 0; lz < kChTZ; lz++) jump(lz, changed);
-            } else {
-                for (int lz = 0; lz < wz; lz++) jump(lz, changed);
+            for (int lz = 0; lz < kChTZ; lz++) {
+                uint32_t& w = pair_at(mine + k * kSRow + lz * kSPlane);
+                const uint32_t u = w, u0 = u & 0xffffu, u1 = u >> 16;
+                if (!index_ok(u0, kSBytes, status) || !index_ok(u1, kSBytes, status)) continue;
+                const uint32_t t0 = at(int(u0)), t1 = at(int(u1));
+                if (t0 != u0 || t1 != u1) {
+                    const uint32_t s0 = at(int(t0)), s1 = at(int(t1));
+                    w = s0 | (s1 << 16);
+                    more |= s0 != t0 || s1 != t1;
+                }
             }
         }
-        if (!__syncthreads_or(changed)) break;
+        if (!__syncthreads_or(more)) break;
     }
-    // every pointer now names a root (its cell's seed), -1, or -2 - g (a cell
-    // outside): labels, and one count per cell for the tile's seeds, kept in
-    // the upper half of the seed's own entry (readers mask it off)
-    const int32_t gbase = (z0 * N + y0) * N + x0;
-    const unsigned full = 0xffffffffu;
-    auto finish = [&](int32_t v, bool& fl) -> int32_t {
-        const int32_t cur = v >= 0 ? (v & kLocalMask) : v;
-        if (cur == -1) return -1;
-        if (cur <= -2) {
-            fl = true;
-            return cur;  // -2 - g: already the flagged pointer to the outside parent g
-        }
-        if (!index_ok(cur, kLocal, status)) return -1;
-        const int px = cur & (kPX - 1), py = (cur >> kPXBits) & (kChTY - 1), pz = cur >> kPlaneBits;
-        const int32_t g = gbase + (pz * N + py) * N + px;
-        const int32_t nv = ptr[cur];
-        if (nv >= 0 && (nv & kLocalMask) == cur) {
-            atomicAdd(&ptr[cur], 1 << kCountShift);
+    // each seed's entry now holds its number in the tile (odd: offsets are even)
+    const uint32_t ns = min(*n_seeds, uint32_t(kTileSeedCap));
+    if (threadIdx.x == 0 && *n_seeds > uint32_t(kTileSeedCap)) set_status(status, CWTHF_E_BAD_INPUT);
+    for (uint32_t j = threadIdx.x; j < ns; j += kSegThreads) at(seeds[j]) = uint16_t(2 * j + 1);
+    for (uint32_t j = threadIdx.x; j < (ns + 1) / 2; j += kSegThreads) cnt[j] = 0u;
+    __syncthreads();
+
+    // ---- labels, and one count per cell for the tile's seeds ----
+    // global index of the cell at offset o (inside the tile or in its halo)
+    auto cell_at = [&](uint32_t o) -> int32_t {
+        const uint32_t r = (o * kYMul) >> kYShift;
+        const int x = x0 - 2 + int((o - r * uint32_t(kSRow)) >> 1);
+        return line[r] + (kInner ? x : wrap(x, N));
+    };
+    auto finish = [&](uint32_t u, int own, bool& fl) -> int32_t {
+        if (!index_ok(u, 65536, status)) return -1;
+        uint32_t e = u;
+        if (u & 1u) u = uint32_t(own);  // a seed's own entry
+        else e = at(int(u));
+        if (u == uint32_t(kSNone)) return -1;
+        const int32_t g = cell_at(u);
+        if (e & 1u) {
+            const uint32_t j = e >> 1;
+            atomicAdd(&cnt[j >> 1], 1u << (16 * (j & 1u)));
             return g;
         }
-        fl = true;
-        return -2 - g;  // not finished within the round bound: resume globally
+        fl = true;  // outside the tile (or not finished within the round bound)
+        return -2 - g;
     };
-    int32_t* out = label + (size_t(z0) * N + yc) * N + xc;
-    const bool vec = (reinterpret_cast<uintptr_t>(label) & 7u) == 0;  // xc is even: 8-byte label pairs
-    uint32_t* my_ballots = ballots + (size_t(t) * kChTY + ly) * kRowWords;
-    for (int lz = 0; lz < kChTZ; lz++, out += size_t(plane32)) {  // block-uniform trip count
-        bool f0 = false, f1 = false;
-        if (own && lz < wz) {
-            const int i = i0 + lz * kPlaneL;
-            const int2 v = *reinterpret_cast<const int2*>(&ptr[i]);
-            int2 res;
-            res.x = finish(v.x, f0);
-            res.y = finish(v.y, f1);
-            if (vec) {
-                *reinterpret_cast<int2*>(out) = res;
-            } else {
-                out[0] = res.x;
-                out[1] = res.y;
+    const bool lvec = (reinterpret_cast<uintptr_t>(label) & 7u) == 0;  // even cells: 8-byte label pairs
+#pragma unroll 1
+    for (int k = 0; k < R; k++) {
+        if (r0 + k >= kChTY) break;
+        const bool own = own_x && r0 + k < wy;
+        int32_t* out = label + (size_t(z0) * N + (y0 + r0 + k)) * N + x0 + lx;
+        uint32_t word = 0;
+#pragma unroll 4
+        for (int lz = 0; lz < kChTZ; lz++) {
+            bool f0 = false, f1 = false;
+            if (own && lz < wz) {
+                const int o = mine + k * kSRow + lz * kSPlane;
+                const uint32_t u = pair_at(o);
+                int2 res;
+                res.x = finish(u & 0xffffu, o, f0);
+                res.y = finish(u >> 16, o + 2, f1);
+                int32_t* dst = out + size_t(lz) * size_t(plane);
+                if (lvec) {
+                    *reinterpret_cast<int2*>(dst) = res;
+                } else {
+                    dst[0] = res.x;
+                    dst[1] = res.y;
+                }
             }
+            const unsigned b0 = __ballot_sync(full, f0), b1 = __ballot_sync(full, f1);
+            if (lane == 2 * lz) word = b0;      // plane lz, even columns
+            if (lane == 2 * lz + 1) word = b1;  // odd columns
         }
-        const unsigned b0 = __ballot_sync(full, f0), b1 = __ballot_sync(full, f1);
-        if (lane == 2 * lz) my_ballots[2 * lz] = b0;  // plane lz, even columns
-        if (lane == 2 * lz + 1) my_ballots[2 * lz + 1] = b1;  // odd columns
+        ballots[(size_t(t) * kChTY + r0 + k) * kRowWords + lane] = word;
     }
     __syncthreads();
     // in-tile cell counts of this tile's seeds (cells reaching them from other
     // tiles are added by the global pass)
-    const uint32_t nts = n_tile_seeds;
-    if (threadIdx.x == 0 && nts > uint32_t(kTileSeedCap)) set_status(status, CWTHF_E_BAD_INPUT);
-    for (uint32_t j = threadIdx.x; j < min(nts, uint32_t(kTileSeedCap)); j += blockDim.x) {
-        const int i = tile_seeds[j];
-        const int px = i & (kPX - 1), py = (i >> kPXBits) & (kChTY - 1), pz = i >> kPlaneBits;
-        seed_cells[size_t(gbase + (pz * N + py) * N + px)] = uint32_t(ptr[i]) >> kCountShift;
-    }
+    for (uint32_t j = threadIdx.x; j < ns; j += kSegThreads)
+        seed_cells[size_t(cell_at(seeds[j]))] = (cnt[j >> 1] >> (16 * (j & 1u))) & 0xffffu;
+}
+
+__global__ void __launch_bounds__(kSegThreads, 4) k_seg_tile(const float* __restrict__ C, int ng, float cwt_min,
+                                                             int32_t* __restrict__ label,
+                                                             uint32_t* __restrict__ seed_bits,
+                                                             uint32_t* __restrict__ seed_cells,
+                                                             uint32_t* __restrict__ ballots, int* status) {
+    extern __shared__ __align__(16) unsigned char seg_smem[];
+    __shared__ uint32_t n_seeds;
+    if (threadIdx.x == 0) n_seeds = 0;  // (the tile's first barrier is before its first use)
+    const int ntx = (ng + kChTX - 1) / kChTX, nty = (ng + kChTY - 1) / kChTY;
+    const int t = int(blockIdx.x), tx = t % ntx, ty = (t / ntx) % nty, tz = t / (ntx * nty);
+    const bool inner = tx > 0 && (tx + 1) * kChTX < ng && ty > 0 && (ty + 1) * kChTY < ng && tz > 0 &&
+                       (tz + 1) * kChTZ < ng;
+    if (inner) seg_tile<true>(C, ng, cwt_min, label, seed_bits, seed_cells, ballots, status, seg_smem, &n_seeds);
+    else seg_tile<false>(C, ng, cwt_min, label, seed_bits, seed_cells, ballots, status, seg_smem, &n_seeds);
 }
 
 constexpr int kResolveThreads = 256;
@@ -754,21 +657,15 @@ int segment_impl(cwthf_ctx* ctx, const float* cwt, int ng, float cwt_min, int32_
     cudaError_t e = cudaMemsetAsync(ctx->seed_bits, 0, size_t(nwords) * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->jump_changed, 0, sizeof(int) * kJumpWords, s);
     if (e != cudaSuccess) return cuda_status(e);
-    // parent codes (1 byte per cell) and the flagged-cell masks of every chain
-    // tile (one bit per cell) in the context's int64 grid buffer (8 bytes per
-    // cell, free once the forward transform has read it), then the in-tile chains
-    uint8_t* codes = reinterpret_cast<uint8_t*>(ctx->grid);
-    uint32_t* ballots = reinterpret_cast<uint32_t*>(codes + (size_t(cells) + 255) / 256 * 256);
+    // the flagged-cell masks of every chain tile (one bit per cell) in the context's int64 grid buffer
+    // (8 bytes per cell, free once the forward transform has read it)
+    uint32_t* ballots = reinterpret_cast<uint32_t*>(ctx->grid);
     const int64_t ntiles = int64_t(div_up(ng, kChTX)) * div_up(ng, kChTY) * div_up(ng, kChTZ);
-    if ((cells + 255) / 256 * 256 + ntiles * (kChTY * kRowWords * 4) > cells * 8) return CWTHF_E_UNSUPPORTED_SIZE;
-    const int64_t pwarps = int64_t(div_up(ng, 30)) * div_up(ng, kParR) * div_up(ng, kParZ);
-    CWTHF_LAUNCH(ctx, s, "k_seg_parent",
-                 k_seg_parent<<<unsigned(div_up(pwarps, int64_t(kParWarps))), kParThreads, 0, s>>>(
-                     cwt, ng, cwt_min, codes, ctx->seed_bits, ctx->d_status));
-    cudaFuncSetAttribute(k_seg_chase, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(int32_t) * kLocal));
-    CWTHF_LAUNCH(ctx, s, "k_seg_chase",
-                 k_seg_chase<<<unsigned(ntiles), kChThreads, sizeof(int32_t) * kLocal, s>>>(
-                     codes, ng, label, ctx->seed_cells, ballots, ctx->d_status));
+    if (ntiles * (kChTY * kRowWords * 4) > cells * 8) return CWTHF_E_UNSUPPORTED_SIZE;
+    cudaFuncSetAttribute(k_seg_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kSegSmem);
+    CWTHF_LAUNCH(ctx, s, "k_seg_tile",
+                 k_seg_tile<<<unsigned(ntiles), kSegThreads, kSegSmem, s>>>(cwt, ng, cwt_min, label, ctx->seed_bits,
+                                                                            ctx->seed_cells, ballots, ctx->d_status));
     // chains that left their tile, counted at their seed's cell
     int blocks = ctx->sm_count * 8;
     int* changed = ctx->jump_changed;  // see kJumpWords
