@@ -113,7 +113,7 @@ void for_each_buffer(cwthf_ctx* c, int max_ng, int64_t max_np, int max_scales, u
         // the whole-grid path for large groups: per-CTA partial sums and digit counts, barrier
         f(reinterpret_cast<void**>(&c->ub_part), size_t(kUnbindGridCtaCap) * 16 * 8);
         f(reinterpret_cast<void**>(&c->ub_hist), size_t(kUnbindGridCtaCap) * 2 * 256 * 4);
-        f(reinterpret_cast<void**>(&c->ub_bar), 16);
+        f(reinterpret_cast<void**>(&c->ub_bar), kUbBarWords * 4);
     }
     f(reinterpret_cast<void**>(&c->scan_tmp), z.scan_words * 4);
     f(reinterpret_cast<void**>(&c->grid), size_t(z.cells) * 8);

@@ -59,8 +59,15 @@ constexpr int kDefaultChaseLimit = 64;
 // Groups of the self-boundness check with more members than this are
 // processed by the whole grid, one at a time; smaller ones by one CTA each.
 constexpr int64_t kUnbindGridMin = 1 << 16;
-// Most CTAs of that whole-grid launch (its per-CTA scratch is sized for them).
-constexpr int kUnbindGridCtaCap = 1024;
+// Most CTAs of the launch for groups of several CTAs (its per-CTA scratch is
+// sized for them); its control words: the whole grid's barrier (2), the counts
+// of medium and large groups, the next of either for the teams, and from
+// kUbTeamWords on four words per team (barrier, next group): the teams of
+// kUnbindTeam CTAs, then the bigger ones of kUnbindBigTeam.
+constexpr int kUnbindGridCtaCap = 1024, kUnbindTeam = 8, kUnbindBigTeam = 32;
+constexpr int kUbMedium = 2, kUbLarge = 3, kUbNext = 4, kUbNextBig = 5, kUbTeamWords = 8;
+constexpr size_t kUbBarWords =
+    kUbTeamWords + 4 * (kUnbindGridCtaCap / kUnbindTeam + kUnbindGridCtaCap / kUnbindBigTeam);
 
 // A bounded device wait gives up after this many polls.
 constexpr long long kSpinLimit = 1ll << 20;
@@ -158,7 +165,7 @@ struct cwthf_ctx {
 
     // self-boundness check scratch (cwthf_unbind)
     uint32_t* ub_off = nullptr;   // [max groups + 2] members per group, then their offsets
-    uint32_t* ub_cur = nullptr;   // [max groups + 1] scatter cursors
+    uint32_t* ub_cur = nullptr;   // [max groups + 1] scatter cursors, then the lists of medium and large groups
     int32_t* ub_mem = nullptr;    // [max_np] members, grouped
     uint64_t* ub_key = nullptr;   // [2 max_np] sort keys
     int32_t* ub_val = nullptr;    // [2 max_np] sort values
@@ -172,7 +179,7 @@ struct cwthf_ctx {
     uint32_t* dep_nparts = nullptr;          // [1] parts listed
     double* ub_part = nullptr;       // [ub_grid_blocks][16] per-CTA partial sums of the whole-grid path
     uint32_t* ub_hist = nullptr;     // [2][ub_grid_blocks][256] per-CTA digit counts of its radix sort
-    unsigned* ub_bar = nullptr;      // [2] its grid barrier
+    unsigned* ub_bar = nullptr;      // [kUbBarWords] its barriers and group counts
     int ub_grid_blocks = 0;          // CTAs of the whole-grid path's cooperative launch
 
     // cwthf_find internals
@@ -243,7 +250,8 @@ __device__ __forceinline__ bool index_ok(long long i, long long n, int* status) 
 // gives up after kSpinLimit polls, records CWTHF_E_TIMEOUT and returns false;
 // the CTA then leaves the kernel.  Data that other CTAs wrote before the
 // barrier is read with L1-bypassing loads (__ldcg) after it.
-__device__ __forceinline__ bool grid_sync(unsigned* bar, int* status) {
+// `n` CTAs meet at it (all of the grid by default, or a team of its CTAs with a barrier of its own).
+__device__ __forceinline__ bool grid_sync(unsigned* bar, int* status, unsigned n) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -251,7 +259,7 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, int* status) {
         cuda::atomic_ref<unsigned, cuda::thread_scope_device> cnt(bar[0]), gen(bar[1]);
         const unsigned g = gen.load(cuda::memory_order_acquire);
         __threadfence();
-        if (cnt.fetch_add(1u, cuda::memory_order_acq_rel) == gridDim.x - 1) {
+        if (cnt.fetch_add(1u, cuda::memory_order_acq_rel) == n - 1) {
             cnt.store(0u, cuda::memory_order_relaxed);
             gen.store(g + 1u, cuda::memory_order_release);
         } else {
@@ -270,6 +278,7 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, int* status) {
     __syncthreads();
     return ok != 0;
 }
+__device__ __forceinline__ bool grid_sync(unsigned* bar, int* status) { return grid_sync(bar, status, gridDim.x); }
 
 // Slot (rank among all seeds, in cell order) of seed cell `lab`, from the seed
 // bitmap and its per-word popcount prefix; false if lab is not a seed or its
@@ -291,6 +300,28 @@ __device__ __forceinline__ void shared_add64(uint32_t* lo, uint32_t* hi, int c, 
     const uint32_t old = atomicAdd(&lo[c], vl);
     vh += (old + vl < old) ? 1u : 0u;
     if (vh) atomicAdd(&hi[c], vh);
+}
+
+// A CTA's open-addressing table of 32-bit keys in shared memory (cleared to
+// kEmpty).  The entry of `key`: found, or claimed (and listed in tused) when
+// an empty entry comes first; -1 after kProbe probes.
+constexpr int kTabBits = 10, kTab = 1 << kTabBits;  // entries
+constexpr int kProbe = 16;
+constexpr uint32_t kEmpty = 0xffffffffu;
+__device__ __forceinline__ int table_find(uint32_t* tkey, uint32_t* tused, uint32_t* used, uint32_t key) {
+    uint32_t h = (key * 2654435761u) >> (32 - kTabBits);  // multiplicative hash
+    for (int pr = 0; pr < kProbe; pr++, h = (h + 1) & (kTab - 1)) {
+        uint32_t k = tkey[h];
+        if (k == kEmpty) {
+            k = atomicCAS(&tkey[h], kEmpty, key);
+            if (k == kEmpty) {
+                tused[atomicAdd(used, 1u)] = h;
+                return int(h);
+            }
+        }
+        if (k == key) return int(h);
+    }
+    return -1;
 }
 
 // ---- warp helpers -------------------------------------------------------------

@@ -30,37 +30,91 @@ namespace {
 constexpr int kUbThreads = 512;
 constexpr int kUbWarps = kUbThreads / 32;
 constexpr int kUbSmemElems = 2048;  // groups up to this size sort in shared memory
+// Groups up to this size take one CTA, larger ones a team of kUnbindTeam CTAs
+// (up to the whole-grid threshold): a CTA alone worked 10 ms on a group of
+// 60,000 members while the rest of the GPU had long finished.
+constexpr int kUbCtaMax = 4096;
+// Groups above the whole-grid threshold but within these sizes take a team of
+// kUnbindBigTeam CTAs: several at a time, and with cheaper barriers, than one
+// after another with every CTA (six scales on 2^24 particles, 22 such groups:
+// the check's groups 53 ms with the grid for each, 38 ms with these teams).
+constexpr int kUbBigMin = int(kUnbindGridMin), kUbBigMax = 1 << 20;
+__device__ __forceinline__ bool big_team_group(uint32_t n) { return n > uint32_t(kUbBigMin) && n <= uint32_t(kUbBigMax); }
 
-// Integer mass quanta (the deposit's rule): 1 when masses are equal, else
-// rint(m / mass_unit); invalid masses are reported once here.
-__global__ void k_ub_count(const float* __restrict__ mass, double mass_unit, const int32_t* __restrict__ group,
-                           int64_t np, int64_t n_groups, const uint32_t* __restrict__ d_groups,
-                           uint32_t* __restrict__ cnt, int32_t* __restrict__ group_out, int* status) {
+// Counting sort of the particles by group, in two passes of one form: count
+// (kScatter false, which also clears group_out and checks the masses), then,
+// after the scan, scatter.  Particles come in snapshot order and a few hundred
+// groups hold most of them, so one atomic per particle queues up at the
+// groups' counters; a CTA takes kBinItems particles per thread, ranks them in
+// a shared table, and takes one range per group and chunk from the global
+// counter (2^24 particles: 0.60 ms per pass with an atomic each).
+constexpr int kBinThreads = 256, kBinItems = 8;
+template <bool kScatter>
+__global__ void __launch_bounds__(kBinThreads) k_ub_bin(const float* __restrict__ mass, double mass_unit,
+                                                        const int32_t* __restrict__ group, int64_t np,
+                                                        int64_t n_groups, const uint32_t* __restrict__ d_groups,
+                                                        const uint32_t* __restrict__ off,
+                                                        uint32_t* __restrict__ counter, int32_t* __restrict__ mem,
+                                                        int32_t* __restrict__ group_out, int* status) {
+    __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab];
+    __shared__ uint32_t n_used;
     if (d_groups) n_groups = *d_groups;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
-        group_out[i] = -1;
-        if (mass) {
-            const double r = rint(__ddiv_rn(double(mass[i]), mass_unit));
-            if (!(r >= 0.0)) set_status(status, CWTHF_E_BAD_INPUT);
-            else if (!(r < 2147483648.0)) set_status(status, CWTHF_E_OVERFLOW);
-        }
-        const int32_t g = group[i];
-        if (g >= 0 && int64_t(g) < n_groups) atomicAdd(&cnt[g], 1u);
+    for (int e = threadIdx.x; e < kTab; e += kBinThreads) {
+        tkey[e] = kEmpty;
+        tcnt[e] = 0u;
     }
-}
-
-__global__ void k_ub_scatter(const int32_t* __restrict__ group, int64_t np, int64_t n_groups,
-                             const uint32_t* __restrict__ d_groups, const uint32_t* __restrict__ off,
-                             uint32_t* __restrict__ cur, int32_t* __restrict__ mem, int* status) {
-    if (d_groups) n_groups = *d_groups;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
-        const int32_t g = group[i];
-        if (g >= 0 && int64_t(g) < n_groups) {
-            const uint32_t k = off[g] + atomicAdd(&cur[g], 1u);
-            if (index_ok(k, np, status)) mem[k] = int32_t(i);
+    if (threadIdx.x == 0) n_used = 0;
+    __syncthreads();
+    const int64_t chunk = int64_t(kBinThreads) * kBinItems;
+    for (int64_t c0 = int64_t(blockIdx.x) * chunk; c0 < np; c0 += int64_t(gridDim.x) * chunk) {
+        int slot[kBinItems];
+        uint32_t rank[kBinItems];
+#pragma unroll
+        for (int u = 0; u < kBinItems; u++) {
+            const int64_t i = c0 + u * kBinThreads + threadIdx.x;
+            slot[u] = -1;
+            if (i >= np) continue;
+            if (!kScatter) {
+                group_out[i] = -1;
+                if (mass) {
+                    const double r = rint(__ddiv_rn(double(mass[i]), mass_unit));
+                    if (!(r >= 0.0)) set_status(status, CWTHF_E_BAD_INPUT);
+                    else if (!(r < 2147483648.0)) set_status(status, CWTHF_E_OVERFLOW);
+                }
+            }
+            const int32_t g = group[i];
+            if (g < 0 || int64_t(g) >= n_groups) continue;
+            slot[u] = table_find(tkey, tused, &n_used, uint32_t(g));
+            if (slot[u] >= 0) {
+                rank[u] = atomicAdd(&tcnt[slot[u]], 1u);
+            } else {  // table crowded: straight to the group's counter
+                const uint32_t k = atomicAdd(&counter[g], 1u);
+                if (kScatter && index_ok(off[g] + k, np, status)) mem[off[g] + k] = int32_t(i);
+            }
         }
+        __syncthreads();
+        const uint32_t nu = n_used;
+        for (uint32_t j = threadIdx.x; j < nu; j += kBinThreads) {  // the chunk's range of each group
+            const uint32_t h = tused[j], g = tkey[h];
+            const uint32_t base = atomicAdd(&counter[g], tcnt[h]);
+            if (kScatter) tcnt[h] = off[g] + base;
+            else tcnt[h] = 0u;
+            tkey[h] = kEmpty;
+        }
+        if (kScatter) {
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < kBinItems; u++) {
+                if (slot[u] < 0) continue;
+                const uint32_t k = tcnt[slot[u]] + rank[u];
+                if (index_ok(k, np, status)) mem[k] = int32_t(c0 + u * kBinThreads + threadIdx.x);
+            }
+        }
+        __syncthreads();
+        if (kScatter)
+            for (uint32_t j = threadIdx.x; j < nu; j += kBinThreads) tcnt[tused[j]] = 0u;
+        if (threadIdx.x == 0) n_used = 0;
+        __syncthreads();
     }
 }
 
@@ -76,6 +130,9 @@ struct UbArgs {
     int32_t* val;         // [2 np] sort values (the same layout)
     int max_iter;
     int64_t grid_min;            // larger groups are left to the whole-grid path
+    uint32_t* list;              // [list_cap] groups of the team path from the front, of the whole-grid path
+    int64_t list_cap;            // from the back
+    unsigned* ctl;               // control words (kUbMedium, ...)
     int64_t n_groups;            // groups (or read from d_groups when given)
     const uint32_t* d_groups;
     int32_t* group_out;
@@ -170,21 +227,21 @@ __device__ void bitonic(K* k, int32_t* v, int P) {
         }
 }
 
-// Stable LSD radix sort (8-bit digits, the lowest nbytes bytes of the keys)
+// Stable LSD radix sort (8-bit digits, bytes byte0 .. byte1 - 1 of the keys)
 // of the n pairs K[0..n), V[0..n), with K[n..2n), V[n..2n) as the other
 // buffer; the result ends in K[0..n), V[0..n).  Every warp owns a contiguous
 // chunk: per pass, per-warp digit counts (shared memory), their offsets
 // digit-major then warp by warp, and a scatter that keeps each warp's chunk in
 // order (lanes of one digit ranked by match_any).  A pass in which every key
 // has the same digit moves nothing and is skipped.  All threads of the block.
-__device__ void radix_sort_pairs(uint64_t* K, int32_t* V, int n, int nbytes, uint32_t* hist, int* skip) {
+__device__ void radix_sort_pairs(uint64_t* K, int32_t* V, int n, int byte0, int byte1, uint32_t* hist, int* skip) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int chunk = (n + nw - 1) / nw;
     const int c0 = min(n, warp * chunk), c1 = min(n, c0 + chunk);
     const uint32_t lt = (1u << lane) - 1u;
     uint64_t *ka = K, *kb = K + n;
     int32_t *va = V, *vb = V + n;
-    for (int pass = 0; pass < nbytes; pass++) {
+    for (int pass = byte0; pass < byte1; pass++) {
         const int sh = 8 * pass;
         for (int i = threadIdx.x; i < nw * 256; i += blockDim.x) hist[i] = 0u;
         if (threadIdx.x == 0) *skip = 0;
@@ -251,10 +308,42 @@ __device__ void radix_sort_pairs(uint64_t* K, int32_t* V, int n, int nbytes, uin
     __syncthreads();
 }
 
-// Sorts the group's first n pairs of (K, V) (keys below 2^(8 nbytes)): a
-// bitonic sort in shared memory when the padded length fits, else the radix
-// sort in the group's slice of global scratch (2n entries).
-__device__ void sort_pairs(uint64_t* K, int32_t* V, int n, int nbytes, uint64_t* sk, int32_t* sv, uint32_t* hist,
+// After a stable sort by the keys' upper halves: the pair at k, if it starts a
+// run of pairs with one upper half, sorts the run by the whole keys (a stable
+// insertion).  Runs are rare and short (the upper half holds 20 bits of a
+// radius' mantissa); returns false for one longer than kMaxRun, left as it is.
+// Only the run's first pair moves it, and every pair keeps its upper half, so
+// the tests of the pairs beside it see the same runs at any time.
+constexpr int kMaxRun = 32;
+__device__ __forceinline__ bool fix_run(uint64_t* K, int32_t* V, int n, int k) {
+    const uint32_t h = uint32_t(__ldcg(K + k) >> 32);
+    if (k + 1 >= n || uint32_t(__ldcg(K + k + 1) >> 32) != h) return true;
+    if (k > 0 && uint32_t(__ldcg(K + k - 1) >> 32) == h) return true;
+    int m = 2;
+    while (m <= kMaxRun && k + m < n && uint32_t(__ldcg(K + k + m) >> 32) == h) m++;
+    if (m > kMaxRun) return false;
+    for (int i = 1; i < m; i++) {
+        const uint64_t x = __ldcg(K + k + i);
+        const int32_t v = __ldcg(V + k + i);
+        int j = i;
+        for (; j > 0; j--) {
+            const uint64_t y = __ldcg(K + k + j - 1);
+            if (y <= x) break;
+            __stcg(K + k + j, y);
+            __stcg(V + k + j, __ldcg(V + k + j - 1));
+        }
+        __stcg(K + k + j, x);
+        __stcg(V + k + j, v);
+    }
+    return true;
+}
+
+// Sorts the group's first n pairs of (K, V): a bitonic sort in shared memory
+// when the padded length fits, else the radix sort in the group's slice of
+// global scratch (2n entries).  index: keys below 2^32; otherwise whole
+// 64-bit keys, by their upper halves and the short runs those leave (eight
+// digits' passes took most of a round).
+__device__ void sort_pairs(uint64_t* K, int32_t* V, int n, bool index, uint64_t* sk, int32_t* sv, uint32_t* hist,
                            int* skip) {
     int P = 1;
     while (P < n) P <<= 1;
@@ -270,8 +359,16 @@ __device__ void sort_pairs(uint64_t* K, int32_t* V, int n, int nbytes, uint64_t*
             V[t] = sv[t];
         }
         __syncthreads();
+    } else if (index) {
+        radix_sort_pairs(K, V, n, 0, 4, hist, skip);
     } else {
-        radix_sort_pairs(K, V, n, nbytes, hist, skip);
+        radix_sort_pairs(K, V, n, 4, 8, hist, skip);
+        bool ok = true;
+        for (int t = threadIdx.x; t < n; t += blockDim.x) ok &= fix_run(K, V, n, t);
+        if (__syncthreads_or(!ok)) {
+            radix_sort_pairs(K, V, n, 0, 4, hist, skip);
+            radix_sort_pairs(K, V, n, 4, 8, hist, skip);
+        }
     }
 }
 
@@ -281,7 +378,13 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
     const uint32_t base = a.off[g];
     const int n0 = int(a.off[g + 1] - base);
     const int tid = threadIdx.x;
-    if (int64_t(n0) > a.grid_min) return;  // the whole-grid path's group
+    if (int64_t(n0) > a.grid_min || n0 > kUbCtaMax) {  // left to the whole grid, or to a team of CTAs
+        if (tid == 0) {
+            if (int64_t(n0) > a.grid_min) a.list[a.list_cap - 1 - int64_t(atomicAdd(a.ctl + kUbLarge, 1u))] = uint32_t(g);
+            else a.list[atomicAdd(a.ctl + kUbMedium, 1u)] = uint32_t(g);
+        }
+        return;
+    }
     if (n0 == 0) {
         if (tid == 0) {
             a.n_kept[g] = 0;
@@ -298,7 +401,7 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
         V[t] = X[t];
     }
     __syncthreads();
-    sort_pairs(K, V, n0, 4, sk, sv, hist, skip);
+    sort_pairs(K, V, n0, true, sk, sv, hist, skip);
     for (int t = tid; t < n0; t += blockDim.x) X[t] = V[t];
     __syncthreads();
     const float* a0 = a.pos + 3 * size_t(X[0]);
@@ -338,7 +441,7 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
             V[t] = i;
         }
         __syncthreads();
-        sort_pairs(K, V, n, 8, sk, sv, hist, skip);
+        sort_pairs(K, V, n, false, sk, sv, hist, skip);
         // 2-3. shell sums per member and the exclusions.  Thread t walks the
         // chunk [t ch, (t+1) ch): mass before the chunk and m/r after it come
         // from block scans of the chunk totals.  Massive members at the centre
@@ -404,8 +507,11 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
     }
 }
 
-// ---- the whole-grid path: one large group at a time, every CTA ---------------
+// ---- several CTAs per group ---------------------------------------------------
 //
+// The largest groups one at a time with every CTA of the grid, then large ones
+// with teams of kUnbindBigTeam CTAs and medium ones with teams of kUnbindTeam,
+// each team taking the next group when it is done.
 // The same steps as unbind_group, with each CTA owning a contiguous chunk of
 // the group's members and grid barriers between the phases.  Partial sums go
 // through per-CTA slots and are combined in CTA order by every CTA, so the
@@ -415,27 +521,31 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
 
 constexpr int kUbPart = 16;  // per-CTA partial slots: 0-6 centre of mass, 8-10 shell sums, 11 kept
 
-struct UbGrid {
-    double* part;    // [gridDim][kUbPart]
-    uint32_t* hist;  // [2][gridDim][256] by pass parity
+struct UbGrid {      // the grid, or one team of it
+    double* part;    // [size][kUbPart]
+    uint32_t* hist;  // [2][size][256] by pass parity
     unsigned* bar;
     int* status;
+    int size, rank;  // CTAs that work together, this CTA's place among them
 };
 
+__device__ __forceinline__ bool team_sync(const UbGrid& b) { return grid_sync(b.bar, b.status, unsigned(b.size)); }
+
 // [b, e) of the CTA's chunk of n members
-__device__ __forceinline__ void cta_chunk(int n, int& b, int& e) {
-    const int ch = (n + int(gridDim.x) - 1) / int(gridDim.x);
-    b = min(n, int(blockIdx.x) * ch);
+__device__ __forceinline__ void cta_chunk(const UbGrid& tm, int n, int& b, int& e) {
+    const int ch = (n + tm.size - 1) / tm.size;
+    b = min(n, tm.rank * ch);
     e = min(n, b + ch);
 }
 
 // Sums over the CTAs of partial slot k, in CTA order: over all CTAs (*all)
 // and over the CTAs before this one (returned).  Thread-local.
-__device__ __forceinline__ double part_prefix(const double* part, int k, double* all) {
+__device__ __forceinline__ double part_prefix(const UbGrid& tm, int k, double* all) {
     double s = 0.0, before = 0.0;
-    for (int c = 0; c < int(gridDim.x); c++) {
-        if (c == int(blockIdx.x)) before = s;
-        s += __ldcg(part + size_t(c) * kUbPart + k);
+#pragma unroll 8
+    for (int c = 0; c < tm.size; c++) {
+        if (c == tm.rank) before = s;
+        s += __ldcg(tm.part + size_t(c) * kUbPart + k);
     }
     *all = s;
     return before;
@@ -444,36 +554,37 @@ __device__ __forceinline__ double part_prefix(const double* part, int k, double*
 // The stable LSD radix sort of radix_sort_pairs over the whole grid: the
 // digit offsets add the counts of all CTAs before this one.  Returns false on
 // a barrier timeout.
-__device__ bool grid_radix(uint64_t* K, int32_t* V, int n, int nbytes, const UbGrid& b, uint32_t* hist,
+__device__ bool grid_radix(uint64_t* K, int32_t* V, int n, int byte0, int byte1, const UbGrid& b, uint32_t* hist,
                            uint32_t* dsum, uint32_t* dbase, int* skip, int& parity) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     int C0, C1;
-    cta_chunk(n, C0, C1);
+    cta_chunk(b, n, C0, C1);
     const int wch = (C1 - C0 + nw - 1) / nw;
     const int w0 = min(C1, C0 + warp * wch), w1 = min(C1, w0 + wch);
     const uint32_t lt = (1u << lane) - 1u;
     __shared__ uint32_t wsum[8];
     uint64_t *ka = K, *kb = K + n;
     int32_t *va = V, *vb = V + n;
-    for (int pass = 0; pass < nbytes; pass++) {
+    for (int pass = byte0; pass < byte1; pass++) {
         const int sh = 8 * pass;
         for (int i = tid; i < nw * 256; i += blockDim.x) hist[i] = 0u;
         if (tid == 0) *skip = 0;
         __syncthreads();
         for (int k = w0 + lane; k < w1; k += 32) atomicAdd(&hist[warp * 256 + int((__ldcg(ka + k) >> sh) & 255u)], 1u);
         __syncthreads();
-        uint32_t* gh = b.hist + (size_t(parity) * gridDim.x + blockIdx.x) * 256;
+        uint32_t* gh = b.hist + (size_t(parity) * b.size + b.rank) * 256;
         if (tid < 256) {
             uint32_t t = 0;
             for (int w = 0; w < nw; w++) t += hist[w * 256 + tid];
             gh[tid] = t;
         }
-        if (!grid_sync(b.bar, b.status)) return false;
+        if (!team_sync(b)) return false;
         if (tid < 256) {
             uint32_t all = 0, before = 0;
-            const uint32_t* col = b.hist + size_t(parity) * gridDim.x * 256 + tid;
-            for (int c = 0; c < int(gridDim.x); c++) {
-                if (c == int(blockIdx.x)) before = all;
+            const uint32_t* col = b.hist + size_t(parity) * b.size * 256 + tid;
+#pragma unroll 8
+            for (int c = 0; c < b.size; c++) {
+                if (c == b.rank) before = all;
                 all += __ldcg(col + size_t(c) * 256);
             }
             dsum[tid] = all;
@@ -522,7 +633,7 @@ __device__ bool grid_radix(uint64_t* K, int32_t* V, int n, int nbytes, const UbG
             if (valid && lane == __ffs(peers) - 1) off[d] += __popc(peers);
             __syncwarp();
         }
-        if (!grid_sync(b.bar, b.status)) return false;  // every scatter lands before the next pass reads
+        if (!team_sync(b)) return false;  // every scatter lands before the next pass reads
         uint64_t* tk = ka;
         ka = kb;
         kb = tk;
@@ -535,7 +646,7 @@ __device__ bool grid_radix(uint64_t* K, int32_t* V, int n, int nbytes, const UbG
             K[i] = __ldcg(ka + i);
             V[i] = __ldcg(va + i);
         }
-        if (!grid_sync(b.bar, b.status)) return false;
+        if (!team_sync(b)) return false;
     }
     return true;
 }
@@ -547,22 +658,22 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
     const uint32_t base = a.off[g];
     const int n0 = int(a.off[g + 1] - base);
     const int tid = threadIdx.x;
-    double* mypart = b.part + size_t(blockIdx.x) * kUbPart;
+    double* mypart = b.part + size_t(b.rank) * kUbPart;
     int32_t* X = a.mem + base;
     uint64_t* K = a.key + 2 * size_t(base);
     int32_t* V = a.val + 2 * size_t(base);
     int C0, C1;
     // members in particle order
-    cta_chunk(n0, C0, C1);
+    cta_chunk(b, n0, C0, C1);
     for (int t = C0 + tid; t < C1; t += blockDim.x) {
         const int32_t i = X[t];
         K[t] = uint64_t(uint32_t(i));
         V[t] = i;
     }
-    if (!grid_sync(b.bar, b.status)) return false;
-    if (!grid_radix(K, V, n0, 4, b, hist, dsum, dbase, skip, parity)) return false;
+    if (!team_sync(b)) return false;
+    if (!grid_radix(K, V, n0, 0, 4, b, hist, dsum, dbase, skip, parity)) return false;
     for (int t = C0 + tid; t < C1; t += blockDim.x) X[t] = __ldcg(V + t);
-    if (!grid_sync(b.bar, b.status)) return false;
+    if (!team_sync(b)) return false;
     const int32_t first = __ldcg(X);
     const float* a0 = a.pos + 3 * size_t(first);
     const float ax = a0[0], ay = a0[1], az = a0[2];
@@ -570,7 +681,7 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
     int n = n0, it = 0;
     while (it < a.max_iter) {
         it++;
-        cta_chunk(n, C0, C1);
+        cta_chunk(b, n, C0, C1);
         // 1. centre of mass and mean velocity: CTA sums, then all CTAs in order
         double s[7] = {0, 0, 0, 0, 0, 0, 0};
         for (int k = C0 + tid; k < C1; k += blockDim.x) {
@@ -588,10 +699,10 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
         }
         block_sums<7>(s, shd);
         if (tid < 7) mypart[tid] = s[tid];
-        if (!grid_sync(b.bar, b.status)) return false;
+        if (!team_sync(b)) return false;
         if (tid < 7) {
             double all;
-            (void)part_prefix(b.part, tid, &all);
+            (void)part_prefix(b, tid, &all);
             bc[tid] = all;
         }
         __syncthreads();
@@ -609,8 +720,22 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
             K[t] = uint64_t(__double_as_longlong(__dsqrt_rn(r2)));
             V[t] = i;
         }
-        if (!grid_sync(b.bar, b.status)) return false;
-        if (!grid_radix(K, V, n, 8, b, hist, dsum, dbase, skip, parity)) return false;
+        if (!team_sync(b)) return false;
+        if (!grid_radix(K, V, n, 4, 8, b, hist, dsum, dbase, skip, parity)) return false;
+        bool ok = true;
+        for (int t = C0 + tid; t < C1; t += blockDim.x) ok &= fix_run(K, V, n, t);
+        const int longrun = __syncthreads_or(!ok);
+        if (tid == 0) mypart[12] = longrun ? 1.0 : 0.0;
+        if (!team_sync(b)) return false;
+        if (tid == 0) {
+            double all;
+            (void)part_prefix(b, 12, &all);
+            bc[7] = all;
+        }
+        __syncthreads();
+        if (bc[7] > 0.0 && !(grid_radix(K, V, n, 0, 4, b, hist, dsum, dbase, skip, parity) &&
+                             grid_radix(K, V, n, 4, 8, b, hist, dsum, dbase, skip, parity)))
+            return false;
         // 2-3. shell sums: thread chunks inside the CTA's chunk; the mass
         // before and m/r after come from block scans and the CTA partials
         const int ch = (C1 - C0 + int(blockDim.x) - 1) / int(blockDim.x);
@@ -636,10 +761,10 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
             mypart[9] = cta_q;
             mypart[10] = double(cta_z);
         }
-        if (!grid_sync(b.bar, b.status)) return false;
+        if (!team_sync(b)) return false;
         if (tid < 3) {
             double all;
-            const double before = part_prefix(b.part, 8 + tid, &all);
+            const double before = part_prefix(b, 8 + tid, &all);
             bc[tid] = before;
             bc[3 + tid] = all;
         }
@@ -668,10 +793,10 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
         long long cta_keep;
         const long long dst_t = block_exclusive((long long)nk, reinterpret_cast<long long*>(shi), &cta_keep);
         if (tid == 0) mypart[11] = double(cta_keep);
-        if (!grid_sync(b.bar, b.status)) return false;
+        if (!team_sync(b)) return false;
         if (tid == 0) {
             double all;
-            const double before = part_prefix(b.part, 11, &all);
+            const double before = part_prefix(b, 11, &all);
             bc[0] = before;
             bc[1] = all;
         }
@@ -683,35 +808,64 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
             const int32_t i = V[k];  // this thread's own marks
             if (i >= 0) X[d++] = i;
         }
-        if (!grid_sync(b.bar, b.status)) return false;
+        if (!team_sync(b)) return false;
         n = int(n_keep);
     }
     const bool discard = 5ll * (n0 - n) > 2ll * n0;
-    cta_chunk(n, C0, C1);
+    cta_chunk(b, n, C0, C1);
     if (!discard)
         for (int k = C0 + tid; k < C1; k += blockDim.x) a.group_out[__ldcg(X + k)] = int32_t(g);
-    if (blockIdx.x == 0 && tid == 0) {
+    if (b.rank == 0 && tid == 0) {
         a.n_kept[g] = discard ? 0 : n;
         a.iters[g] = it;
     }
     // the partial slots and X are reused by the next group
-    return grid_sync(b.bar, b.status);
+    return team_sync(b);
 }
 
-// The groups above a.grid_min, one after another, each with the whole grid
-// (a cooperative launch: every CTA resident).  A barrier that runs out ends
-// the kernel with CWTHF_E_TIMEOUT.
-__global__ void __launch_bounds__(kUbThreads) k_ub_grid(UbArgs a, UbGrid b) {
+// The listed groups above a.grid_min, one after another with the whole grid
+// (those of a big team's size left out), then the teams' groups (a cooperative
+// launch: every CTA resident).  A barrier that runs out ends the kernel with
+// CWTHF_E_TIMEOUT.  A team's scratch is that of its CTAs, so teams of either
+// size never share any.
+__global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
     __shared__ double shd[8 * kUbWarps];
     __shared__ int64_t shi[kUbWarps + 1];
     __shared__ uint32_t hist[kUbWarps * 256];
     __shared__ uint32_t dsum[256], dbase[256];
     __shared__ int skip;
-    const int64_t n_groups = a.d_groups ? int64_t(*a.d_groups) : a.n_groups;
+    b.size = int(gridDim.x);
+    b.rank = int(blockIdx.x);
+    const unsigned n_large = a.ctl[kUbLarge], n_medium = a.ctl[kUbMedium];  // counted by k_ub_group
     int parity = 0;
-    for (int64_t g = 0; g < n_groups; g++) {
-        if (int64_t(a.off[g + 1] - a.off[g]) <= a.grid_min) continue;
+    for (unsigned i = 0; i < n_large; i++) {
+        const uint32_t g = a.list[a.list_cap - 1 - int64_t(i)];
+        if (big_team_group(a.off[g + 1] - a.off[g])) continue;
         if (!unbind_group_grid(a, b, g, shd, shi, hist, dsum, dbase, &skip, parity)) return;
+    }
+    for (int big = 1; big >= 0; big--) {
+        const int size = big ? kUnbindBigTeam : kUnbindTeam;
+        const int team = int(blockIdx.x) / size, first = team * size;
+        if (first + size > int(gridDim.x)) continue;  // a rest too small for a team
+        UbGrid tm;
+        tm.part = b.part + size_t(first) * kUbPart;
+        tm.hist = b.hist + size_t(first) * 2 * 256;
+        unsigned* words = b.bar + kUbTeamWords + 4 * (team + (big ? kUnbindGridCtaCap / kUnbindTeam : 0));
+        tm.bar = words;
+        tm.status = b.status;
+        tm.size = size;
+        tm.rank = int(blockIdx.x) - first;
+        parity = 0;
+        for (;;) {
+            if (tm.rank == 0 && threadIdx.x == 0) __stcg(words + 2, atomicAdd(a.ctl + (big ? kUbNextBig : kUbNext), 1u));
+            if (!team_sync(tm)) return;
+            const unsigned i = __ldcg(words + 2);
+            if (!team_sync(tm)) return;  // every CTA has read the number before the next one is written
+            if (i >= (big ? n_large : n_medium)) break;  // the same in the whole team
+            const uint32_t g = big ? a.list[a.list_cap - 1 - int64_t(i)] : a.list[i];
+            if (big && !big_team_group(a.off[g + 1] - a.off[g])) continue;  // done by the whole grid
+            if (!unbind_group_grid(a, tm, g, shd, shi, hist, dsum, dbase, &skip, parity)) return;
+        }
     }
 }
 
@@ -743,14 +897,14 @@ int unbind_groups(cwthf_ctx* ctx, const float* pos, const float* vel, const floa
     if (e != cudaSuccess) return cuda_status(e);
     const int blocks = ctx->sm_count * 8;
     CWTHF_LAUNCH(ctx, s, "k_ub_count",
-                 k_ub_count<<<blocks, 256, 0, s>>>(mass, mass_unit, group, np, n_groups, d_groups, cnt, group_out,
-                                                   ctx->d_status));
+                 k_ub_bin<false><<<blocks, kBinThreads, 0, s>>>(mass, mass_unit, group, np, n_groups, d_groups, nullptr,
+                                                                cnt, nullptr, group_out, ctx->d_status));
     // in place: offsets, cnt[groups] = members
     int rc = d_groups ? scan_u32_dev(ctx, cnt, cnt, d_groups, n_groups, s) : scan_u32(ctx, cnt, cnt, n_groups, s);
     if (rc) return rc;
     CWTHF_LAUNCH(ctx, s, "k_ub_scatter",
-                 k_ub_scatter<<<blocks, 256, 0, s>>>(group, np, n_groups, d_groups, cnt, cur, ctx->ub_mem,
-                                                     ctx->d_status));
+                 k_ub_bin<true><<<blocks, kBinThreads, 0, s>>>(nullptr, 1.0, group, np, n_groups, d_groups, cnt, cur,
+                                                               ctx->ub_mem, nullptr, ctx->d_status));
     if (n_groups > 0) {
         UbArgs a;
         a.pos = pos;
@@ -770,12 +924,17 @@ int unbind_groups(cwthf_ctx* ctx, const float* pos, const float* vel, const floa
         a.group_out = group_out;
         a.n_kept = n_kept;
         a.iters = iters;
+        // the lists of larger groups take the place of the scatter's cursors
+        a.list = cur;
+        a.list_cap = n_groups;
+        a.ctl = ctx->ub_bar;
+        if ((e = cudaMemsetAsync(ctx->ub_bar, 0, kUbBarWords * 4, s)) != cudaSuccess) return cuda_status(e);
         const unsigned grid = unsigned(std::min<int64_t>(n_groups, int64_t(ctx->sm_count) * 4));
         CWTHF_LAUNCH(ctx, s, "k_ub_group", k_ub_group<<<grid, kUbThreads, 0, s>>>(a));
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e);
-        // the large groups: one cooperative launch (its barrier state starts cleared)
-        if ((e = cudaMemsetAsync(ctx->ub_bar, 0, 16, s)) != cudaSuccess) return cuda_status(e);
+        // the larger groups: one cooperative launch
         UbGrid b;
+        b.size = b.rank = 0;  // set on the device
         b.part = ctx->ub_part;
         b.hist = ctx->ub_hist;
         b.bar = ctx->ub_bar;
