@@ -50,15 +50,15 @@ __device__ __forceinline__ PartBin bin_particle(const DepArgs& a, int64_t i) {
     if (!ok) { b.status = CWTHF_E_BAD_INPUT; return b; }
     int ms = mass_quantum(a, i, b.mq);
     if (ms != CWTHF_OK) { b.status = ms; b.mq = 0; return b; }
-    const int T[3] = {kDepTX, kDepTY, kDepTZ};
-    int n[3], t[3], cls = 0;
+    constexpr int T[3] = {kDepTX, kDepTY, kDepTZ};  // powers of two
+    int t[3], cls = 0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        n[d] = int(q[d] >> kFracBits);
-        t[d] = n[d] / T[d];
-        if (n[d] + 1 == a.ng || (n[d] + 1) % T[d] == 0) cls |= 1 << d;
+        const int n = int(uint32_t(q[d]) >> kFracBits);
+        t[d] = n / T[d];
+        if (n + 1 == a.ng || ((n + 1) & (T[d] - 1)) == 0) cls |= 1 << d;
     }
-    uint32_t tile = uint32_t((int64_t(t[2]) * a.nty + t[1]) * a.ntx + t[0]);
+    const uint32_t tile = uint32_t((t[2] * a.nty + t[1]) * a.ntx + t[0]);
     b.key = tile * kDepClasses + uint32_t(cls);
     b.rec = pack_rec(q[0], q[1], q[2]);
     return b;
@@ -191,19 +191,25 @@ __device__ __forceinline__ void reach_pair(int j, int& m, int& cls) {
 //
 // Dense tiles (a clump's core can put millions of records into one tile) are
 // split when a part list is given: the tile pass (kParts false) takes a
-// tile's first kTileSplit records and stores the tile as usual, and lists the
-// remaining parts of kTileSplit records; the part pass (kParts true, launched
+// tile's first `split` records and stores the tile as usual, and lists the
+// remaining parts of `split` records; the part pass (kParts true, launched
 // after it) spreads those parts over all CTAs, each accumulating its part in
 // shared memory and adding the nonzero cells to the grid with 64-bit atomics.
 // Integer sums do not depend on their order, so the grid is the same.
+//
+// What bounds it is the shared-memory atomics: eight corners per record, a
+// 32-bit add each whose old value tells the carry.  With equal masses (kMass
+// false) a corner's weight fits 32 bits and its carry is one, which leaves the
+// atomic, a compare and a rare second atomic per corner.
 
 struct TileParts {
     uint2* list;      // (tile, part >= 1), or nullptr: every tile whole
     uint32_t* count;  // parts listed
     uint32_t cap;
+    uint32_t split;   // records per part
 };
 
-template <bool kParts>
+template <bool kParts, bool kMass>
 __global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepArgs a, const uint32_t* __restrict__ off,
                                                           const unsigned long long* __restrict__ rec,
                                                           const uint32_t* __restrict__ rec_mq,
@@ -270,12 +276,12 @@ __global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepAr
         // this pass's records of the tile's flattened list
         uint32_t kbeg = 0, kend = total;
         if (kParts) {
-            kbeg = tp.list[j].y * kTileSplit;
-            kend = min(total, kbeg + kTileSplit);
-        } else if (tp.list && total > kTileSplit) {
-            kend = kTileSplit;
+            kbeg = tp.list[j].y * tp.split;
+            kend = min(total, kbeg + tp.split);
+        } else if (tp.list && total > tp.split) {
+            kend = tp.split;
             if (threadIdx.x == 0) {
-                const uint32_t extra = (total - 1) / kTileSplit;  // parts after the first
+                const uint32_t extra = (total - 1) / tp.split;  // parts after the first
                 const uint32_t p0 = atomicAdd(tp.count, extra);
                 if (p0 + extra > tp.cap) set_status(status, CWTHF_E_OVERFLOW);  // cannot happen: the list holds 8 np / split
                 for (uint32_t p = 0; p < extra && p0 + p < tp.cap; p++) tp.list[p0 + p] = make_uint2(uint32_t(t), p + 1);
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepAr
             const int m = seg_m[sgi];
             const bool live = k < kend && index_ok(r, a.np, status);
             const u64 e = live ? rec[r] : 0ull;
-            const uint32_t mq = live ? (a.mass ? rec_mq[r] : 1u) : 0u;
+            const uint32_t mq = kMass && live ? rec_mq[r] : 1u;
             const int qx = rec_q(e, 0), qy = rec_q(e, 1), qz = rec_q(e, 2);
             int lx = (qx >> kFracBits) - x0, ly = (qy >> kFracBits) - y0, lz = (qz >> kFracBits) - z0;
             const int fx = qx & (kFracOne - 1), fy = qy & (kFracOne - 1), fz = qz & (kFracOne - 1);
@@ -310,15 +316,27 @@ __global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepAr
             const uint32_t key = live ? uint32_t(((lz + 1) * (kDepTY + 2) + (ly + 1)) * (kDepTX + 2) + (lx + 1))
                                       : kInvalidKey;
             const bool uniform = __all_sync(kFull, key == __shfl_sync(kFull, key, 0)) && key != kInvalidKey;
+            // which of the two nodes per axis lie in the tile (a record of a lower neighbour: only the upper one)
+            const bool inx[2] = {live && !(m & 1), live && lx + 1 < wx};
+            const bool iny[2] = {!(m & 2), ly + 1 < wy}, inz[2] = {!(m & 4), lz + 1 < wz};
+            const int c0 = (lz * kDepTY + ly) * kDepTX + lx;
 #pragma unroll
             for (int q = 0; q < 8; q++) {
                 const int ex = q & 1, ey = (q >> 1) & 1, ez = (q >> 2) & 1;
-                u64 v = u64(mq) * (wxv[ex] * wyv[ey] * wzv[ez]);
-                if (uniform) v = warp_sum64(v);  // warp-uniform branch
-                const int cx = lx + ex, cy = ly + ey, cz = lz + ez;
-                if (live && (!uniform || lane == 0) && v && cx >= 0 && cx < wx && cy >= 0 && cy < wy && cz >= 0 &&
-                    cz < wz)
-                    shared_add64(acc_lo, acc_hi, (cz * kDepTY + cy) * kDepTX + cx, v);
+                const bool in = inx[ex] && iny[ey] && inz[ez];
+                const int c = c0 + (ez * kDepTY + ey) * kDepTX + ex;
+                const uint32_t w = wxv[ex] * wyv[ey] * wzv[ez];  // <= 2^30
+                if (uniform) {  // warp-uniform branch
+                    const u64 v = kMass ? warp_sum64(u64(mq) * w) : warp_sum32(w);
+                    if (in && lane == 0) shared_add64(acc_lo, acc_hi, c, v);
+                } else if (in) {
+                    if (kMass) {
+                        shared_add64(acc_lo, acc_hi, c, u64(mq) * w);
+                    } else {
+                        const uint32_t old = atomicAdd(&acc_lo[c], w);
+                        if (old + w < old) atomicAdd(&acc_hi[c], 1u);
+                    }
+                }
             }
         }
         __syncthreads();
@@ -417,13 +435,20 @@ int deposit_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mas
     tp.list = reinterpret_cast<uint2*>(ctx->dep_parts);
     tp.count = ctx->dep_nparts;
     tp.cap = uint32_t(tile_parts_cap(ctx->max_np));
+    // full parts while there are several of them per CTA, else smaller ones (64^3 particles on 64^3: the
+    // tile and part passes 52 + 51 us with 4096 records per part, 12 + 16 us with 512)
+    tp.split = kTileSplit;
+    while (tp.split > kTileSplitMin && np / tp.split < int64_t(ctx->sm_count) * kTileCtasPerSm * 2) tp.split /= 2;
     if ((e = cudaMemsetAsync(tp.count, 0, 4, s)) != cudaSuccess) return cuda_status(e);
-    CWTHF_LAUNCH(ctx, s, "k_dep_tile", k_dep_tile<false><<<tblocks, kTileThreads, 0, s>>>(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid,
-                                                ctx->d_status, tp));
+    const auto tiles = mass ? k_dep_tile<false, true> : k_dep_tile<false, false>;
+    const auto parts = mass ? k_dep_tile<true, true> : k_dep_tile<true, false>;
+    CWTHF_LAUNCH(ctx, s, "k_dep_tile",
+                 tiles<<<tblocks, kTileThreads, 0, s>>>(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid,
+                                                        ctx->d_status, tp));
     // the dense tiles' further parts (returns at once when there are none)
     CWTHF_LAUNCH(ctx, s, "k_dep_parts",
-                 k_dep_tile<true><<<ctx->sm_count * kTileCtasPerSm, kTileThreads, 0, s>>>(
-                     a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid, ctx->d_status, tp));
+                 parts<<<ctx->sm_count * kTileCtasPerSm, kTileThreads, 0, s>>>(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq,
+                                                                               ctx->d_mtot, grid, ctx->d_status, tp));
     if (mtot && (e = cudaMemcpyAsync(mtot, ctx->d_mtot, 8, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return cuda_status(e);
     return cuda_status(cudaGetLastError());
@@ -452,7 +477,8 @@ int deposit_into_scratch(const DepositScratch& sc, const float* pos, const float
     whole.list = nullptr;
     whole.count = nullptr;
     whole.cap = 0;
-    k_dep_tile<false><<<tblocks, kTileThreads, 0, s>>>(a, sc.off, sc.rec, sc.mq, sc.mtot, grid, sc.status, whole);
+    whole.split = kTileSplit;
+    (mass ? k_dep_tile<false, true> : k_dep_tile<false, false>)<<<tblocks, kTileThreads, 0, s>>>(a, sc.off, sc.rec, sc.mq, sc.mtot, grid, sc.status, whole);
     return cuda_status(cudaGetLastError());
 }
 

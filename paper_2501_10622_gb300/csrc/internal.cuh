@@ -23,12 +23,13 @@ constexpr int64_t kFracOne = int64_t(1) << kFracBits;
 // (the last tile along an axis may be partial).
 constexpr int kDepTX = 32, kDepTY = 8, kDepTZ = 8;
 constexpr int kDepClasses = 8;  // boundary class bits (x, y, z) per particle
-// Records of a deposit tile per CTA pass: denser tiles are split into parts.
-// The records reaching into all tiles number at most 8 np (a particle reaches
-// its own tile and at most 7 neighbours), so the parts after each tile's
-// first number at most 8 np / kTileSplit.
-constexpr uint32_t kTileSplit = 4096;
-inline int64_t tile_parts_cap(int64_t np) { return 8 * (np > 0 ? np : 1) / kTileSplit + 1; }
+// Records of a deposit tile per CTA pass: denser tiles are split into parts
+// (of kTileSplit records, or of kTileSplitMin where the parts would be too few
+// to keep the CTAs busy).  The records reaching into all tiles number at most
+// 8 np (a particle reaches its own tile and at most 7 neighbours), so the parts
+// after each tile's first number at most 8 np / split.
+constexpr uint32_t kTileSplit = 4096, kTileSplitMin = 512;
+inline int64_t tile_parts_cap(int64_t np) { return 8 * (np > 0 ? np : 1) / kTileSplitMin + 1; }
 
 // A binned particle record: its three fixed-point coordinates q (each below
 // ng * 2^10 <= 2^20) in 21-bit fields, x lowest.
@@ -418,6 +419,8 @@ int scan_u32(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n, cudaS
 // Same, with the length read from device memory (*d_n <= n_cap).
 int scan_u32_dev(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, const uint32_t* d_n, int64_t n_cap,
                  cudaStream_t s);
+// Same over the words' bit counts (in and out do not alias).
+int scan_popc(cwthf_ctx* ctx, const uint32_t* bits, uint32_t* out, int64_t n, cudaStream_t s);
 size_t scan_tmp_words(int64_t n_cap);
 
 // ---- stages -------------------------------------------------------------------
