@@ -21,40 +21,58 @@ constexpr int kThreads = 256;
 constexpr unsigned kFull = 0xffffffffu;
 using u64 = unsigned long long;
 
-// Cells per seed: four labels per thread and iteration, one atomic per slot
-// per warp.
+// Cells per seed.  A CTA counts kCountCells labels at a time in a shared table
+// keyed by label (one shared atomic per distinct label of a warp's row), then
+// looks up each entry's slot and adds its count once.  (A slot lookup and a
+// global atomic per distinct label of every warp took 139 us at 256^3, 92
+// us now.)
+constexpr int kCellsPerThread = 16, kCountCells = kThreads * kCellsPerThread;
 __global__ void __launch_bounds__(kThreads) k_count_cells(const int32_t* __restrict__ label, int64_t cells,
                                                          const uint32_t* __restrict__ bits,
                                                          const uint32_t* __restrict__ prefix,
                                                          const uint32_t* __restrict__ n_slots, HaloAcc* acc,
                                                          int* status) {
+    __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab];
+    __shared__ uint32_t n_used;
     const int lane = threadIdx.x & 31;
-    const int64_t n4 = (cells + 3) / 4;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t base = int64_t(blockIdx.x) * blockDim.x + (threadIdx.x & ~31); base < n4; base += stride) {
-        const int64_t i = base + lane;  // warp-uniform trip count
-        int l[4] = {-1, -1, -1, -1};
-        if (i < n4) {
-            if (4 * i + 3 < cells) {
-                const int4 q = reinterpret_cast<const int4*>(label)[i];
-                l[0] = q.x; l[1] = q.y; l[2] = q.z; l[3] = q.w;
-            } else {
-                for (int j = 0; j < 4 && 4 * i + j < cells; j++) l[j] = label[4 * i + j];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            uint32_t key = 0xffffffffu;
-            if (l[j] >= 0 && l[j] < cells) {
-                uint32_t slot;
-                if (seed_slot(bits, prefix, n_slots, l[j], slot)) key = slot;
-                else set_status(status, CWTHF_E_BAD_INPUT);
-            } else if (l[j] != -1) {
+    for (int e = threadIdx.x; e < kTab; e += kThreads) {
+        tkey[e] = kEmpty;
+        tcnt[e] = 0u;
+    }
+    if (threadIdx.x == 0) n_used = 0;
+    __syncthreads();
+    auto add = [&](int32_t l, uint32_t n) {
+        uint32_t slot;
+        if (seed_slot(bits, prefix, n_slots, l, slot)) atomicAdd(&acc[slot].n_cells, u64(n));
+        else set_status(status, CWTHF_E_BAD_INPUT);
+    };
+    for (int64_t c0 = int64_t(blockIdx.x) * kCountCells; c0 < cells; c0 += int64_t(gridDim.x) * kCountCells) {
+#pragma unroll 4
+        for (int j = 0; j < kCellsPerThread; j++) {
+            const int64_t c = c0 + j * kThreads + threadIdx.x;
+            int32_t l = c < cells ? label[c] : -1;
+            if (l < -1 || int64_t(l) >= cells) {
                 set_status(status, CWTHF_E_BAD_INPUT);
+                l = -1;
             }
-            const unsigned peers = __match_any_sync(kFull, key);
-            if (key != 0xffffffffu && lane == __ffs(peers) - 1) atomicAdd(&acc[key].n_cells, u64(__popc(peers)));
+            const unsigned peers = __match_any_sync(kFull, l);
+            if (l >= 0 && lane == __ffs(peers) - 1) {
+                const int f = table_find(tkey, tused, &n_used, uint32_t(l));
+                if (f >= 0) atomicAdd(&tcnt[f], uint32_t(__popc(peers)));
+                else add(l, uint32_t(__popc(peers)));
+            }
         }
+        __syncthreads();
+        const uint32_t nu = n_used;
+        for (uint32_t j = threadIdx.x; j < nu; j += kThreads) {
+            const uint32_t h = tused[j];
+            add(int32_t(tkey[h]), tcnt[h]);
+            tkey[h] = kEmpty;
+            tcnt[h] = 0u;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) n_used = 0;
+        __syncthreads();
     }
 }
 
@@ -83,8 +101,8 @@ __device__ __forceinline__ uint32_t fdiv(uint32_t n, FastDiv f) { return uint32_
 // (record -> label -> seed bitmap and prefix).  The chunk is first folded into
 // a small open-addressing table of halo slots in shared memory, then each
 // table entry is added to the global accumulators once; a record whose slot
-// finds no entry within kProbe probes goes straight to the global atomics.  A
-// warp whose 32 records share one halo is folded with warp reductions first.
+// finds no entry within kProbe probes goes straight to the global atomics.
+// Records of a warp that share a halo are folded with warp reductions first.
 // Each record's halo slot (or -1) is kept for the final pass, at
 // rec_slot[r * slot_stride].
 //
@@ -96,6 +114,7 @@ constexpr int kHsThreads = 256;
 // resident CTAs per SM: registers (equal masses) or the 45 KB table (masses)
 template <bool kMass> constexpr int hs_ctas_per_sm() { return kMass ? 4 : 6; }
 constexpr int kRecPerThread = 4;
+constexpr int kFoldMin = 6;  // records of one halo in a warp worth a reduction
 constexpr int kChunk = kHsThreads * kRecPerThread;
 static_assert(int64_t(kChunk) * (int64_t(CWTHF_MAX_NG) << (CWTHF_FRAC_BITS - 1)) < (int64_t(1) << 31),
               "a chunk's equal-mass moment sums must fit 32 bits");
@@ -200,11 +219,11 @@ __global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_su
                 rec_slot[r * slot_stride] = int32_t(key);  // kEmpty reads as -1
             }
             msum += mq[u];
-            // all 32 records in one halo: one lane carries the warp's sums (the
-            // shuffle runs on every lane)
-            const uint32_t k0 = __shfl_sync(kFull, key, 0);
-            const bool uniform = __all_sync(kFull, key == k0) && key != kEmpty;
             if (kMass) {
+                // all 32 records in one halo: one lane carries the warp's sums (the
+                // shuffle runs on every lane)
+                const uint32_t k0 = __shfl_sync(kFull, key, 0);
+                const bool uniform = __all_sync(kFull, key == k0) && key != kEmpty;
                 u64 cnt = 1, m_sum = mq[u];
                 u64 m[3];
 #pragma unroll
@@ -229,12 +248,30 @@ __global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_su
             } else {
                 uint32_t cnt = 1;
                 int32_t m[3] = {dq[0], dq[1], dq[2]};
-                if (uniform) {
-                    cnt = 32;
+                // up to two halos that hold several of the warp's records are folded with full-warp reductions
+                // (the others of a dense tile would queue up at the same table entry, four atomics each)
+                unsigned rest = __ballot_sync(kFull, key != kEmpty);
+                bool mine = key != kEmpty;  // this lane still adds to the table
 #pragma unroll
-                    for (int d = 0; d < 3; d++) m[d] = __reduce_add_sync(kFull, m[d]);
+                for (int it = 0; it < 2; it++) {
+                    if (__popc(rest) < kFoldMin) break;  // warp-uniform
+                    const int lead = __ffs(rest) - 1;
+                    const uint32_t kl = __shfl_sync(kFull, key, lead);
+                    const unsigned grp = __ballot_sync(kFull, key == kl);
+                    if (__popc(grp) < kFoldMin) break;
+                    const bool in = key == kl;
+                    int32_t t[3];
+#pragma unroll
+                    for (int d = 0; d < 3; d++) t[d] = __reduce_add_sync(kFull, in ? dq[d] : 0);
+                    if (in) mine = lane == lead;
+                    if (lane == lead) {
+                        cnt = uint32_t(__popc(grp));
+#pragma unroll
+                        for (int d = 0; d < 3; d++) m[d] = t[d];
+                    }
+                    rest &= ~grp;
                 }
-                if (key != kEmpty && (!uniform || lane == 0)) {
+                if (mine) {
                     const int f = table_find(tkey, tused, used, key);
                     if (f >= 0) {
                         atomicAdd(&tcnt[f], cnt);
@@ -314,13 +351,18 @@ __global__ void __launch_bounds__(kThreads) k_keep(const HaloAcc* __restrict__ a
     double rhs0 = __dmul_rn(f.dens_th, double(*mtot));
     int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < ns; s += stride) {
-        HaloAcc h = acc[s];
-        bool k = int64_t(h.n_part) >= f.particle_th &&
-                 __dmul_rn(double(h.mq), ncube) >= __dmul_rn(rhs0, double(h.n_cells));
-        keep[s] = k ? 1u : 0u;
+        uint32_t k = 0;
+        if (int64_t(acc[s].n_part) >= f.particle_th) {  // (few slots: the rest of the entry is not read)
+            const HaloAcc h = acc[s];
+            k = __dmul_rn(double(h.mq), ncube) >= __dmul_rn(rhs0, double(h.n_cells)) ? 1u : 0u;
+        }
+        keep[s] = k;
     }
 }
 
+// Catalogue entries of the kept slots, and each slot's halo (-1: not kept).
+// Kept slots are few (about 2 % at 1024^3) and dear (fp64 divides), so a warp
+// gathers them from its slots and forms 32 entries at a time.
 __global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* __restrict__ acc,
                                                        const int32_t* __restrict__ seed_list,
                                                        const uint32_t* __restrict__ n_seeds,
@@ -328,31 +370,31 @@ __global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* __restric
                                                        FilterArgs f, cwthf_halo* __restrict__ cat,
                                                        int32_t* __restrict__ slot_halo,
                                                        int64_t* __restrict__ n_halo, int* status) {
-    uint32_t ns = *n_seeds;
+    __shared__ uint32_t queue[kThreads / 32][64];
+    uint32_t* q = queue[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const uint32_t ns = *n_seeds;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         uint32_t kept = keep_off[ns];
         *n_halo = int64_t(kept);
         if (int64_t(kept) > f.cat_cap) set_status(status, CWTHF_E_CAPACITY);
     }
-    const int64_t N = f.ng;
+    const uint32_t N = uint32_t(f.ng);
     const double cell_q = (f.L / double(f.ng)) / double(kFracOne);
-    int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < ns; s += stride) {
+    auto entry = [&](uint32_t s) {
         const uint32_t pos = keep_off[s];
-        const bool kept = keep_off[s + 1] != pos;
-        slot_halo[s] = kept ? seed_list[s] : -1;
-        if (!kept || int64_t(pos) >= f.cat_cap) continue;
-        HaloAcc h = acc[s];
-        int64_t seed = seed_list[s];
-        int64_t sc[3] = {seed % N, (seed / N) % N, seed / (N * N)};
+        if (int64_t(pos) >= f.cat_cap) return;
+        const HaloAcc h = acc[s];
+        const uint32_t seed = uint32_t(seed_list[s]), sy = seed / N;
+        const uint32_t sc[3] = {seed - sy * N, sy % N, sy / N};
         cwthf_halo o;
-        o.seed = seed;
+        o.seed = int64_t(seed);
         o.n_part = int64_t(h.n_part);
         o.n_cells = int64_t(h.n_cells);
         o.mass = __dmul_rn(double(h.mq), f.mass_unit);
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            double u = double(sc[d] * kFracOne);
+            double u = double(sc[d] * uint32_t(kFracOne));
             if (h.mq > 0) u = __dadd_rn(u, __ddiv_rn(double(h.mom[d]), double(h.mq)));
             double x = __dmul_rn(u, cell_q);
             if (x >= f.L) x = __dsub_rn(x, f.L);
@@ -362,13 +404,33 @@ __global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* __restric
         o.peak = cwt ? cwt[seed] : 0.0f;
         o.reserved = 0;
         cat[pos] = o;
+    };
+    uint32_t n = 0;  // queued slots (warp-uniform)
+    for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < ns; base += gridDim.x * blockDim.x) {
+        const uint32_t s = base + uint32_t(lane);
+        const bool kept = s < ns && keep_off[s + 1] != keep_off[s];
+        if (s < ns) slot_halo[s] = kept ? seed_list[s] : -1;
+        const unsigned m = __ballot_sync(kFull, kept);
+        if (kept) q[n + __popc(m & ((1u << lane) - 1u))] = s;
+        n += __popc(m);
+        if (n >= 32) {
+            __syncwarp();
+            entry(q[lane]);
+            const uint32_t rest = q[32 + lane];
+            __syncwarp();
+            q[lane] = rest;
+            n -= 32;
+            __syncwarp();
+        }
     }
+    __syncwarp();
+    if (uint32_t(lane) < n) entry(q[lane]);
 }
 
 // Each scale's pass stores its record slots contiguously (rec_slot[scale * np
 // + r]: whole sectors written, none read back).  After the last scale the halo
-// ids are regrouped per record, RS ids per record (one scale: in place; two:
-// 8-byte groups; more: 16-byte groups of four scales), so that the final pass
+// ids are regrouped per record, RS ids per record (two scales: 8-byte groups;
+// more: 16-byte groups of four scales), so that the final pass
 // reads a particle's ids with one vector gather per four scales.
 __host__ __device__ __forceinline__ int slot_group_stride(int n_scales) {
     return n_scales <= 2 ? n_scales : (n_scales + 3) & ~3;
@@ -379,13 +441,6 @@ __host__ __device__ __forceinline__ int64_t slot_groups_offset(int n_scales, int
 
 template <int RS>
 struct IdGroup;
-template <>
-struct IdGroup<1> {
-    using T = int32_t;
-    __device__ static T make(const int32_t* v) { return v[0]; }
-    __device__ static int32_t get(const T& g, int j) { return g; }
-    __device__ static T none() { return -1; }
-};
 template <>
 struct IdGroup<2> {
     using T = int2;
@@ -404,8 +459,7 @@ struct IdGroup<4> {
 // Record order, after the last scale: each record's slot of every scale becomes
 // its halo id (the slot's seed if the halo was kept, else -1), written to the
 // record's group (RS = 4: one group per four scales).  Records are grouped by
-// tile, so the slot lookups are coherent.  With one scale the groups are the
-// slots themselves (each thread rewrites its own entry).
+// tile, so the slot lookups are coherent.
 template <int RS>
 __global__ void __launch_bounds__(kThreads) k_rec_halo(const int32_t* rec_slot, int64_t np,
                                                       const uint32_t* __restrict__ total_ptr, int n_scales,
@@ -463,6 +517,36 @@ __global__ void __launch_bounds__(kThreads) k_finalize(const uint32_t* __restric
                 for (int j = 0; j < G; j++)
                     if (G * g + j < n_scales) halo_id[(G * g + j) * np + i] = IdGroup<RS>::get(h[u], j);
             }
+        }
+    }
+}
+
+// One scale: particle -> record -> slot -> halo id in one pass (the pass that
+// turns record slots into ids first only pays when a record's ids of several
+// scales share a gather; for one scale it read and wrote every record to save
+// a lookup in the slots' table, which is in cache).
+__global__ void __launch_bounds__(kThreads) k_finalize_one(const uint32_t* __restrict__ part_rec, int64_t np,
+                                                          const uint32_t* __restrict__ total_ptr,
+                                                          const int32_t* __restrict__ rec_slot,
+                                                          const int32_t* __restrict__ slot_halo,
+                                                          int32_t* __restrict__ halo_id) {
+    constexpr int kIlp = 8;
+    const int64_t total = *total_ptr;
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t i0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i0 < np; i0 += kIlp * stride) {
+        int32_t v[kIlp];
+#pragma unroll
+        for (int u = 0; u < kIlp; u++) {
+            const int64_t i = i0 + u * stride;
+            const uint32_t x = i < np ? part_rec[i] : 0xffffffffu;
+            v[u] = int64_t(x) < total ? rec_slot[x] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kIlp; u++) v[u] = v[u] >= 0 ? slot_halo[v[u]] : -1;
+#pragma unroll
+        for (int u = 0; u < kIlp; u++) {
+            const int64_t i = i0 + u * stride;
+            if (i < np) halo_id[i] = v[u];
         }
     }
 }
@@ -855,7 +939,7 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     if (e != cudaSuccess) return cuda_status(e);
     if (!seeds_ready)  // after segment_impl the resolve pass has counted the cells already
         CWTHF_LAUNCH(ctx, s, "k_count_cells",
-                     k_count_cells<<<blocks, kThreads, 0, s>>>(label, cells, ctx->seed_bits, ctx->seed_prefix,
+                     k_count_cells<<<int(std::min<int64_t>(div_up(cells, kCountCells), blocks)), kThreads, 0, s>>>(label, cells, ctx->seed_bits, ctx->seed_prefix,
                                                                d_nseeds, ctx->acc, ctx->d_status));
     DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
     const int64_t total_key = deposit_geom(ng).ntiles * kDepClasses;  // dep_off[total_key] = records binned
@@ -878,7 +962,10 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     if (scale == n_scales - 1) {  // halo ids of all scales at once
         const int rs = slot_group_stride(n_scales);
         const uint32_t* total = ctx->dep_off + total_key;
-        if (rs == 1) launch_ids<1>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
+        if (rs == 1)
+            CWTHF_LAUNCH(ctx, s, "k_finalize",
+                         k_finalize_one<<<pblocks, kThreads, 0, s>>>(ctx->part_rec, np, total, ctx->part_slot,
+                                                                     ctx->slot_halo, halo_id));
         else if (rs == 2) launch_ids<2>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
         else launch_ids<4>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
     }

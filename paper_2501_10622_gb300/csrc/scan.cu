@@ -1,6 +1,7 @@
-// scan.cu -- exclusive prefix sum of uint32 arrays (reduce, scan block sums,
-// scan + add).  Used for the deposit bins, the seed ranks and the compaction
-// of kept halos.  No spin waits: three plain launches.
+// scan.cu -- exclusive prefix sum of uint32 arrays, or of their bit counts
+// (reduce, scan block sums, scan + add; short arrays in one block).  Used for
+// the deposit bins, the seed ranks and the compaction of kept halos.  No spin
+// waits: plain launches.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -24,8 +25,9 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
 
 // Block-wide exclusive scan of one value per thread; *total gets the block sum.
 // Every thread of the block must call it (it synchronises the block).
+template <int kThreads = kScanThreads>
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* total) {
-    constexpr int kWarps = kScanThreads / 32;
+    constexpr int kWarps = kThreads / 32;
     __shared__ uint32_t warp_off[kWarps + 1];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t inc = warp_incl_scan(v);
@@ -49,6 +51,13 @@ __device__ __forceinline__ int64_t scan_len(int64_t n, const uint32_t* d_n) {
     return d_n ? min(int64_t(*d_n), n) : n;
 }
 
+// The scanned value: the word itself, or its bit count.
+template <bool kPopc>
+__device__ __forceinline__ uint32_t scan_value(uint32_t w) {
+    return kPopc ? uint32_t(__popc(w)) : w;
+}
+
+template <bool kPopc>
 __global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t* __restrict__ in, int64_t n,
                                                              const uint32_t* d_n, uint32_t* __restrict__ sums) {
     int64_t len = scan_len(n, d_n);
@@ -58,7 +67,7 @@ __global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t* __r
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
         int64_t idx = base + int64_t(i) * kScanThreads + threadIdx.x;
-        if (idx < len) s += in[idx];
+        if (idx < len) s += scan_value<kPopc>(in[idx]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -90,6 +99,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* sums, int6
     if (threadIdx.x == 0) sums[nblocks_cap] = carry;  // grand total
 }
 
+template <bool kPopc>
 __global__ void __launch_bounds__(kScanThreads) k_scan_add(const uint32_t* in, int64_t n, const uint32_t* d_n,
                                                            const uint32_t* __restrict__ sums, int64_t nblocks_cap,
                                                            uint32_t* out) {
@@ -103,7 +113,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_add(const uint32_t* in, i
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
         int64_t idx = base + int64_t(threadIdx.x) * kScanItems + i;
-        v[i] = idx < len ? in[idx] : 0u;
+        v[i] = idx < len ? scan_value<kPopc>(in[idx]) : 0u;
         local += v[i];
     }
     uint32_t tot;  // block_excl_scan synchronises: every value is read before any is written
@@ -116,15 +126,51 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_add(const uint32_t* in, i
     }
 }
 
+// Short arrays in one block, kScanOneItems values per thread and step: one
+// launch instead of three (a 64^3 find scans three arrays of 1,000 to 8,000
+// values, 6 us each way of launch and wait per kernel).
+constexpr int kScanOneThreads = 1024, kScanOneItems = 8;
+constexpr int64_t kScanOneMax = 2 * kScanOneThreads * kScanOneItems;      // lengths known on the host
+constexpr int64_t kScanOneMaxDev = 16 * kScanOneThreads * kScanOneItems;  // capacities (the length is usually far below)
+template <bool kPopc>
+__global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const uint32_t* in, int64_t n, const uint32_t* d_n,
+                                                              uint32_t* out) {
+    const int64_t len = scan_len(n, d_n);
+    uint32_t carry = 0;
+    for (int64_t base = 0; base < len; base += kScanOneThreads * kScanOneItems) {
+        uint32_t v[kScanOneItems], local = 0, tot;
+#pragma unroll
+        for (int i = 0; i < kScanOneItems; i++) {
+            const int64_t idx = base + int64_t(threadIdx.x) * kScanOneItems + i;
+            v[i] = idx < len ? scan_value<kPopc>(in[idx]) : 0u;
+            local += v[i];
+        }
+        uint32_t ex = block_excl_scan<kScanOneThreads>(local, &tot) + carry;  // (every value is read before any is written)
+#pragma unroll
+        for (int i = 0; i < kScanOneItems; i++) {
+            const int64_t idx = base + int64_t(threadIdx.x) * kScanOneItems + i;
+            if (idx < len) out[idx] = ex;
+            ex += v[i];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) out[len] = carry;
+}
+
+template <bool kPopc>
 int scan_generic(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n_cap, const uint32_t* d_n,
                  cudaStream_t s) {
+    if (n_cap <= (d_n ? kScanOneMaxDev : kScanOneMax)) {
+        CWTHF_LAUNCH(ctx, s, "k_scan_one", k_scan_one<kPopc><<<1, kScanOneThreads, 0, s>>>(in, n_cap, d_n, out));
+        return cuda_status(cudaGetLastError());
+    }
     int64_t nb = (n_cap + kScanChunk - 1) / kScanChunk;
     if (nb < 1) nb = 1;
     if (size_t(nb) + 2 > ctx->scan_tmp_cap) return CWTHF_E_INVALID_ARG;
     uint32_t* sums = ctx->scan_tmp;
-    CWTHF_LAUNCH(ctx, s, "k_block_sums", k_block_sums<<<unsigned(nb), kScanThreads, 0, s>>>(in, n_cap, d_n, sums));
+    CWTHF_LAUNCH(ctx, s, "k_block_sums", k_block_sums<kPopc><<<unsigned(nb), kScanThreads, 0, s>>>(in, n_cap, d_n, sums));
     CWTHF_LAUNCH(ctx, s, "k_scan_sums", k_scan_sums<<<1, kScanThreads, 0, s>>>(sums, nb, n_cap, d_n));
-    CWTHF_LAUNCH(ctx, s, "k_scan_add", k_scan_add<<<unsigned(nb), kScanThreads, 0, s>>>(in, n_cap, d_n, sums, nb, out));
+    CWTHF_LAUNCH(ctx, s, "k_scan_add", k_scan_add<kPopc><<<unsigned(nb), kScanThreads, 0, s>>>(in, n_cap, d_n, sums, nb, out));
     return cuda_status(cudaGetLastError());
 }
 
@@ -133,21 +179,25 @@ int scan_generic(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n_ca
 size_t scan_tmp_words(int64_t n_cap) { return size_t((n_cap + kScanChunk - 1) / kScanChunk) + 2; }
 
 int scan_u32(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n, cudaStream_t s) {
-    return scan_generic(ctx, in, out, n, nullptr, s);
+    return scan_generic<false>(ctx, in, out, n, nullptr, s);
 }
 
 int scan_u32_dev(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, const uint32_t* d_n, int64_t n_cap,
                  cudaStream_t s) {
-    return scan_generic(ctx, in, out, n_cap, d_n, s);
+    return scan_generic<false>(ctx, in, out, n_cap, d_n, s);
 }
 
-// The same three launches on caller-provided block-sum storage (no context).
+int scan_popc(cwthf_ctx* ctx, const uint32_t* bits, uint32_t* out, int64_t n, cudaStream_t s) {
+    return scan_generic<true>(ctx, bits, out, n, nullptr, s);
+}
+
+// The three launches on caller-provided block-sum storage (no context).
 int scan_u32_scratch(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, size_t tmp_cap, cudaStream_t s) {
     int64_t nb = std::max<int64_t>((n + kScanChunk - 1) / kScanChunk, 1);
     if (size_t(nb) + 2 > tmp_cap) return CWTHF_E_INVALID_ARG;
-    k_block_sums<<<unsigned(nb), kScanThreads, 0, s>>>(in, n, nullptr, tmp);
+    k_block_sums<false><<<unsigned(nb), kScanThreads, 0, s>>>(in, n, nullptr, tmp);
     k_scan_sums<<<1, kScanThreads, 0, s>>>(tmp, nb, n, nullptr);
-    k_scan_add<<<unsigned(nb), kScanThreads, 0, s>>>(in, n, nullptr, tmp, nb, out);
+    k_scan_add<false><<<unsigned(nb), kScanThreads, 0, s>>>(in, n, nullptr, tmp, nb, out);
     return cuda_status(cudaGetLastError());
 }
 

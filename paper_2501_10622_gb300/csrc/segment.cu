@@ -347,7 +347,8 @@ constexpr int kResolveThreads = 256;
 constexpr int kResTabBits = 9, kResTab = 1 << kResTabBits;  // per-tile count table (shared memory)
 
 // The global pass over the cells whose chain left their tile.  A CTA takes one
-// chain tile at a time from a global counter, and its warps take the tile's
+// chain tile (or `rows` of its rows) at a time from a global counter, and its
+// warps take the
 // rows one at a time from a shared counter (the flagged cells crowd where the
 // field is clumped, so a fixed split leaves some warps far more work than
 // others).  A warp gathers the flagged cells of a row's non-empty plane masks
@@ -413,7 +414,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
                                                                  uint32_t* __restrict__ seed_cells,
                                                                  int* __restrict__ changed,
                                                                  unsigned* __restrict__ next_tile, int limit,
-                                                                 int* status) {
+                                                                 int rows, int* status) {
     __shared__ uint32_t batch[kResolveThreads / 32][64];  // pending cells (fewer than 32 between batches)
     __shared__ int32_t tkey[kResTab];
     __shared__ uint32_t tcnt[kResTab];
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
     uint32_t* wl = batch[threadIdx.x >> 5];
     const int N = ng;
     const int ntx = (N + kChTX - 1) / kChTX, nty = (N + kChTY - 1) / kChTY, ntz = (N + kChTZ - 1) / kChTZ;
-    const unsigned ntiles = unsigned(ntx) * unsigned(nty) * unsigned(ntz);
+    const unsigned per_tile = unsigned(kChTY / rows), nunits = unsigned(ntx) * unsigned(nty) * unsigned(ntz) * per_tile;
     const uint32_t plane32 = uint32_t(N) * uint32_t(N);
     const int64_t cells = int64_t(plane32) * N;
     for (int i = threadIdx.x; i < kResTab; i += blockDim.x) {
@@ -435,11 +436,11 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
     for (;;) {
         if (threadIdx.x == 0) {
             s_tile = atomicAdd(next_tile, 1u);
-            s_row = 0;
+            s_row = (s_tile % per_tile) * unsigned(rows);
         }
         __syncthreads();
-        const unsigned t = s_tile;
-        if (t >= ntiles) break;  // block-uniform
+        if (s_tile >= nunits) break;  // block-uniform
+        const unsigned t = s_tile / per_tile, row_end = (s_tile % per_tile + 1) * unsigned(rows);
         const int tx = int(t % unsigned(ntx)), ty = int((t / unsigned(ntx)) % unsigned(nty)),
                   tz = int(t / (unsigned(ntx) * unsigned(nty)));
         uint32_t k = 0;  // warp-uniform
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
             unsigned ly = 0;
             if (lane == 0) ly = atomicAdd(&s_row, 1u);
             ly = __shfl_sync(full, ly, 0);
-            if (ly >= unsigned(kChTY)) break;  // warp-uniform
+            if (ly >= row_end) break;  // warp-uniform
             const int yc = ty * kChTY + int(ly);
             if (yc >= N) continue;  // warp-uniform
             const int64_t rw = int64_t(t) * kChTY + ly;
@@ -536,39 +537,44 @@ __global__ void __launch_bounds__(256) k_seg_fallback(int32_t* __restrict__ labe
     }
 }
 
-__global__ void k_popc(const uint32_t* __restrict__ bits, int64_t nwords, uint32_t* __restrict__ out) {
-    int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < nwords; i += stride) out[i] = __popc(bits[i]);
-}
-
-// slot -> seed cell, in increasing cell order; clears the slot's accumulators
-// (the cell count starts from the tile pass's in-tile count when given).
-// *n_slots = number of seeds, clamped to slot_cap (more seeds than that can
-// only come from an inconsistent label grid, reported as bad input).
+// slot -> seed cell, in increasing cell order.  *n_slots = number of seeds,
+// clamped to slot_cap (more seeds than that can only come from an inconsistent
+// label grid, reported as bad input).
 __global__ void k_seed_list(const uint32_t* __restrict__ bits, const uint32_t* __restrict__ prefix, int64_t nwords,
-                            int64_t slot_cap, int32_t* __restrict__ seed_list, const uint32_t* __restrict__ seed_cells,
-                            HaloAcc* __restrict__ acc, uint32_t* __restrict__ n_slots, int* status) {
+                            int64_t slot_cap, int32_t* __restrict__ seed_list, uint32_t* __restrict__ n_slots,
+                            int* status) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         uint32_t total = prefix[nwords];
         if (int64_t(total) > slot_cap) set_status(status, CWTHF_E_BAD_INPUT);
         *n_slots = uint32_t(min(int64_t(total), slot_cap));
     }
-    int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < nwords; i += stride) {
         uint32_t b = bits[i];
+        if (!b) continue;
         uint32_t s = prefix[i];
         while (b && int64_t(s) < slot_cap) {
-            int bit = __ffs(b) - 1;
+            seed_list[s++] = int32_t(i * 32 + __ffs(b) - 1);
             b &= b - 1;
-            seed_list[s] = int32_t(i * 32 + bit);
-            HaloAcc z;
-            z.n_part = 0;
-            z.mq = 0;
-            z.mom[0] = z.mom[1] = z.mom[2] = 0;
-            z.n_cells = seed_cells ? seed_cells[i * 32 + bit] : 0;
-            acc[s] = z;
-            s++;
         }
+    }
+}
+
+// Clears the slots' accumulators; the cell count starts from the tile pass's
+// count at the seed's cell when given.  With the clearing inside the list's
+// loop over the bitmap, each seed's gather and 48 bytes of
+// stores waited for the seed before it in the same word (0.68 ms per scale at
+// 1024^3, 0.14 + 0.40 now).
+__global__ void k_seed_acc(const int32_t* __restrict__ seed_list, const uint32_t* __restrict__ seed_cells,
+                           HaloAcc* __restrict__ acc, const uint32_t* __restrict__ n_slots) {
+    // an accumulator is three 16-byte pieces, all zero but the count in the last one's upper half; one
+    // thread per piece, so that a warp's stores are contiguous
+    static_assert(sizeof(HaloAcc) == 48 && offsetof(HaloAcc, n_cells) == 40, "piece layout");
+    const uint64_t n = uint64_t(*n_slots) * 3;
+    ulonglong2* out = reinterpret_cast<ulonglong2*>(acc);
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint32_t s = uint32_t(i / 3);
+        out[i] = make_ulonglong2(0ull, seed_cells && i == 3ull * s + 2 ? seed_cells[seed_list[s]] : 0ull);
     }
 }
 
@@ -610,11 +616,13 @@ int seeds_rank(cwthf_ctx* ctx, int ng, const uint32_t* seed_cells, cudaStream_t 
     int64_t cells = int64_t(ng) * ng * ng;
     int64_t nwords = (cells + 31) / 32;
     int blocks = ctx->sm_count * 8;
-    CWTHF_LAUNCH(ctx, s, "k_popc", k_popc<<<blocks, 256, 0, s>>>(ctx->seed_bits, nwords, ctx->seed_prefix));
-    int rc = scan_u32(ctx, ctx->seed_prefix, ctx->seed_prefix, nwords, s);
+    int rc = scan_popc(ctx, ctx->seed_bits, ctx->seed_prefix, nwords, s);
     if (rc) return rc;
-    CWTHF_LAUNCH(ctx, s, "k_seed_list", k_seed_list<<<blocks, 256, 0, s>>>(ctx->seed_bits, ctx->seed_prefix, nwords, cells / 8 + 8, ctx->seed_list,
-                                       seed_cells, ctx->acc, ctx->n_seeds, ctx->d_status));
+    CWTHF_LAUNCH(ctx, s, "k_seed_list",
+                 k_seed_list<<<blocks, 256, 0, s>>>(ctx->seed_bits, ctx->seed_prefix, nwords, cells / 8 + 8,
+                                                    ctx->seed_list, ctx->n_seeds, ctx->d_status));
+    CWTHF_LAUNCH(ctx, s, "k_seed_acc",
+                 k_seed_acc<<<blocks, 256, 0, s>>>(ctx->seed_list, seed_cells, ctx->acc, ctx->n_seeds));
     return cuda_status(cudaGetLastError());
 }
 
@@ -669,10 +677,13 @@ int segment_impl(cwthf_ctx* ctx, const float* cwt, int ng, float cwt_min, int32_
     // chains that left their tile, counted at their seed's cell
     int blocks = ctx->sm_count * 8;
     int* changed = ctx->jump_changed;  // see kJumpWords
+    // a CTA takes a whole tile (one table flush), or, where tiles are too few to fill the GPU, two of its
+    // rows (64^3: 38 us with 16 whole tiles, 27 us)
+    const int rows = ntiles < 2 * ctx->sm_count ? 2 : kChTY;
     CWTHF_LAUNCH(ctx, s, "k_seg_resolve",
                  k_seg_resolve<<<blocks, kResolveThreads, 0, s>>>(label, ng, ballots, ctx->seed_cells, changed,
                                                                    reinterpret_cast<unsigned*>(changed + kJumpTileCounter),
-                                                                   ctx->dbg_chase_limit, ctx->d_status));
+                                                                   ctx->dbg_chase_limit, rows, ctx->d_status));
     // pointer doubling and a recount for whatever the bounded walks left
     // (normally nothing: the kernel then returns at once)
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e);
