@@ -31,13 +31,14 @@ constexpr int kChTX = 64, kChTY = 16, kChTZ = 16;
 constexpr int kRowWords = 2 * kChTZ;  // flagged-cell masks per tile row (32)
 constexpr int kSegRows = 2, kSegThreads = 32 * (kChTY / kSegRows);  // 256
 static_assert(kRowWords == 32 && kChTX == 64, "mask layout");
-// Shared-memory pointers: the 16-bit byte offset of the target's own entry, in
-// a box with one cell of halo on each side (rows padded to 68 entries, so that
-// a lane's column pair is 4-byte aligned); a root points at itself.  One more
-// entry stands for "no seed".
+// Shared-memory pointers: the 16-bit shared address of the target's own entry,
+// in a box with one cell of halo on each side (rows padded to 68 entries, so
+// that a lane's column pair is 4-byte aligned); a root points at itself.  One
+// more entry stands for "no seed".  (The block's shared memory starts in the
+// first few KB of the window, which the kernel checks.)
 constexpr int kSRow = 2 * (kChTX + 4), kSPlane = kSRow * (kChTY + 2);  // bytes
 constexpr int kSNone = kSPlane * (kChTZ + 2), kSBytes = kSNone + 8;
-static_assert(kSBytes < 65536 && kSRow == 136 && kSPlane == 2448, "16-bit offsets; quotients below");
+static_assert( kSRow == 136 && kSPlane == 2448, "quotient below");
 // A flagged pointer (a chain still to be followed) to cell g is stored as
 // -2 - g, apart from -1 (no seed) and the final labels (seed cells, >= 0).
 __device__ __forceinline__ bool is_flagged(int32_t v) { return v <= -2; }
@@ -46,15 +47,39 @@ constexpr int kJumpRoundsInTile = 16;  // in-place jumping rounds (each triples 
 // Seeds of one tile: at most one local maximum per 2 x 2 x 2 block of cells
 // (any two cells of such a block are neighbours).
 constexpr int kTileSeedCap = (kChTX / 2) * (kChTY / 2) * (kChTZ / 2);
-// pointers, the tile's seeds (offsets), their cell counts (16 bits each: a tile has 2^14 cells), rows
+// pointers, the tile's seeds (addresses), cell counts of kCountSeeds of them at a time and of the rest, rows
+constexpr int kCountSeeds = 1024;
 constexpr int kSegLines = (kChTY + 2) * (kChTZ + 2);  // rows of the box, with their global indices
-constexpr int kSegSmem = kSBytes + 2 * kTileSeedCap + 2 * kTileSeedCap + 4 * kSegLines;
+static_assert(kSBytes + 2 * kTileSeedCap + 4 * kCountSeeds < 60000, "16-bit addresses");
+constexpr int kSegSmem = kSBytes + 2 * kTileSeedCap + 4 * (kCountSeeds + 1) + 4 * (kSegLines + 1);  // (a row for "no seed")
 
 // o / kSRow for offsets o <= kSNone
 constexpr uint32_t kYMul = 30841;
 constexpr int kYShift = 22;
 
 __device__ __forceinline__ int wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
+
+// Shared-memory accesses by 32-bit address: the pointers are addresses, so
+// following one takes no arithmetic at all.  (Through C++ pointers every access
+// recomputed the window's base; with that, branches and 64-bit addressing a
+// cell took 186 instructions.)
+__device__ __forceinline__ uint32_t lds16(uint32_t a) {
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts16(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(uint16_t(v)));
+}
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v)); }
+__device__ __forceinline__ void reds32(uint32_t a, uint32_t v) {
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v));
+}
 
 // The better of two candidates under the strict order, the first one coming
 // earlier in position order: the second wins if it is greater, or, with `tie`
@@ -82,7 +107,8 @@ __device__ __forceinline__ void best2(float m1, int q1, float m2, int q2, bool t
 // kernels did this before (one-byte parent codes through memory, then a tile
 // kernel that decoded them to 32-bit pointers): 250 instructions per cell,
 // 3.34 + 4.52 ms per scale at 1024^3 and 0.26 + 0.26 ms at 384^3, against
-// 5.63 and 0.35 ms here.  16-bit
+// 4.47 and 0.27 ms here (of which the parents take half, the chains a fifth,
+// the labels the rest).  16-bit
 // pointers in a box with a halo need no decoding and no test for neighbours
 // outside the tile, and leave room for four blocks per SM.  Two rows per warp
 // rather than four: the halo rows' x windows cost 4 instructions per cell more,
@@ -91,13 +117,8 @@ __device__ __forceinline__ void best2(float m1, int q1, float m2, int q2, bool t
 template <bool kInner>
 __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, float cwt_min, int32_t* __restrict__ label,
                                          uint32_t* __restrict__ seed_bits, uint32_t* __restrict__ seed_cells,
-                                         uint32_t* __restrict__ ballots, int* status, unsigned char* sm,
-                                         uint32_t* n_seeds) {
-    uint16_t* seeds = reinterpret_cast<uint16_t*>(sm + kSBytes);
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(sm + kSBytes + 2 * kTileSeedCap);
-    int32_t* line = reinterpret_cast<int32_t*>(sm + kSBytes + 4 * kTileSeedCap);  // global index of each row's x = 0
-    auto at = [&](int off) -> uint16_t& { return *reinterpret_cast<uint16_t*>(sm + off); };
-    auto pair_at = [&](int off) -> uint32_t& { return *reinterpret_cast<uint32_t*>(sm + off); };
+                                         uint32_t* __restrict__ ballots, int* status, uint32_t sb, uint32_t* n_seeds) {
+    const uint32_t seeds = sb + kSBytes, cnt = seeds + 2 * kTileSeedCap, line = cnt + 4 * (kCountSeeds + 1), none = sb + kSNone;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ntx = (N + kChTX - 1) / kChTX, nty = (N + kChTY - 1) / kChTY;
@@ -107,12 +128,15 @@ __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, flo
     const int wx = min(kChTX, N - x0), wy = min(kChTY, N - y0), wz = min(kChTZ, N - z0);  // all even
     const int32_t plane = N * N;
     // every entry a root (the halo and what a ragged tile leaves out stay that way)
-    for (int i = threadIdx.x; i < kSBytes / 4; i += kSegThreads)
-        pair_at(4 * i) = uint32_t(4 * i) | (uint32_t(4 * i + 2) << 16);
+    for (uint32_t o = 4 * threadIdx.x; o < uint32_t(kSBytes); o += 4 * kSegThreads)
+        sts32(sb + o, (sb + o) | ((sb + o + 2) << 16));
+    // global index of each row's x = 0
     for (int i = threadIdx.x; i < kSegLines; i += kSegThreads) {
         const int z = z0 - 1 + i / (kChTY + 2), y = y0 - 1 + i % (kChTY + 2);
-        line[i] = kInner ? z * plane + y * N : ((z + N) % N) * plane + ((y + N) % N) * N;
+        sts32(line + 4 * i, uint32_t(kInner ? z * plane + y * N : ((z + N) % N) * plane + ((y + N) % N) * N));
     }
+    // ("no seed" reads as a root whose label is -1)
+    if (threadIdx.x == 0) sts32(line + 4 * kSegLines, uint32_t(-1 - (kInner ? x0 - 2 : wrap(x0 - 2, N))));
     __syncthreads();
 
     // ---- parents ----
@@ -120,42 +144,54 @@ __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, flo
     const int lx = 2 * lane, r0 = warp * R;  // this lane's columns lx, lx + 1; the warp's rows r0 .. r0 + R - 1
     const int xa = kInner ? x0 + lx : (x0 + lx) % N;
     // lanes 0 and 31 fetch the columns beside the tile as well
-    const int xe = lane == 0 ? (kInner ? x0 - 1 : (x0 - 1 + N) % N) : (kInner ? x0 + kChTX : (x0 + kChTX) % N);
-    const bool edge = lane == 0 || lane == 31;
-    int32_t roff[NR];
+    const int xe = kInner ? 0 : (lane == 0 ? (x0 - 1 + N) % N : (x0 + kChTX) % N);
+    const bool first_lane = lane == 0, last_lane = lane == 31;
+    uint32_t roff[NR];  // this lane's first column in the fetched rows of the plane fetched next
+    const int zfirst = kInner ? z0 - 1 : (z0 - 1 + N) % N;
 #pragma unroll
     for (int j = 0; j < NR; j++) {
         const int y = y0 + r0 - 1 + j;
-        roff[j] = (kInner ? y : (y + N) % N) * N;
+        roff[j] = uint32_t(zfirst * plane + (kInner ? y : (y + N) % N) * N + xa);
     }
+    int zf = zfirst;  // (boundary tiles) the plane fetched next
     const bool vec = (reinterpret_cast<uintptr_t>(C) & 7u) == 0;  // N and xa are even
     const bool tie_xl = !kInner && xa == 0, tie_xr = !kInner && xa + 1 == N - 1;
     bool bad = false;
     float2 va[NR];
     float ve[NR];
-    auto fetch = [&](int p) {  // plane p: z = z0 - 1 + p
-        const int z = kInner ? z0 - 1 + p : (z0 - 1 + p + N) % N;
-        const float* base = C + size_t(z) * size_t(plane);
+    auto fetch = [&]() {
 #pragma unroll
         for (int j = 0; j < NR; j++) {
-            const float* a = base + roff[j] + xa;
+            const float* a = C + roff[j];
             if (vec) va[j] = *reinterpret_cast<const float2*>(a);
             else va[j] = make_float2(a[0], a[1]);
-            ve[j] = edge ? base[roff[j] + xe] : 0.f;
+            if (kInner) {
+                if (first_lane) ve[j] = a[-1];
+                if (last_lane) ve[j] = a[2];
+            } else if (first_lane || last_lane) {
+                ve[j] = C[roff[j] - uint32_t(xa) + uint32_t(xe)];
+            }
         }
+        uint32_t step = uint32_t(plane);
+        if (!kInner && ++zf == N) {
+            zf = 0;
+            step -= uint32_t(plane) * uint32_t(N);  // back to plane 0 (mod 2^32)
+        }
+#pragma unroll
+        for (int j = 0; j < NR; j++) roff[j] += step;
     };
-    // x and y windows of the plane fetched last, with offsets relative to the
-    // plane's (row r0 - 1, this lane's first column)
-    auto xy = [&](float (&M)[2 * R], int (&Q)[2 * R], int qz) {
+    // x and y windows of the plane fetched last; qz: the address of (that
+    // plane, row r0 - 1, this lane's first column)
+    auto xy = [&](float (&M)[2 * R], uint32_t (&Q)[2 * R], uint32_t qz) {
         float m[2 * NR];
         int q[2 * NR];
 #pragma unroll
         for (int j = 0; j < NR; j++) {
             const float a = va[j].x, b = va[j].y;
-            bad |= (a != a) | (b != b);
+            if (j >= 1 && j <= R) bad |= (a != a) | (b != b);  // (the halo rows are other warps')
             float l = __shfl_up_sync(full, b, 1), r = __shfl_down_sync(full, a, 1);
-            if (lane == 0) l = ve[j];
-            if (lane == 31) r = ve[j];
+            if (first_lane) l = ve[j];
+            if (last_lane) r = ve[j];
             const int o = j * kSRow;
             const float pm = fmaxf(a, b);
             const int pq = b > a ? o + 2 : o;
@@ -168,163 +204,226 @@ __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, flo
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 float pm;
-                int pq;
+                int pq, qa, qb;
                 best2<true>(m[2 * (k + 1) + c], q[2 * (k + 1) + c], m[2 * (k + 2) + c], q[2 * (k + 2) + c], false, pm, pq);
-                best2<kInner>(m[2 * k + c], q[2 * k + c], pm, pq, !kInner && y == 0, M[2 * k + c], Q[2 * k + c]);
+                best2<kInner>(m[2 * k + c], q[2 * k + c], pm, pq, !kInner && y == 0, M[2 * k + c], qa);
                 best2<kInner>(pm, pq, m[2 * (k + 3) + c], q[2 * (k + 3) + c], !kInner && y + 1 == N - 1,
-                              M[2 * (k + 1) + c], Q[2 * (k + 1) + c]);
-                Q[2 * k + c] += qz;
-                Q[2 * (k + 1) + c] += qz;
+                              M[2 * (k + 1) + c], qb);
+                Q[2 * k + c] = qz + uint32_t(qa);
+                Q[2 * (k + 1) + c] = qz + uint32_t(qb);
             }
         }
     };
-    const int lane0 = r0 * kSRow + 2 * (lx + 2);  // offset of (plane 0, row r0 - 1, column lx)
+    const uint32_t lane0 = sb + uint32_t(r0 * kSRow + 2 * (lx + 2));  // (plane 0, row r0 - 1, column lx)
     const bool own_x = lx < wx;
-    // stores the pointers of tile plane lz = p - 1 from the choices (m1, q1), (m2, q2) along z
-    auto emit = [&](int p, const float (&m1)[2 * R], const int (&q1)[2 * R], const float (&m2)[2 * R],
-                    const int (&q2)[2 * R], bool tie, bool first) {
-        const int own0 = lane0 + p * kSPlane + kSRow;
+    // the lane's seeds: bit 2 lz + c of its row's mask (listed after the planes: a seed in half of all rows of
+    // 64 made the listing inside the loop a third of its instructions)
+    uint32_t smask[R] = {};
+    uint32_t bit = 1;
+    // stores the pointers of tile plane p - 1 from the choices (m1, q1), (m2, q2) along z
+    auto emit = [&](int p, const float (&m1)[2 * R], const uint32_t (&q1)[2 * R], const float (&m2)[2 * R],
+                    const uint32_t (&q2)[2 * R], bool tie, bool first) {
+        const uint32_t own0 = lane0 + uint32_t(p * kSPlane + kSRow), half = sb + uint32_t(kSPlane);
 #pragma unroll
         for (int k = 0; k < R; k++) {
-            float m[2];
-            int q[2];
+            const uint32_t own = own0 + uint32_t(k * kSRow);
+            const bool in = own_x && r0 + k < wy;
+            uint32_t q[2];
             // (first: the pair's choice may lie in the plane across the boundary, which loses ties)
-            best2<kInner>(m1[2 * k], q1[2 * k], m2[2 * k], q2[2 * k], tie || (first && q1[2 * k] < kSPlane), m[0], q[0]);
-            best2<kInner>(m1[2 * k + 1], q1[2 * k + 1], m2[2 * k + 1], q2[2 * k + 1],
-                          tie || (first && q1[2 * k + 1] < kSPlane), m[1], q[1]);
-            const int own = own0 + k * kSRow;
-            if (own_x && r0 + k < wy) {
 #pragma unroll
-                for (int c = 0; c < 2; c++)
-                    if (q[c] == own + 2 * c) {  // a local maximum
-                        if (m[c] > cwt_min) {
-                            const uint32_t g = uint32_t((z0 + p - 1) * plane + (y0 + r0 + k) * N + x0 + lx + c);
-                            atomicOr(&seed_bits[g >> 5], 1u << (g & 31));
-                            const uint32_t j = atomicAdd(n_seeds, 1u);
-                            if (j < uint32_t(kTileSeedCap)) seeds[j] = uint16_t(q[c]);
-                        } else {
-                            q[c] = kSNone;
-                        }
-                    }
-                pair_at(own) = uint32_t(q[0]) | (uint32_t(q[1]) << 16);
+            for (int c = 0; c < 2; c++) {
+                const int i = 2 * k + c;
+                const bool w = kInner ? m2[i] > m1[i]
+                                      : (m2[i] > m1[i] || ((tie || (first && q1[i] < half)) && m2[i] == m1[i]));
+                const float m = fmaxf(m1[i], m2[i]);
+                q[c] = w ? q2[i] : q1[i];
+                if (q[c] == own + 2 * c) {  // a local maximum
+                    if (!(m > cwt_min)) q[c] = none;
+                    else if (in) smask[k] |= bit << c;
+                }
             }
+            if (in) sts32(own, q[0] | (q[1] << 16));
         }
+        bit <<= 2;
     };
     // along z: the better of the last two planes, and the last plane
     float mP[2 * R], mL[2 * R], mN[2 * R];
-    int qP[2 * R], qL[2 * R], qN[2 * R];
-    fetch(0);
+    uint32_t qP[2 * R], qL[2 * R], qN[2 * R];
+    fetch();
     xy(mP, qP, lane0);
-    fetch(1);
+    fetch();
     xy(mL, qL, lane0 + kSPlane);
-    fetch(2);
+    fetch();
     // planes 0 and 1: the first one wins ties unless it lies across the boundary
 #pragma unroll
-    for (int i = 0; i < 2 * R; i++)
-        best2<kInner>(mP[i], qP[i], mL[i], qL[i], !kInner && z0 == 0, mP[i], qP[i]);
+    for (int i = 0; i < 2 * R; i++) {
+        const bool w = mL[i] > mP[i] || (!kInner && z0 == 0 && mL[i] == mP[i]);
+        mP[i] = fmaxf(mP[i], mL[i]);
+        qP[i] = w ? qL[i] : qP[i];
+    }
 #pragma unroll 1
     for (int p = 1; p <= wz; p++) {
-        xy(mN, qN, lane0 + (p + 1) * kSPlane);
-        if (p < wz) fetch(p + 2);
+        xy(mN, qN, lane0 + uint32_t((p + 1) * kSPlane));
+        if (p < wz) fetch();
         emit(p, mP, qP, mN, qN, !kInner && z0 + p == N, !kInner && z0 == 0 && p == 1);
 #pragma unroll
         for (int i = 0; i < 2 * R; i++) {
-            best2<true>(mL[i], qL[i], mN[i], qN[i], false, mP[i], qP[i]);
+            const bool w = mN[i] > mL[i];
+            mP[i] = fmaxf(mL[i], mN[i]);
+            qP[i] = w ? qN[i] : qL[i];
             mL[i] = mN[i];
             qL[i] = qN[i];
         }
     }
     if (bad) set_status(status, CWTHF_E_BAD_INPUT);
+    const uint32_t mine = lane0 + kSPlane + kSRow;  // (plane lz 0, row r0)
+    {  // list the warp's seeds
+        uint32_t n = 0;
+#pragma unroll
+        for (int k = 0; k < R; k++) n += uint32_t(__popc(smask[k]));
+        uint32_t incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(full, incl, o);
+            if (lane >= o) incl += y;
+        }
+        uint32_t j = 0;
+        if (last_lane && incl) j = atomicAdd(n_seeds, incl);
+        j = __shfl_sync(full, j, 31) + incl - n;
+#pragma unroll
+        for (int k = 0; k < R; k++)
+            for (uint32_t m = smask[k]; m; m &= m - 1, j++) {
+                const int i = __ffs(m) - 1;
+                if (j < uint32_t(kTileSeedCap))
+                    sts16(seeds + 2 * j, mine + uint32_t(k * kSRow + (i >> 1) * kSPlane + 2 * (i & 1)));
+            }
+    }
     __syncthreads();
 
     // ---- chains inside the tile: pointer jumping in place, every cell in
     // lockstep; a pointer takes its target's target's target, until every
     // pointer names a root.  A value read while another thread rewrites it is
-    // the old or the new pointer, both points of the same chain. ----
-    const int mine = lane0 + kSPlane + kSRow;  // (plane lz 0, row r0)
+    // the old or the new pointer, both points of the same chain.  The loads of
+    // kBatch pairs go together. ----
+    constexpr int kBatch = 8;
+    auto ok = [&](uint32_t u) { return index_ok(int64_t(u) - int64_t(sb), kSBytes, status); };
     for (int round = 0; round < kJumpRoundsInTile; round++) {
         bool more = false;
 #pragma unroll 1
-        for (int k = 0; k < R; k++) {
-#pragma unroll 8
-            for (int lz = 0; lz < kChTZ; lz++) {
-                uint32_t& w = pair_at(mine + k * kSRow + lz * kSPlane);
-                const uint32_t u = w, u0 = u & 0xffffu, u1 = u >> 16;
-                if (!index_ok(u0, kSBytes, status) || !index_ok(u1, kSBytes, status)) continue;
-                const uint32_t t0 = at(int(u0)), t1 = at(int(u1));
-                if (t0 != u0 || t1 != u1) {
-                    const uint32_t s0 = at(int(t0)), s1 = at(int(t1));
-                    w = s0 | (s1 << 16);
-                    more |= s0 != t0 || s1 != t1;
+        for (int i0 = 0; i0 < R * kChTZ; i0 += kBatch) {  // plane pairs of row i0 / kChTZ
+            const uint32_t a0 = mine + uint32_t((i0 / kChTZ) * kSRow + (i0 % kChTZ) * kSPlane);
+            uint32_t u[kBatch], t0[kBatch], t1[kBatch];
+#pragma unroll
+            for (int i = 0; i < kBatch; i++) u[i] = lds32(a0 + i * kSPlane);
+#pragma unroll
+            for (int i = 0; i < kBatch; i++) {
+                t0[i] = ok(u[i] & 0xffffu) ? lds16(u[i] & 0xffffu) : u[i] & 0xffffu;
+                t1[i] = ok(u[i] >> 16) ? lds16(u[i] >> 16) : u[i] >> 16;
+            }
+#pragma unroll
+            for (int i = 0; i < kBatch; i++) {
+                const uint32_t tt = t0[i] | (t1[i] << 16);
+                if (tt != u[i]) {
+                    const uint32_t w = lds16(t0[i]) | (lds16(t1[i]) << 16);
+                    sts32(a0 + i * kSPlane, w);
+                    more |= w != tt;
                 }
             }
         }
         if (!__syncthreads_or(more)) break;
     }
-    // each seed's entry now holds its number in the tile (odd: offsets are even)
+    // global index of the cell of the entry at address u (inside the tile or in its halo)
+    const uint32_t bias = sb * kYMul;
+    const int xb = 2 * (x0 - 2) - int(sb);
+    auto cell_at = [&](uint32_t u) -> int32_t {
+        const uint32_t r = (u * kYMul - bias) >> kYShift;
+        const int x = (int(u - r * uint32_t(kSRow)) + xb) >> 1;
+        return int32_t(lds32(line + 4 * r)) + (kInner ? x : wrap(x, N));
+    };
+    // each seed's entry now holds the address of its counter (odd: addresses of entries are even), seeds
+    // beyond the counters share one that is not read
     const uint32_t ns = min(*n_seeds, uint32_t(kTileSeedCap));
     if (threadIdx.x == 0 && *n_seeds > uint32_t(kTileSeedCap)) set_status(status, CWTHF_E_BAD_INPUT);
-    for (uint32_t j = threadIdx.x; j < ns; j += kSegThreads) at(seeds[j]) = uint16_t(2 * j + 1);
-    for (uint32_t j = threadIdx.x; j < (ns + 1) / 2; j += kSegThreads) cnt[j] = 0u;
+    auto mark = [&](uint32_t j0) {  // counters of seeds j0 .. j0 + kCountSeeds - 1
+        for (uint32_t j = threadIdx.x; j < ns; j += kSegThreads)
+            sts16(lds16(seeds + 2 * j), cnt + 4 * min(j - j0, uint32_t(kCountSeeds)) + 1);
+        for (uint32_t j = threadIdx.x; j <= uint32_t(kCountSeeds); j += kSegThreads) sts32(cnt + 4 * j, 0u);
+        if (threadIdx.x == 0) sts16(none, cnt + 4 * kCountSeeds + 1);
+    };
+    for (uint32_t j = threadIdx.x; j < ns; j += kSegThreads) {
+        const uint32_t g = uint32_t(cell_at(lds16(seeds + 2 * j)));
+        atomicOr(&seed_bits[g >> 5], 1u << (g & 31));
+    }
+    mark(0);
     __syncthreads();
 
     // ---- labels, and one count per cell for the tile's seeds ----
-    // global index of the cell at offset o (inside the tile or in its halo)
-    auto cell_at = [&](uint32_t o) -> int32_t {
-        const uint32_t r = (o * kYMul) >> kYShift;
-        const int x = x0 - 2 + int((o - r * uint32_t(kSRow)) >> 1);
-        return line[r] + (kInner ? x : wrap(x, N));
-    };
-    auto finish = [&](uint32_t u, int own, bool& fl) -> int32_t {
-        if (!index_ok(u, 65536, status)) return -1;
-        uint32_t e = u;
-        if (u & 1u) u = uint32_t(own);  // a seed's own entry
-        else e = at(int(u));
-        if (u == uint32_t(kSNone)) return -1;
+    auto finish = [&](uint32_t u, uint32_t own, uint32_t& flags, uint32_t fbit) -> int32_t {
+        u = (u & 1u) ? own : u;  // a seed's own entry
+        const uint32_t e = ok(u) ? lds16(u) : u;
         const int32_t g = cell_at(u);
         if (e & 1u) {
-            const uint32_t j = e >> 1;
-            atomicAdd(&cnt[j >> 1], 1u << (16 * (j & 1u)));
+            reds32(e - 1, 1u);
             return g;
         }
-        fl = true;  // outside the tile (or not finished within the round bound)
+        flags |= fbit;  // outside the tile (or not finished within the round bound)
         return -2 - g;
     };
     const bool lvec = (reinterpret_cast<uintptr_t>(label) & 7u) == 0;  // even cells: 8-byte label pairs
 #pragma unroll 1
     for (int k = 0; k < R; k++) {
-        if (r0 + k >= kChTY) break;
         const bool own = own_x && r0 + k < wy;
         int32_t* out = label + (size_t(z0) * N + (y0 + r0 + k)) * N + x0 + lx;
-        uint32_t word = 0;
+        uint32_t flags = 0;  // bit 2 lz + p: this lane's cell of plane lz, column parity p is flagged
+        if (own) {
+            uint32_t o = mine + uint32_t(k * kSRow), fbit = 1;
 #pragma unroll 4
-        for (int lz = 0; lz < kChTZ; lz++) {
-            bool f0 = false, f1 = false;
-            if (own && lz < wz) {
-                const int o = mine + k * kSRow + lz * kSPlane;
-                const uint32_t u = pair_at(o);
+            for (int lz = 0; lz < wz; lz++, out += plane, o += kSPlane, fbit <<= 2) {
+                const uint32_t u = lds32(o);
                 int2 res;
-                res.x = finish(u & 0xffffu, o, f0);
-                res.y = finish(u >> 16, o + 2, f1);
-                int32_t* dst = out + size_t(lz) * size_t(plane);
+                res.x = finish(u & 0xffffu, o, flags, fbit);
+                res.y = finish(u >> 16, o + 2, flags, fbit << 1);
                 if (lvec) {
-                    *reinterpret_cast<int2*>(dst) = res;
+                    *reinterpret_cast<int2*>(out) = res;
                 } else {
-                    dst[0] = res.x;
-                    dst[1] = res.y;
+                    out[0] = res.x;
+                    out[1] = res.y;
                 }
             }
-            const unsigned b0 = __ballot_sync(full, f0), b1 = __ballot_sync(full, f1);
-            if (lane == 2 * lz) word = b0;      // plane lz, even columns
-            if (lane == 2 * lz + 1) word = b1;  // odd columns
         }
-        ballots[(size_t(t) * kChTY + r0 + k) * kRowWords + lane] = word;
+        __syncwarp();
+        // transposed over the warp: word w (lane w) gets bit w of every lane
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const uint32_t low = d == 16 ? 0x0000ffffu : (d == 8 ? 0x00ff00ffu : (d == 4 ? 0x0f0f0f0fu : (d == 2 ? 0x33333333u : 0x55555555u)));
+            const uint32_t other = __shfl_xor_sync(full, flags, d);
+            flags = (lane & d) ? ((flags & ~low) | ((other & ~low) >> d)) : ((flags & low) | ((other & low) << d));
+        }
+        ballots[(size_t(t) * kChTY + r0 + k) * kRowWords + lane] = flags;
     }
     __syncthreads();
     // in-tile cell counts of this tile's seeds (cells reaching them from other
     // tiles are added by the global pass)
-    for (uint32_t j = threadIdx.x; j < ns; j += kSegThreads)
-        seed_cells[size_t(cell_at(seeds[j]))] = (cnt[j >> 1] >> (16 * (j & 1u))) & 0xffffu;
+    for (uint32_t j0 = 0;;) {  // one turn but for tiles of more than kCountSeeds seeds
+        for (uint32_t j = j0 + threadIdx.x; j < min(ns, j0 + uint32_t(kCountSeeds)); j += kSegThreads)
+            seed_cells[size_t(cell_at(lds16(seeds + 2 * j)))] = lds32(cnt + 4 * (j - j0));
+        j0 += uint32_t(kCountSeeds);
+        if (j0 >= ns) break;  // block-uniform
+        __syncthreads();
+        mark(j0);
+        __syncthreads();
+        for (int k = 0; k < R; k++)
+            if (own_x && r0 + k < wy)
+                for (int lz = 0; lz < wz; lz++) {
+                    const uint32_t o = mine + uint32_t(k * kSRow + lz * kSPlane), w = lds32(o);
+                    for (int c = 0; c < 2; c++) {
+                        const uint32_t u = c ? w >> 16 : w & 0xffffu;
+                        const uint32_t e = (u & 1u) ? u : (ok(u) ? lds16(u) : u);
+                        if (e & 1u) reds32(e - 1, 1u);
+                    }
+                }
+        __syncthreads();
+    }
 }
 
 __global__ void __launch_bounds__(kSegThreads, 4) k_seg_tile(const float* __restrict__ C, int ng, float cwt_min,
@@ -335,35 +434,38 @@ __global__ void __launch_bounds__(kSegThreads, 4) k_seg_tile(const float* __rest
     extern __shared__ __align__(16) unsigned char seg_smem[];
     __shared__ uint32_t n_seeds;
     if (threadIdx.x == 0) n_seeds = 0;  // (the tile's first barrier is before its first use)
+    const uint32_t sb = uint32_t(__cvta_generic_to_shared(seg_smem));
+    if (sb + uint32_t(kSegSmem) > 65535u) {  // pointers would not fit 16 bits: cannot happen (see above)
+        set_status(status, CWTHF_E_CUDA);
+        return;
+    }
     const int ntx = (ng + kChTX - 1) / kChTX, nty = (ng + kChTY - 1) / kChTY;
     const int t = int(blockIdx.x), tx = t % ntx, ty = (t / ntx) % nty, tz = t / (ntx * nty);
     const bool inner = tx > 0 && (tx + 1) * kChTX < ng && ty > 0 && (ty + 1) * kChTY < ng && tz > 0 &&
                        (tz + 1) * kChTZ < ng;
-    if (inner) seg_tile<true>(C, ng, cwt_min, label, seed_bits, seed_cells, ballots, status, seg_smem, &n_seeds);
-    else seg_tile<false>(C, ng, cwt_min, label, seed_bits, seed_cells, ballots, status, seg_smem, &n_seeds);
+    if (inner) seg_tile<true>(C, ng, cwt_min, label, seed_bits, seed_cells, ballots, status, sb, &n_seeds);
+    else seg_tile<false>(C, ng, cwt_min, label, seed_bits, seed_cells, ballots, status, sb, &n_seeds);
 }
 
 constexpr int kResolveThreads = 256;
-constexpr int kResTabBits = 9, kResTab = 1 << kResTabBits;  // per-tile count table (shared memory)
+constexpr int kResTabBits = 10, kResTab = 1 << kResTabBits;  // per-tile count table (shared memory)
 
-// The global pass over the cells whose chain left their tile.  A CTA takes one
-// chain tile (or `rows` of its rows) at a time from a global counter, and its
-// warps take the
-// rows one at a time from a shared counter (the flagged cells crowd where the
-// field is clumped, so a fixed split leaves some warps far more work than
+// The global pass over the cells whose chain left their tile.  A CTA takes
+// `rows` rows of chain tiles at a time from a global counter, and its warps
+// take them one at a time from a shared counter (the flagged cells crowd where
+// the field is clumped, so a fixed split leaves some warps far more work than
 // others).  A warp gathers the flagged cells of a row's non-empty plane masks
 // into a shared batch; every full batch of 32 cells (and the warp's last,
-// partial one of the tile) is resolved by the whole warp: each lane follows
-// its cell's chain through the label grid (at most `limit` steps, kDefaultChaseLimit
-// by default) and takes the label it reaches.  The tile's cells are counted
-// per seed in a shared table (one entry per distinct seed, one shared atomic
-// per distinct seed of a batch) that is added to the counts kept at the seeds'
-// cells once per tile (the tile pass wrote each seed's in-tile count there;
-// seed slots are ranked only afterwards).  A cell still unfinished at the
-// limit stays flagged and sets changed[0]; the doubling rounds then finish it
-// and the cells are recounted.  Labels read while other threads update them
-// are always a later point of the same chain, so the result does not depend
-// on timing.
+// partial one) is resolved by the whole warp: each lane follows its cell's
+// chain through the label grid (at most `limit` steps, kDefaultChaseLimit by
+// default) and takes the label it reaches.  The cells are counted per seed in a
+// shared table (one entry per distinct seed, one shared atomic per distinct
+// seed of a batch) that is added to the counts kept at the seeds' cells once
+// per turn (the tile pass wrote each seed's in-tile count there; seed slots are
+// ranked only afterwards).  A cell still unfinished at the limit stays flagged
+// and sets changed[0]; the doubling rounds then finish it and the cells are
+// recounted.  Labels read while other threads update them are always a later
+// point of the same chain, so the result does not depend on timing.
 __device__ __forceinline__ void table_add(int32_t* tkey, uint32_t* tcnt, uint32_t* __restrict__ seed_cells,
                                           int32_t lab, uint32_t n) {
     uint32_t h = (uint32_t(lab) * 2654435761u) >> (32 - kResTabBits);
@@ -413,19 +515,19 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
                                                                  const uint32_t* __restrict__ ballots,
                                                                  uint32_t* __restrict__ seed_cells,
                                                                  int* __restrict__ changed,
-                                                                 unsigned* __restrict__ next_tile, int limit,
+                                                                 unsigned* __restrict__ next_rows, int limit,
                                                                  int rows, int* status) {
     __shared__ uint32_t batch[kResolveThreads / 32][64];  // pending cells (fewer than 32 between batches)
     __shared__ int32_t tkey[kResTab];
     __shared__ uint32_t tcnt[kResTab];
-    __shared__ unsigned s_tile, s_row;
+    __shared__ unsigned s_end, s_row;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     uint32_t* wl = batch[threadIdx.x >> 5];
     const int N = ng;
     const int ntx = (N + kChTX - 1) / kChTX, nty = (N + kChTY - 1) / kChTY, ntz = (N + kChTZ - 1) / kChTZ;
-    const unsigned per_tile = unsigned(kChTY / rows), nunits = unsigned(ntx) * unsigned(nty) * unsigned(ntz) * per_tile;
+    const unsigned nrows = unsigned(ntx) * unsigned(nty) * unsigned(ntz) * unsigned(kChTY);  // rows of all tiles
     const uint32_t plane32 = uint32_t(N) * uint32_t(N);
     const int64_t cells = int64_t(plane32) * N;
     for (int i = threadIdx.x; i < kResTab; i += blockDim.x) {
@@ -435,24 +537,25 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
     bool left = false;
     for (;;) {
         if (threadIdx.x == 0) {
-            s_tile = atomicAdd(next_tile, 1u);
-            s_row = (s_tile % per_tile) * unsigned(rows);
+            const unsigned r = atomicAdd(next_rows, 1u) * unsigned(rows);  // (far below 2^32: CTAs stop at nrows)
+            s_row = r;
+            s_end = r < nrows ? min(nrows, r + unsigned(rows)) : 0u;
         }
         __syncthreads();
-        if (s_tile >= nunits) break;  // block-uniform
-        const unsigned t = s_tile / per_tile, row_end = (s_tile % per_tile + 1) * unsigned(rows);
-        const int tx = int(t % unsigned(ntx)), ty = int((t / unsigned(ntx)) % unsigned(nty)),
-                  tz = int(t / (unsigned(ntx) * unsigned(nty)));
+        const unsigned row_end = s_end;
+        if (row_end == 0u) break;  // block-uniform
         uint32_t k = 0;  // warp-uniform
         for (;;) {
-            unsigned ly = 0;
-            if (lane == 0) ly = atomicAdd(&s_row, 1u);
-            ly = __shfl_sync(full, ly, 0);
-            if (ly >= row_end) break;  // warp-uniform
+            unsigned rw = 0;
+            if (lane == 0) rw = atomicAdd(&s_row, 1u);
+            rw = __shfl_sync(full, rw, 0);
+            if (rw >= row_end) break;  // warp-uniform
+            const unsigned t = rw / unsigned(kChTY), ly = rw % unsigned(kChTY);
+            const int tx = int(t % unsigned(ntx)), ty = int((t / unsigned(ntx)) % unsigned(nty)),
+                      tz = int(t / (unsigned(ntx) * unsigned(nty)));
             const int yc = ty * kChTY + int(ly);
             if (yc >= N) continue;  // warp-uniform
-            const int64_t rw = int64_t(t) * kChTY + ly;
-            const uint32_t mine = ballots[rw * kRowWords + lane];  // plane lane / 2, columns of parity lane % 2
+            const uint32_t mine = ballots[size_t(rw) * kRowWords + lane];  // plane lane / 2, columns of parity lane % 2
             uint32_t words = __ballot_sync(full, mine != 0u);
             const uint32_t cell0 =
                 uint32_t((int64_t(tz) * kChTZ * N + yc) * N + int64_t(tx) * kChTX) + 2u * uint32_t(lane);
@@ -478,7 +581,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
             resolve_batch(label, uint32_t(lane) < k, uint32_t(lane) < k ? wl[lane] : 0u, tkey, tcnt, seed_cells,
                           limit, left, cells, status);
         __syncthreads();
-        // the tile's counts go to the seeds' cells; the table is cleared for the next tile
+        // the rows' counts go to the seeds' cells; the table is cleared for the next ones
         for (int i = threadIdx.x; i < kResTab; i += blockDim.x) {
             const int32_t key = tkey[i];
             if (key >= 0) {
@@ -677,9 +780,10 @@ int segment_impl(cwthf_ctx* ctx, const float* cwt, int ng, float cwt_min, int32_
     // chains that left their tile, counted at their seed's cell
     int blocks = ctx->sm_count * 8;
     int* changed = ctx->jump_changed;  // see kJumpWords
-    // a CTA takes a whole tile (one table flush), or, where tiles are too few to fill the GPU, two of its
-    // rows (64^3: 38 us with 16 whole tiles, 27 us)
-    const int rows = ntiles < 2 * ctx->sm_count ? 2 : kChTY;
+    // rows per turn: four tiles' where there are many turns per CTA (the barriers around a turn's table flush
+    // were the pass's largest stall with one tile: 2.14 ms per scale at 1024^3, 1.93 with four), two rows where tiles are too few to fill the
+    // GPU (64^3: 38 us with 16 whole tiles, 27 us)
+    const int rows = ntiles < 2 * ctx->sm_count ? 2 : (ntiles < 16 * blocks ? kChTY : 4 * kChTY);
     CWTHF_LAUNCH(ctx, s, "k_seg_resolve",
                  k_seg_resolve<<<blocks, kResolveThreads, 0, s>>>(label, ng, ballots, ctx->seed_cells, changed,
                                                                    reinterpret_cast<unsigned*>(changed + kJumpTileCounter),
