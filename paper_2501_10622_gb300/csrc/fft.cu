@@ -457,6 +457,7 @@ int x_args(cwthf_ctx* ctx, int ng, const Tables* t, XArgs& a, const CtEntry*& ct
     a.M = ng / 2;
     a.P = spec_pitch(ng);
     a.rows = int64_t(ng) * ng;
+    a.inv_ng = ~0ull / unsigned(ng);
     a.twM = p.Lb ? t->tw_x : t->twM;
     a.twN = t->twN;
     return CWTHF_OK;

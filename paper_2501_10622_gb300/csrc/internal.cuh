@@ -325,6 +325,18 @@ __device__ __forceinline__ int table_find(uint32_t* tkey, uint32_t* tused, uint3
     return -1;
 }
 
+// The float nearest to a 64-bit integer (half to even, as __ll2float_rn).
+// 64-bit conversions run at a small fraction of the arithmetic rate; below 2^45
+// in magnitude the integer is a 2^23 + b with both parts exact in a float, built
+// by adding to a constant's mantissa, and one fused multiply-add rounds once.
+__device__ __forceinline__ float ll2float(long long x) {
+    const int a = int(x >> 23);
+    if (x < -(1ll << 45) || x >= (1ll << 45)) return __ll2float_rn(x);
+    const float hi = __int_as_float(0x4b400000 + a) - 12582912.0f;                            // |a| <= 2^22
+    const float lo = __int_as_float(0x4b000000 | (int(x) & 0x7fffff)) - 8388608.0f;          // b < 2^23
+    return fmaf(hi, 8388608.0f, lo);
+}
+
 // ---- warp helpers -------------------------------------------------------------
 // Lane of the n-th (0-based) member of the lane set `group`, or 32 if the
 // group has no more than n members.

@@ -58,11 +58,11 @@ __global__ void __launch_bounds__(32 * kXWarps) k_sten_x_reg(const int64_t* __re
     if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {  // ng is even
         for (int x = 2 * lane; x < ng; x += 64) {
             const longlong2 v = *reinterpret_cast<const longlong2*>(src + x);
-            buf[RC + x] = __ll2float_rn(v.x) * kUnit;
-            buf[RC + x + 1] = __ll2float_rn(v.y) * kUnit;
+            buf[RC + x] = ll2float(v.x) * kUnit;
+            buf[RC + x + 1] = ll2float(v.y) * kUnit;
         }
     } else {
-        for (int x = lane; x < ng; x += 32) buf[RC + x] = __ll2float_rn(src[x]) * kUnit;
+        for (int x = lane; x < ng; x += 32) buf[RC + x] = ll2float(src[x]) * kUnit;
     }
     __syncwarp();
     if (lane < RC) {  // RC <= ng: the radius class is at most R + 3, and ng >= 2 R + 1, ng >= 8
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(32 * kXWarps) k_sten_x(const int64_t* __restri
     for (int j = lane; j < W; j += 32) {
         int x = j - R;
         x = x < 0 ? x + ng : (x >= ng ? x - ng : x);
-        buf[j] = __ll2float_rn(src[x]) * kUnit;
+        buf[j] = ll2float(src[x]) * kUnit;
     }
     __syncwarp();
     float* a = A + row * ng;
