@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(kThreads) k_count_cells(const int32_t* __restr
                                                          const uint32_t* __restrict__ prefix,
                                                          const uint32_t* __restrict__ n_slots, HaloAcc* acc,
                                                          int* status) {
+    pdl_wait();
     __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab];
     __shared__ uint32_t n_used;
     const int lane = threadIdx.x & 31;
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_su
                                                        const uint32_t* __restrict__ n_slots, HaloAcc* acc,
                                                        int32_t* __restrict__ rec_slot, int slot_stride,
                                                        u64* __restrict__ mtot, int skip_marked, int* status) {
+    pdl_wait();
     constexpr int kW = kMass ? kTab : 1;  // the 64-bit words exist with masses only
     __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab];
     __shared__ uint32_t tm_lo[3][kTab];  // moments (equal masses: the whole 32-bit sum)
@@ -325,13 +327,13 @@ void launch_halo_sums(cwthf_ctx* ctx, cudaStream_t s, int64_t np, const DepArgs&
     const int64_t chunks = div_up(std::max<int64_t>(np, 1), kChunk);
     if (a.mass)
         CWTHF_LAUNCH(ctx, s, "k_halo_sums",
-                     k_halo_sums<true><<<int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * hs_ctas_per_sm<true>())),
-                                         kHsThreads, 0, s>>>(a, dn, total, rec, rec_mq, label, bits, prefix, n_slots,
+                     pdl(k_halo_sums<true>, int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * hs_ctas_per_sm<true>())),
+                                         kHsThreads, 0, s)(a, dn, total, rec, rec_mq, label, bits, prefix, n_slots,
                                                              acc, rec_slot, slot_stride, mtot, skip_marked, st));
     else
         CWTHF_LAUNCH(ctx, s, "k_halo_sums",
-                     k_halo_sums<false><<<int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * hs_ctas_per_sm<false>())),
-                                          kHsThreads, 0, s>>>(a, dn, total, rec, rec_mq, label, bits, prefix, n_slots,
+                     pdl(k_halo_sums<false>, int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * hs_ctas_per_sm<false>())),
+                                          kHsThreads, 0, s)(a, dn, total, rec, rec_mq, label, bits, prefix, n_slots,
                                                               acc, rec_slot, slot_stride, mtot, skip_marked, st));
 }
 
@@ -346,6 +348,7 @@ struct FilterArgs {
 __global__ void __launch_bounds__(kThreads) k_keep(const HaloAcc* __restrict__ acc, const uint32_t* __restrict__ n_seeds,
                                                   const u64* __restrict__ mtot, FilterArgs f,
                                                   uint32_t* __restrict__ keep) {
+    pdl_wait();
     uint32_t ns = *n_seeds;
     double ncube = double(int64_t(f.ng) * f.ng * f.ng);
     double rhs0 = __dmul_rn(f.dens_th, double(*mtot));
@@ -370,6 +373,7 @@ __global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* __restric
                                                        FilterArgs f, cwthf_halo* __restrict__ cat,
                                                        int32_t* __restrict__ slot_halo,
                                                        int64_t* __restrict__ n_halo, int* status) {
+    pdl_wait();
     __shared__ uint32_t queue[kThreads / 32][64];
     uint32_t* q = queue[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -465,6 +469,7 @@ __global__ void __launch_bounds__(kThreads) k_rec_halo(const int32_t* rec_slot, 
                                                       const uint32_t* __restrict__ total_ptr, int n_scales,
                                                       const int32_t* __restrict__ slot_halo, int64_t slot_stride,
                                                       typename IdGroup<RS>::T* groups) {
+    pdl_wait();
     constexpr int G = RS < 4 ? RS : 4;  // ids per stored group
     const int64_t total = *total_ptr;
     const int ngr = (n_scales + G - 1) / G;
@@ -491,6 +496,7 @@ __global__ void __launch_bounds__(kThreads) k_finalize(const uint32_t* __restric
                                                       const uint32_t* __restrict__ total_ptr,
                                                       const typename IdGroup<RS>::T* __restrict__ groups,
                                                       int n_scales, int32_t* __restrict__ halo_id) {
+    pdl_wait();
     constexpr int kIlp = 8;
     constexpr int G = RS < 4 ? RS : 4;
     using T = typename IdGroup<RS>::T;
@@ -530,6 +536,7 @@ __global__ void __launch_bounds__(kThreads) k_finalize_one(const uint32_t* __res
                                                           const int32_t* __restrict__ rec_slot,
                                                           const int32_t* __restrict__ slot_halo,
                                                           int32_t* __restrict__ halo_id) {
+    pdl_wait();
     constexpr int kIlp = 8;
     const int64_t total = *total_ptr;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -557,10 +564,10 @@ void launch_ids(cwthf_ctx* ctx, cudaStream_t s, int blocks, int pblocks, int64_t
     using T = typename IdGroup<RS>::T;
     T* groups = reinterpret_cast<T*>(ctx->part_slot + slot_groups_offset(n_scales, np));
     CWTHF_LAUNCH(ctx, s, "k_rec_halo",
-                 k_rec_halo<RS><<<blocks, kThreads, 0, s>>>(ctx->part_slot, np, total, n_scales, ctx->slot_halo,
+                 pdl(k_rec_halo<RS>, blocks, kThreads, 0, s)(ctx->part_slot, np, total, n_scales, ctx->slot_halo,
                                                             slot_cap, groups));
     CWTHF_LAUNCH(ctx, s, "k_finalize",
-                 k_finalize<RS><<<pblocks, kThreads, 0, s>>>(ctx->part_rec, np, total, groups, n_scales, halo_id));
+                 pdl(k_finalize<RS>, pblocks, kThreads, 0, s)(ctx->part_rec, np, total, groups, n_scales, halo_id));
 }
 
 // ---- the multi-scale loop (Sec. 2, Fig. 1; App. B; Sec. 2.4) -----------------
@@ -572,6 +579,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_mark(const int32_t* __restrict_
                                                      const uint32_t* __restrict__ part_rec, int64_t np,
                                                      const uint32_t* __restrict__ total_ptr,
                                                      unsigned long long* __restrict__ rec) {
+    pdl_wait();
     const int64_t total = *total_ptr;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
@@ -585,6 +593,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_mark(const int32_t* __restrict_
 __global__ void __launch_bounds__(kThreads) k_ms_pslot(const uint32_t* __restrict__ part_rec, int64_t np,
                                                       const uint32_t* __restrict__ total_ptr,
                                                       const int32_t* __restrict__ rec_slot, int32_t* __restrict__ pslot) {
+    pdl_wait();
     const int64_t total = *total_ptr;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
@@ -660,6 +669,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_keep(const HaloAcc* __restrict_
                                                      const u64* __restrict__ mtot, FilterArgs f,
                                                      const float* __restrict__ C, const float* __restrict__ Cn,
                                                      int ngn, uint32_t* __restrict__ keep) {
+    pdl_wait();
     const uint32_t ns = *n_seeds;
     const double ncube = double(int64_t(f.ng) * f.ng * f.ng);
     const double rhs0 = __dmul_rn(f.dens_th, double(*mtot));
@@ -684,6 +694,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_catalogue(const HaloAcc* __rest
                                                           int ngn, int scale, const int64_t* __restrict__ n_halo,
                                                           cwthf_ms_halo* __restrict__ cat,
                                                           int32_t* __restrict__ slot_halo) {
+    pdl_wait();
     const uint32_t ns = *n_seeds;
     const int64_t base = *n_halo;
     const int64_t N = f.ng;
@@ -721,6 +732,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_catalogue(const HaloAcc* __rest
 // The number of kept groups (keep_off[n_seeds]) as the check's group count.
 __global__ void k_ms_ub_count(const uint32_t* __restrict__ keep_off, const uint32_t* __restrict__ n_seeds,
                               uint32_t* __restrict__ n_groups) {
+    pdl_wait();
     *n_groups = keep_off[*n_seeds];
 }
 
@@ -731,6 +743,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_group(const int32_t* __restr
                                                          const int32_t* __restrict__ halo_id, int64_t np,
                                                          const uint32_t* __restrict__ keep_off,
                                                          int32_t* __restrict__ grp) {
+    pdl_wait();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
         const int32_t sl = pslot[i];
@@ -750,6 +763,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_keep(const uint32_t* __restr
                                                         const uint32_t* __restrict__ keep_off,
                                                         const int64_t* __restrict__ n_kept, HaloAcc* acc,
                                                         uint32_t* __restrict__ keep2) {
+    pdl_wait();
     const uint32_t ns = *n_seeds;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < ns; s += stride) {
@@ -774,6 +788,7 @@ constexpr int kUbSumItems = 8;
 __global__ void __launch_bounds__(kThreads) k_ms_ub_sums(DepArgs a, const int32_t* __restrict__ pslot,
                                                         const int32_t* __restrict__ bound,
                                                         const int32_t* __restrict__ seed_list, HaloAcc* acc) {
+    pdl_wait();
     __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab], t_lo[4][kTab], t_hi[4][kTab];  // mass, moments
     __shared__ uint32_t n_used;
     const int N = a.ng;
@@ -841,6 +856,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_sums(DepArgs a, const int32_
 __global__ void __launch_bounds__(kThreads) k_ms_ids(const int32_t* __restrict__ pslot, int64_t np,
                                                     const int32_t* __restrict__ slot_halo,
                                                     const int32_t* __restrict__ bound, int32_t* __restrict__ halo_id) {
+    pdl_wait();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
         const int32_t sl = pslot[i];
@@ -855,6 +871,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_ids(const int32_t* __restrict__
 // than cat_cap is reported as CWTHF_E_CAPACITY (the count is still exact).
 __global__ void k_ms_advance(const uint32_t* __restrict__ keep_off, const uint32_t* __restrict__ n_seeds,
                              int64_t* __restrict__ n_halo, int64_t cat_cap, int* status) {
+    pdl_wait();
     const int64_t n = *n_halo + int64_t(keep_off[*n_seeds]);
     *n_halo = n;
     if (n > cat_cap) set_status(status, CWTHF_E_CAPACITY);
@@ -867,12 +884,12 @@ int ms_scale_sums(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     const int64_t total_key = deposit_geom(ng).ntiles * kDepClasses;
     const uint32_t* total = ctx->dep_off + total_key;
     const int pblocks = int(std::min<int64_t>(div_up(std::max<int64_t>(np, 1), kThreads), int64_t(ctx->sm_count) * 16));
-    CWTHF_LAUNCH(ctx, s, "k_ms_mark", k_ms_mark<<<pblocks, kThreads, 0, s>>>(halo_id, ctx->part_rec, np, total, ctx->dep_rec));
+    CWTHF_LAUNCH(ctx, s, "k_ms_mark", pdl(k_ms_mark, pblocks, kThreads, 0, s)(halo_id, ctx->part_rec, np, total, ctx->dep_rec));
     DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
     int32_t* rec_slot = ctx->part_slot;
     launch_halo_sums(ctx, s, np, a, total, ctx->dep_rec, ctx->dep_mq, ctx->label, ctx->seed_bits,
                      ctx->seed_prefix, ctx->n_seeds, ctx->acc, rec_slot, 1, ctx->d_mtot, 1);
-    CWTHF_LAUNCH(ctx, s, "k_ms_pslot", k_ms_pslot<<<pblocks, kThreads, 0, s>>>(ctx->part_rec, np, total, rec_slot, pslot));
+    CWTHF_LAUNCH(ctx, s, "k_ms_pslot", pdl(k_ms_pslot, pblocks, kThreads, 0, s)(ctx->part_rec, np, total, rec_slot, pslot));
     return cuda_status(cudaGetLastError());
 }
 
@@ -890,7 +907,7 @@ int ms_finalize(cwthf_ctx* ctx, const float* pos, const float* mass, const float
     f.dens_th = dens_th;
     f.particle_th = particle_th;
     f.cat_cap = cat_cap;
-    CWTHF_LAUNCH(ctx, s, "k_ms_keep", k_ms_keep<<<blocks, kThreads, 0, s>>>(ctx->acc, ctx->seed_list, ctx->n_seeds, mtot, f,
+    CWTHF_LAUNCH(ctx, s, "k_ms_keep", pdl(k_ms_keep, blocks, kThreads, 0, s)(ctx->acc, ctx->seed_list, ctx->n_seeds, mtot, f,
                                                                            C, Cn, ngn, ctx->keep_off));
     int rc = scan_u32_dev(ctx, ctx->keep_off, ctx->keep_off, ctx->n_seeds, slot_cap, s);
     if (rc) return rc;
@@ -899,27 +916,27 @@ int ms_finalize(cwthf_ctx* ctx, const float* pos, const float* mass, const float
     if (vel) {
         // step 9: the self-boundness check of the kept groups' candidates
         CWTHF_LAUNCH(ctx, s, "k_ms_ub_group",
-                     k_ms_ub_group<<<pblocks, kThreads, 0, s>>>(pslot, halo_id, np, ctx->keep_off, ctx->ub_grp));
+                     pdl(k_ms_ub_group, pblocks, kThreads, 0, s)(pslot, halo_id, np, ctx->keep_off, ctx->ub_grp));
         CWTHF_LAUNCH(ctx, s, "k_ms_ub_count",
-                     k_ms_ub_count<<<1, 1, 0, s>>>(ctx->keep_off, ctx->n_seeds, ctx->ub_ngroups));
+                     pdl(k_ms_ub_count, 1, 1, 0, s)(ctx->keep_off, ctx->n_seeds, ctx->ub_ngroups));
         if ((rc = unbind_groups(ctx, pos, vel, mass, mass_unit, np, L, G, ctx->ub_grp, slot_cap, ctx->ub_ngroups,
                                 max_iter, ctx->ub_out, ctx->ub_nk, ctx->ub_it, s)))
             return rc;
         CWTHF_LAUNCH(ctx, s, "k_ms_ub_keep",
-                     k_ms_ub_keep<<<blocks, kThreads, 0, s>>>(ctx->n_seeds, ctx->keep_off, ctx->ub_nk, ctx->acc,
+                     pdl(k_ms_ub_keep, blocks, kThreads, 0, s)(ctx->n_seeds, ctx->keep_off, ctx->ub_nk, ctx->acc,
                                                               ctx->ub_keep));
         if ((rc = scan_u32_dev(ctx, ctx->ub_keep, ctx->ub_keep, ctx->n_seeds, slot_cap, s))) return rc;
         const DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
         CWTHF_LAUNCH(ctx, s, "k_ms_ub_sums",
-                     k_ms_ub_sums<<<pblocks, kThreads, 0, s>>>(a, pslot, ctx->ub_out, ctx->seed_list, ctx->acc));
+                     pdl(k_ms_ub_sums, pblocks, kThreads, 0, s)(a, pslot, ctx->ub_out, ctx->seed_list, ctx->acc));
         keep = ctx->ub_keep;
         bound = ctx->ub_out;
     }
     CWTHF_LAUNCH(ctx, s, "k_ms_catalogue",
-                 k_ms_catalogue<<<blocks, kThreads, 0, s>>>(ctx->acc, ctx->seed_list, ctx->n_seeds, keep, f, C,
+                 pdl(k_ms_catalogue, blocks, kThreads, 0, s)(ctx->acc, ctx->seed_list, ctx->n_seeds, keep, f, C,
                                                             Cn, ngn, scale, n_halo, cat, ctx->slot_halo));
-    CWTHF_LAUNCH(ctx, s, "k_ms_ids", k_ms_ids<<<pblocks, kThreads, 0, s>>>(pslot, np, ctx->slot_halo, bound, halo_id));
-    CWTHF_LAUNCH(ctx, s, "k_ms_advance", k_ms_advance<<<1, 1, 0, s>>>(keep, ctx->n_seeds, n_halo, cat_cap,
+    CWTHF_LAUNCH(ctx, s, "k_ms_ids", pdl(k_ms_ids, pblocks, kThreads, 0, s)(pslot, np, ctx->slot_halo, bound, halo_id));
+    CWTHF_LAUNCH(ctx, s, "k_ms_advance", pdl(k_ms_advance, 1, 1, 0, s)(keep, ctx->n_seeds, n_halo, cat_cap,
                                                                      ctx->d_status));
     return cuda_status(cudaGetLastError());
 }
@@ -939,7 +956,7 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     if (e != cudaSuccess) return cuda_status(e);
     if (!seeds_ready)  // after segment_impl the resolve pass has counted the cells already
         CWTHF_LAUNCH(ctx, s, "k_count_cells",
-                     k_count_cells<<<int(std::min<int64_t>(div_up(cells, kCountCells), blocks)), kThreads, 0, s>>>(label, cells, ctx->seed_bits, ctx->seed_prefix,
+                     pdl(k_count_cells, int(std::min<int64_t>(div_up(cells, kCountCells), blocks)), kThreads, 0, s)(label, cells, ctx->seed_bits, ctx->seed_prefix,
                                                                d_nseeds, ctx->acc, ctx->d_status));
     DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
     const int64_t total_key = deposit_geom(ng).ntiles * kDepClasses;  // dep_off[total_key] = records binned
@@ -953,10 +970,10 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     f.dens_th = p->dens_th;
     f.particle_th = p->particle_th;
     f.cat_cap = cat_cap;
-    CWTHF_LAUNCH(ctx, s, "k_keep", k_keep<<<blocks, kThreads, 0, s>>>(ctx->acc, d_nseeds, ctx->d_mtot, f, ctx->keep_off));
+    CWTHF_LAUNCH(ctx, s, "k_keep", pdl(k_keep, blocks, kThreads, 0, s)(ctx->acc, d_nseeds, ctx->d_mtot, f, ctx->keep_off));
     if ((rc = scan_u32_dev(ctx, ctx->keep_off, ctx->keep_off, d_nseeds, slot_cap, s))) return rc;
     CWTHF_LAUNCH(ctx, s, "k_catalogue",
-                 k_catalogue<<<blocks, kThreads, 0, s>>>(ctx->acc, ctx->seed_list, d_nseeds, ctx->keep_off, cwt, f,
+                 pdl(k_catalogue, blocks, kThreads, 0, s)(ctx->acc, ctx->seed_list, d_nseeds, ctx->keep_off, cwt, f,
                                                          cat, ctx->slot_halo + int64_t(scale) * slot_cap, n_halo,
                                                          ctx->d_status));
     if (scale == n_scales - 1) {  // halo ids of all scales at once
@@ -964,7 +981,7 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
         const uint32_t* total = ctx->dep_off + total_key;
         if (rs == 1)
             CWTHF_LAUNCH(ctx, s, "k_finalize",
-                         k_finalize_one<<<pblocks, kThreads, 0, s>>>(ctx->part_rec, np, total, ctx->part_slot,
+                         pdl(k_finalize_one, pblocks, kThreads, 0, s)(ctx->part_rec, np, total, ctx->part_slot,
                                                                      ctx->slot_halo, halo_id));
         else if (rs == 2) launch_ids<2>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
         else launch_ids<4>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);

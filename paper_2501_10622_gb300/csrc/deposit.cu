@@ -81,6 +81,7 @@ __device__ __forceinline__ uint32_t* copy_of(uint32_t* counters, Copies c) {
 // Pass 1: particles per (tile, class) and the integer mass total.
 __global__ void __launch_bounds__(kCountThreads) k_dep_count(DepArgs a, uint32_t* __restrict__ counters, Copies cp,
                                                             unsigned long long* __restrict__ mtot, int* status) {
+    pdl_wait();
     uint32_t* count = copy_of(counters, cp);
     int lane = threadIdx.x & 31;
     int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(kCountThreads) k_dep_count(DepArgs a, uint32_t
 template <int N>
 __global__ void __launch_bounds__(kCountThreads) k_dep_merge(uint32_t* __restrict__ counters, uint32_t nkeys,
                                                             uint32_t* __restrict__ total) {
+    pdl_wait();
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nkeys; k += gridDim.x * blockDim.x) {
         uint32_t n[N], t = 0;
 #pragma unroll
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(kCountThreads) k_dep_merge(uint32_t* __restric
 template <int N>
 __global__ void __launch_bounds__(kCountThreads) k_dep_starts(uint32_t* __restrict__ counters, uint32_t nkeys,
                                                              const uint32_t* __restrict__ off) {
+    pdl_wait();
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nkeys; k += gridDim.x * blockDim.x) {
         const uint32_t o = off[k];
         uint32_t n[N];
@@ -139,6 +142,7 @@ __global__ void __launch_bounds__(kCountThreads) k_dep_scatter(DepArgs a, uint32
                                                               unsigned long long* __restrict__ rec,
                                                               uint32_t* __restrict__ rec_mq,
                                                               uint32_t* __restrict__ part_rec, int* status) {
+    pdl_wait();
     uint32_t* cursor = copy_of(cursors, cp);
     int lane = threadIdx.x & 31;
     int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -215,6 +219,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepAr
                                                           const uint32_t* __restrict__ rec_mq,
                                                           const unsigned long long* __restrict__ mtot,
                                                           int64_t* __restrict__ grid, int* status, TileParts tp) {
+    pdl_wait();
     constexpr int kCells = kDepTX * kDepTY * kDepTZ;
     __shared__ __align__(16) uint32_t acc_lo[kCells];
     __shared__ __align__(16) uint32_t acc_hi[kCells];
@@ -400,17 +405,17 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     int blocks = int(std::min<int64_t>(div_up(std::max<int64_t>(np, 1), kCountThreads), int64_t(ctx->sm_count) * 16));
     const int kblocks = int(std::min<int64_t>(div_up(nkeys, kCountThreads), int64_t(ctx->sm_count) * 8));
     CWTHF_LAUNCH(ctx, s, "k_dep_count",
-                 k_dep_count<<<blocks, kCountThreads, 0, s>>>(a, counters, cp, ctx->d_mtot, ctx->d_status));
+                 pdl(k_dep_count, blocks, kCountThreads, 0, s)(a, counters, cp, ctx->d_mtot, ctx->d_status));
     if (cp.n > 1)
         CWTHF_LAUNCH(ctx, s, "k_dep_merge",
-                     (cp.n == 16 ? k_dep_merge<16> : k_dep_merge<8>)<<<kblocks, kCountThreads, 0, s>>>(
+                     pdl((cp.n == 16 ? k_dep_merge<16> : k_dep_merge<8>), kblocks, kCountThreads, 0, s)(
                          counters, cp.nkeys, ctx->dep_count));
     int rc = scan_u32(ctx, ctx->dep_count, ctx->dep_off, nkeys, s);
     if (rc) return rc;
     uint32_t* cursors = cp.n > 1 ? counters : ctx->dep_cursor;
     if (cp.n > 1) {
         CWTHF_LAUNCH(ctx, s, "k_dep_starts",
-                     (cp.n == 16 ? k_dep_starts<16> : k_dep_starts<8>)<<<kblocks, kCountThreads, 0, s>>>(
+                     pdl((cp.n == 16 ? k_dep_starts<16> : k_dep_starts<8>), kblocks, kCountThreads, 0, s)(
                          counters, cp.nkeys, ctx->dep_off));
     } else if ((e = cudaMemcpyAsync(ctx->dep_cursor, ctx->dep_off, size_t(nkeys) * 4, cudaMemcpyDeviceToDevice, s)) !=
                cudaSuccess) {
@@ -418,7 +423,7 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     }
     // (the same blocks as the counting pass: a particle's copy is its block's)
     CWTHF_LAUNCH(ctx, s, "k_dep_scatter",
-                 k_dep_scatter<<<blocks, kCountThreads, 0, s>>>(a, cursors, cp, ctx->dep_rec, ctx->dep_mq,
+                 pdl(k_dep_scatter, blocks, kCountThreads, 0, s)(a, cursors, cp, ctx->dep_rec, ctx->dep_mq,
                                                                 ctx->part_rec, ctx->d_status));
     return cuda_status(cudaGetLastError());
 }
@@ -443,11 +448,11 @@ int deposit_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mas
     const auto tiles = mass ? k_dep_tile<false, true> : k_dep_tile<false, false>;
     const auto parts = mass ? k_dep_tile<true, true> : k_dep_tile<true, false>;
     CWTHF_LAUNCH(ctx, s, "k_dep_tile",
-                 tiles<<<tblocks, kTileThreads, 0, s>>>(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid,
+                 pdl(tiles, tblocks, kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid,
                                                         ctx->d_status, tp));
     // the dense tiles' further parts (returns at once when there are none)
     CWTHF_LAUNCH(ctx, s, "k_dep_parts",
-                 parts<<<ctx->sm_count * kTileCtasPerSm, kTileThreads, 0, s>>>(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq,
+                 pdl(parts, ctx->sm_count * kTileCtasPerSm, kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq,
                                                                                ctx->d_mtot, grid, ctx->d_status, tp));
     if (mtot && (e = cudaMemcpyAsync(mtot, ctx->d_mtot, 8, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return cuda_status(e);
@@ -466,19 +471,19 @@ int deposit_into_scratch(const DepositScratch& sc, const float* pos, const float
     if ((e = cudaMemsetAsync(sc.mtot, 0, 8, s)) != cudaSuccess) return cuda_status(e);
     int blocks = int(std::min<int64_t>(div_up(std::max<int64_t>(np, 1), kCountThreads), int64_t(sc.sm_count) * 16));
     const Copies one{1, uint32_t(nkeys)};
-    k_dep_count<<<blocks, kCountThreads, 0, s>>>(a, sc.count, one, sc.mtot, sc.status);
+    pdl(k_dep_count, blocks, kCountThreads, 0, s)(a, sc.count, one, sc.mtot, sc.status);
     int rc = scan_u32_scratch(sc.count, sc.off, nkeys, sc.scan_tmp, sc.scan_cap, s);
     if (rc) return rc;
     if ((e = cudaMemcpyAsync(sc.cursor, sc.off, size_t(nkeys) * 4, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return cuda_status(e);
-    k_dep_scatter<<<blocks, kCountThreads, 0, s>>>(a, sc.cursor, one, sc.rec, sc.mq, nullptr, sc.status);
+    pdl(k_dep_scatter, blocks, kCountThreads, 0, s)(a, sc.cursor, one, sc.rec, sc.mq, nullptr, sc.status);
     int tblocks = int(std::min<int64_t>(g.ntiles, int64_t(sc.sm_count) * kTileCtasPerSm));
     TileParts whole;  // no part list: every tile whole
     whole.list = nullptr;
     whole.count = nullptr;
     whole.cap = 0;
     whole.split = kTileSplit;
-    (mass ? k_dep_tile<false, true> : k_dep_tile<false, false>)<<<tblocks, kTileThreads, 0, s>>>(a, sc.off, sc.rec, sc.mq, sc.mtot, grid, sc.status, whole);
+    pdl((mass ? k_dep_tile<false, true> : k_dep_tile<false, false>), tblocks, kTileThreads, 0, s)(a, sc.off, sc.rec, sc.mq, sc.mtot, grid, sc.status, whole);
     return cuda_status(cudaGetLastError());
 }
 

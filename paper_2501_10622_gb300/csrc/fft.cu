@@ -440,7 +440,7 @@ int launch_yz(cwthf_ctx* ctx, float2* src, float2* dst, int ng, bool along_z, in
     const YzKernel k = pp.ct ? pp.ct->yz : dyn_yz();
     const size_t smem = yz_smem(p, a.trows);
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    CWTHF_LAUNCH(ctx, s, "k_fft_yz", k<<<unsigned(a.ncc) * ng, p.T, smem, s>>>(in_map, out_map, a));
+    CWTHF_LAUNCH(ctx, s, "k_fft_yz", pdl(k, unsigned(a.ncc) * ng, p.T, smem, s)(in_map, out_map, a));
     return cuda_status(cudaGetLastError());
 }
 
@@ -477,7 +477,7 @@ int transform_forward_xy(cwthf_ctx* ctx, const int64_t* grid, int ng, float2* sp
     if (rc) return rc;
     const XFwdKernel k = ct ? ct->xf : dyn_x_fwd();
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(x_smem(a.p)));
-    CWTHF_LAUNCH(ctx, s, "k_fft_x_fwd", k<<<div_up(a.rows, a.p.C), a.p.T, x_smem(a.p), s>>>(a, grid, spec));
+    CWTHF_LAUNCH(ctx, s, "k_fft_x_fwd", pdl(k, div_up(a.rows, a.p.C), a.p.T, x_smem(a.p), s)(a, grid, spec));
     if ((rc = cuda_status(cudaGetLastError()))) return rc;
     return launch_yz(ctx, spec, spec, ng, false, kYzForward, t, nullptr, 0.0, 1.0, s);
 }
@@ -505,7 +505,7 @@ int transform_wavelet_inverse(cwthf_ctx* ctx, float2* src, float2* dst, int ng, 
     if ((rc = x_args(ctx, ng, t, a, ct))) return rc;
     const XInvKernel k = ct ? ct->xi : dyn_x_inv();
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(x_smem(a.p)));
-    CWTHF_LAUNCH(ctx, s, "k_fft_x_inv", k<<<div_up(a.rows, a.p.C), a.p.T, x_smem(a.p), s>>>(a, dst, cwt));
+    CWTHF_LAUNCH(ctx, s, "k_fft_x_inv", pdl(k, div_up(a.rows, a.p.C), a.p.T, x_smem(a.p), s)(a, dst, cwt));
     return cuda_status(cudaGetLastError());
 }
 

@@ -616,6 +616,7 @@ struct YzArgs {
 template <class F>
 __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks)
     k_fft_yz(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap out_map, YzArgs a) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const Plan& p = a.p;
     const int C = F::cols(p);
@@ -704,6 +705,7 @@ __device__ __forceinline__ unsigned long long row_mean(unsigned long long s, uns
 template <class F>
 __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_fwd(XArgs a, const int64_t* __restrict__ grid,
                                                                           float2* __restrict__ spec) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const Plan& p = a.p;
     const int M = F::kLiteral ? F::len(p) : a.M, C = F::cols(p);
@@ -784,6 +786,7 @@ __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_fwd(XArgs 
 template <class F>
 __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_inv(XArgs a, const float2* __restrict__ spec,
                                                                           float* __restrict__ cwt) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const Plan& p = a.p;
     const int M = F::kLiteral ? F::len(p) : a.M, C = F::cols(p);

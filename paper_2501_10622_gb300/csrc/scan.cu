@@ -60,6 +60,7 @@ __device__ __forceinline__ uint32_t scan_value(uint32_t w) {
 template <bool kPopc>
 __global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t* __restrict__ in, int64_t n,
                                                              const uint32_t* d_n, uint32_t* __restrict__ sums) {
+    pdl_wait();
     int64_t len = scan_len(n, d_n);
     int64_t base = int64_t(blockIdx.x) * kScanChunk;
     if (base >= len) return;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t* __r
 // One block scans the (<= 32 * kScanThreads * ...) block sums in place, sequential chunks.
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* sums, int64_t nblocks_cap, int64_t n,
                                                             const uint32_t* d_n) {
+    pdl_wait();
     int64_t len = scan_len(n, d_n);
     int64_t nb = (len + kScanChunk - 1) / kScanChunk;
     if (nb > nblocks_cap) nb = nblocks_cap;
@@ -103,6 +105,7 @@ template <bool kPopc>
 __global__ void __launch_bounds__(kScanThreads) k_scan_add(const uint32_t* in, int64_t n, const uint32_t* d_n,
                                                            const uint32_t* __restrict__ sums, int64_t nblocks_cap,
                                                            uint32_t* out) {
+    pdl_wait();
     int64_t len = scan_len(n, d_n);
     int64_t base = int64_t(blockIdx.x) * kScanChunk;
     if (blockIdx.x == 0 && threadIdx.x == 0) out[len] = sums[nblocks_cap];
@@ -135,6 +138,7 @@ constexpr int64_t kScanOneMaxDev = 16 * kScanOneThreads * kScanOneItems;  // cap
 template <bool kPopc>
 __global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const uint32_t* in, int64_t n, const uint32_t* d_n,
                                                               uint32_t* out) {
+    pdl_wait();
     const int64_t len = scan_len(n, d_n);
     uint32_t carry = 0;
     for (int64_t base = 0; base < len; base += kScanOneThreads * kScanOneItems) {
@@ -161,16 +165,16 @@ template <bool kPopc>
 int scan_generic(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n_cap, const uint32_t* d_n,
                  cudaStream_t s) {
     if (n_cap <= (d_n ? kScanOneMaxDev : kScanOneMax)) {
-        CWTHF_LAUNCH(ctx, s, "k_scan_one", k_scan_one<kPopc><<<1, kScanOneThreads, 0, s>>>(in, n_cap, d_n, out));
+        CWTHF_LAUNCH(ctx, s, "k_scan_one", pdl(k_scan_one<kPopc>, 1, kScanOneThreads, 0, s)(in, n_cap, d_n, out));
         return cuda_status(cudaGetLastError());
     }
     int64_t nb = (n_cap + kScanChunk - 1) / kScanChunk;
     if (nb < 1) nb = 1;
     if (size_t(nb) + 2 > ctx->scan_tmp_cap) return CWTHF_E_INVALID_ARG;
     uint32_t* sums = ctx->scan_tmp;
-    CWTHF_LAUNCH(ctx, s, "k_block_sums", k_block_sums<kPopc><<<unsigned(nb), kScanThreads, 0, s>>>(in, n_cap, d_n, sums));
-    CWTHF_LAUNCH(ctx, s, "k_scan_sums", k_scan_sums<<<1, kScanThreads, 0, s>>>(sums, nb, n_cap, d_n));
-    CWTHF_LAUNCH(ctx, s, "k_scan_add", k_scan_add<kPopc><<<unsigned(nb), kScanThreads, 0, s>>>(in, n_cap, d_n, sums, nb, out));
+    CWTHF_LAUNCH(ctx, s, "k_block_sums", pdl(k_block_sums<kPopc>, unsigned(nb), kScanThreads, 0, s)(in, n_cap, d_n, sums));
+    CWTHF_LAUNCH(ctx, s, "k_scan_sums", pdl(k_scan_sums, 1, kScanThreads, 0, s)(sums, nb, n_cap, d_n));
+    CWTHF_LAUNCH(ctx, s, "k_scan_add", pdl(k_scan_add<kPopc>, unsigned(nb), kScanThreads, 0, s)(in, n_cap, d_n, sums, nb, out));
     return cuda_status(cudaGetLastError());
 }
 
@@ -195,9 +199,9 @@ int scan_popc(cwthf_ctx* ctx, const uint32_t* bits, uint32_t* out, int64_t n, cu
 int scan_u32_scratch(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, size_t tmp_cap, cudaStream_t s) {
     int64_t nb = std::max<int64_t>((n + kScanChunk - 1) / kScanChunk, 1);
     if (size_t(nb) + 2 > tmp_cap) return CWTHF_E_INVALID_ARG;
-    k_block_sums<false><<<unsigned(nb), kScanThreads, 0, s>>>(in, n, nullptr, tmp);
-    k_scan_sums<<<1, kScanThreads, 0, s>>>(tmp, nb, n, nullptr);
-    k_scan_add<false><<<unsigned(nb), kScanThreads, 0, s>>>(in, n, nullptr, tmp, nb, out);
+    pdl(k_block_sums<false>, unsigned(nb), kScanThreads, 0, s)(in, n, nullptr, tmp);
+    pdl(k_scan_sums, 1, kScanThreads, 0, s)(tmp, nb, n, nullptr);
+    pdl(k_scan_add<false>, unsigned(nb), kScanThreads, 0, s)(in, n, nullptr, tmp, nb, out);
     return cuda_status(cudaGetLastError());
 }
 

@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(kSegThreads, 4) k_seg_tile(const float* __rest
                                                              uint32_t* __restrict__ seed_bits,
                                                              uint32_t* __restrict__ seed_cells,
                                                              uint32_t* __restrict__ ballots, int* status) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char seg_smem[];
     __shared__ uint32_t n_seeds;
     if (threadIdx.x == 0) n_seeds = 0;  // (the tile's first barrier is before its first use)
@@ -517,6 +518,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
                                                                  int* __restrict__ changed,
                                                                  unsigned* __restrict__ next_rows, int limit,
                                                                  int rows, int* status) {
+    pdl_wait();
     __shared__ uint32_t batch[kResolveThreads / 32][64];  // pending cells (fewer than 32 between batches)
     __shared__ int32_t tkey[kResTab];
     __shared__ uint32_t tcnt[kResTab];
@@ -608,6 +610,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
 __global__ void __launch_bounds__(256) k_seg_fallback(int32_t* __restrict__ label, int64_t cells, int* changed,
                                                       int rounds, const uint32_t* __restrict__ bits,
                                                       uint32_t* __restrict__ seed_cells, unsigned* bar, int* status) {
+    pdl_wait();
     if (*reinterpret_cast<volatile int*>(&changed[0]) == 0) return;  // the same answer in every CTA
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t gid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -646,6 +649,7 @@ __global__ void __launch_bounds__(256) k_seg_fallback(int32_t* __restrict__ labe
 __global__ void k_seed_list(const uint32_t* __restrict__ bits, const uint32_t* __restrict__ prefix, int64_t nwords,
                             int64_t slot_cap, int32_t* __restrict__ seed_list, uint32_t* __restrict__ n_slots,
                             int* status) {
+    pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         uint32_t total = prefix[nwords];
         if (int64_t(total) > slot_cap) set_status(status, CWTHF_E_BAD_INPUT);
@@ -670,6 +674,7 @@ __global__ void k_seed_list(const uint32_t* __restrict__ bits, const uint32_t* _
 // 1024^3, 0.14 + 0.40 now).
 __global__ void k_seed_acc(const int32_t* __restrict__ seed_list, const uint32_t* __restrict__ seed_cells,
                            HaloAcc* __restrict__ acc, const uint32_t* __restrict__ n_slots) {
+    pdl_wait();
     // an accumulator is three 16-byte pieces, all zero but the count in the last one's upper half; one
     // thread per piece, so that a warp's stores are contiguous
     static_assert(sizeof(HaloAcc) == 48 && offsetof(HaloAcc, n_cells) == 40, "piece layout");
@@ -684,6 +689,7 @@ __global__ void k_seed_acc(const int32_t* __restrict__ seed_list, const uint32_t
 // Seeds from a label grid: the cells labelled with their own index.
 __global__ void k_seeds_from_labels(const int32_t* __restrict__ label, int64_t cells, uint32_t* __restrict__ bits,
                                     int* status) {
+    pdl_wait();
     int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < cells; c += stride) {
         int32_t l = label[c];
@@ -696,6 +702,7 @@ __global__ void k_seeds_from_labels(const int32_t* __restrict__ label, int64_t c
 __global__ void k_segment_sizes(const int32_t* __restrict__ seed_list, const HaloAcc* __restrict__ acc,
                                 const uint32_t* __restrict__ n_slots, int64_t cap, int32_t* __restrict__ seeds,
                                 int64_t* __restrict__ n_cells, int64_t* __restrict__ n_out) {
+    pdl_wait();
     const int64_t ns = *n_slots;
     if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = ns;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -710,7 +717,7 @@ __global__ void k_segment_sizes(const int32_t* __restrict__ seed_list, const Hal
 int segment_sizes_impl(cwthf_ctx* ctx, int32_t* seeds, int64_t* n_cells, int64_t cap, int64_t* n_seeds,
                        cudaStream_t s) {
     CWTHF_LAUNCH(ctx, s, "k_segment_sizes",
-                 k_segment_sizes<<<ctx->sm_count, 256, 0, s>>>(ctx->seed_list, ctx->acc, ctx->n_seeds, cap, seeds,
+                 pdl(k_segment_sizes, ctx->sm_count, 256, 0, s)(ctx->seed_list, ctx->acc, ctx->n_seeds, cap, seeds,
                                                                n_cells, n_seeds));
     return cuda_status(cudaGetLastError());
 }
@@ -722,10 +729,10 @@ int seeds_rank(cwthf_ctx* ctx, int ng, const uint32_t* seed_cells, cudaStream_t 
     int rc = scan_popc(ctx, ctx->seed_bits, ctx->seed_prefix, nwords, s);
     if (rc) return rc;
     CWTHF_LAUNCH(ctx, s, "k_seed_list",
-                 k_seed_list<<<blocks, 256, 0, s>>>(ctx->seed_bits, ctx->seed_prefix, nwords, cells / 8 + 8,
+                 pdl(k_seed_list, blocks, 256, 0, s)(ctx->seed_bits, ctx->seed_prefix, nwords, cells / 8 + 8,
                                                     ctx->seed_list, ctx->n_seeds, ctx->d_status));
     CWTHF_LAUNCH(ctx, s, "k_seed_acc",
-                 k_seed_acc<<<blocks, 256, 0, s>>>(ctx->seed_list, seed_cells, ctx->acc, ctx->n_seeds));
+                 pdl(k_seed_acc, blocks, 256, 0, s)(ctx->seed_list, seed_cells, ctx->acc, ctx->n_seeds));
     return cuda_status(cudaGetLastError());
 }
 
@@ -734,7 +741,7 @@ int seeds_from_labels(cwthf_ctx* ctx, const int32_t* label, int ng, cudaStream_t
     int64_t nwords = (cells + 31) / 32;
     cudaError_t e = cudaMemsetAsync(ctx->seed_bits, 0, size_t(nwords) * 4, s);
     if (e != cudaSuccess) return cuda_status(e);
-    CWTHF_LAUNCH(ctx, s, "k_seeds_from_labels", k_seeds_from_labels<<<ctx->sm_count * 8, 256, 0, s>>>(label, cells, ctx->seed_bits, ctx->d_status));
+    CWTHF_LAUNCH(ctx, s, "k_seeds_from_labels", pdl(k_seeds_from_labels, ctx->sm_count * 8, 256, 0, s)(label, cells, ctx->seed_bits, ctx->d_status));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e);
     return seeds_rank(ctx, ng, nullptr, s);
 }
@@ -775,7 +782,7 @@ int segment_impl(cwthf_ctx* ctx, const float* cwt, int ng, float cwt_min, int32_
     if (ntiles * (kChTY * kRowWords * 4) > cells * 8) return CWTHF_E_UNSUPPORTED_SIZE;
     cudaFuncSetAttribute(k_seg_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kSegSmem);
     CWTHF_LAUNCH(ctx, s, "k_seg_tile",
-                 k_seg_tile<<<unsigned(ntiles), kSegThreads, kSegSmem, s>>>(cwt, ng, cwt_min, label, ctx->seed_bits,
+                 pdl(k_seg_tile, unsigned(ntiles), kSegThreads, kSegSmem, s)(cwt, ng, cwt_min, label, ctx->seed_bits,
                                                                             ctx->seed_cells, ballots, ctx->d_status));
     // chains that left their tile, counted at their seed's cell
     int blocks = ctx->sm_count * 8;
@@ -785,7 +792,7 @@ int segment_impl(cwthf_ctx* ctx, const float* cwt, int ng, float cwt_min, int32_
     // GPU (64^3: 38 us with 16 whole tiles, 27 us)
     const int rows = ntiles < 2 * ctx->sm_count ? 2 : (ntiles < 16 * blocks ? kChTY : 4 * kChTY);
     CWTHF_LAUNCH(ctx, s, "k_seg_resolve",
-                 k_seg_resolve<<<blocks, kResolveThreads, 0, s>>>(label, ng, ballots, ctx->seed_cells, changed,
+                 pdl(k_seg_resolve, blocks, kResolveThreads, 0, s)(label, ng, ballots, ctx->seed_cells, changed,
                                                                    reinterpret_cast<unsigned*>(changed + kJumpTileCounter),
                                                                    ctx->dbg_chase_limit, rows, ctx->d_status));
     // pointer doubling and a recount for whatever the bounded walks left

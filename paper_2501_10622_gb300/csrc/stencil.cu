@@ -48,6 +48,7 @@ __host__ __device__ constexpr int x_pitch_r(int ng, int RC) { return (ng + 2 * R
 template <int RC>
 __global__ void __launch_bounds__(32 * kXWarps) k_sten_x_reg(const int64_t* __restrict__ grid, int ng, StencilTaps t,
                                                              float* __restrict__ A, float* __restrict__ B) {
+    pdl_wait();
     extern __shared__ __align__(16) float rows[];  // [kXWarps][pitch]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* buf = rows + warp * x_pitch_r(ng, RC);
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(kLineThreads) k_sten_yz_reg(const float* __res
                                                              const float* __restrict__ in1, int ng, StencilTaps t,
                                                              float scale, float* __restrict__ out0,
                                                              float* __restrict__ out1) {
+    pdl_wait();
     constexpr int H = kLine + 2 * RC, W = kOut + 2 * RC;
     extern __shared__ float tile[];  // [2][H][32]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -194,6 +196,7 @@ __global__ void __launch_bounds__(kLineThreads) k_sten_yz_reg(const float* __res
 // columns lane, lane + 32, ...
 __global__ void __launch_bounds__(32 * kXWarps) k_sten_x(const int64_t* __restrict__ grid, int ng, StencilTaps t,
                                                          float* __restrict__ A, float* __restrict__ B) {
+    pdl_wait();
     extern __shared__ float rows[];  // [kXWarps][ng + 2R]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int R = t.R, W = ng + 2 * R;
@@ -230,6 +233,7 @@ template <bool kZ>
 __global__ void __launch_bounds__(kLineThreads) k_sten_yz(const float* __restrict__ in0, const float* __restrict__ in1,
                                                          int ng, StencilTaps t, float scale,
                                                          float* __restrict__ out0, float* __restrict__ out1) {
+    pdl_wait();
     extern __shared__ float tile[];  // [2][kLine + 2R][32]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int R = t.R, H = kLine + 2 * R;
@@ -292,13 +296,13 @@ int launch_reg(cwthf_ctx* ctx, const int64_t* grid, int ng, const StencilTaps& t
                float* P, float* Q, float* cwt, cudaStream_t s) {
     const size_t xs = size_t(kXWarps) * x_pitch_r(ng, RC) * sizeof(float);
     CWTHF_LAUNCH(ctx, s, "k_sten_x",
-                 k_sten_x_reg<RC><<<div_up(int64_t(ng) * ng, kXWarps), 32 * kXWarps, xs, s>>>(grid, ng, t, A, B));
+                 pdl(k_sten_x_reg<RC>, div_up(int64_t(ng) * ng, kXWarps), 32 * kXWarps, xs, s)(grid, ng, t, A, B));
     const size_t ls = size_t(2) * (kLine + 2 * RC) * 32 * sizeof(float);
     const unsigned lblocks = unsigned(div_up(ng, 32) * div_up(ng, kLine) * ng);
     CWTHF_LAUNCH(ctx, s, "k_sten_y",
-                 k_sten_yz_reg<false, RC><<<lblocks, kLineThreads, ls, s>>>(A, B, ng, t, 1.0f, P, Q));
+                 pdl(k_sten_yz_reg<false, RC>, lblocks, kLineThreads, ls, s)(A, B, ng, t, 1.0f, P, Q));
     CWTHF_LAUNCH(ctx, s, "k_sten_z",
-                 k_sten_yz_reg<true, RC><<<lblocks, kLineThreads, ls, s>>>(P, Q, ng, t, scale, cwt, nullptr));
+                 pdl(k_sten_yz_reg<true, RC>, lblocks, kLineThreads, ls, s)(P, Q, ng, t, scale, cwt, nullptr));
     return cuda_status(cudaGetLastError());
 }
 
@@ -329,13 +333,13 @@ int transform_stencil_impl(cwthf_ctx* ctx, const int64_t* grid, int ng, double L
     if (R <= kRegMaxR) return launch_reg<16>(ctx, grid, ng, t, scale, A, B, P, Q, cwt, s);
     const size_t xs = size_t(kXWarps) * (ng + 2 * R) * sizeof(float);
     const int xblocks = div_up(int64_t(ng) * ng, kXWarps);
-    CWTHF_LAUNCH(ctx, s, "k_sten_x", k_sten_x<<<xblocks, 32 * kXWarps, xs, s>>>(grid, ng, t, A, B));
+    CWTHF_LAUNCH(ctx, s, "k_sten_x", pdl(k_sten_x, xblocks, 32 * kXWarps, xs, s)(grid, ng, t, A, B));
     const size_t ls = size_t(2) * (kLine + 2 * R) * 32 * sizeof(float);
     const unsigned lblocks = unsigned(div_up(ng, 32) * div_up(ng, kLine) * ng);
     cudaFuncSetAttribute(k_sten_yz<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ls));
     cudaFuncSetAttribute(k_sten_yz<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ls));
-    CWTHF_LAUNCH(ctx, s, "k_sten_y", k_sten_yz<false><<<lblocks, kLineThreads, ls, s>>>(A, B, ng, t, 1.0f, P, Q));
-    CWTHF_LAUNCH(ctx, s, "k_sten_z", k_sten_yz<true><<<lblocks, kLineThreads, ls, s>>>(P, Q, ng, t, scale, cwt, nullptr));
+    CWTHF_LAUNCH(ctx, s, "k_sten_y", pdl(k_sten_yz<false>, lblocks, kLineThreads, ls, s)(A, B, ng, t, 1.0f, P, Q));
+    CWTHF_LAUNCH(ctx, s, "k_sten_z", pdl(k_sten_yz<true>, lblocks, kLineThreads, ls, s)(P, Q, ng, t, scale, cwt, nullptr));
     return cuda_status(cudaGetLastError());
 }
 

@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(kBinThreads) k_ub_bin(const float* __restrict_
                                                         const uint32_t* __restrict__ off,
                                                         uint32_t* __restrict__ counter, int32_t* __restrict__ mem,
                                                         int32_t* __restrict__ group_out, int* status) {
+    pdl_wait();
     __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab];
     __shared__ uint32_t n_used;
     if (d_groups) n_groups = *d_groups;
@@ -829,6 +830,7 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
 // CWTHF_E_TIMEOUT.  A team's scratch is that of its CTAs, so teams of either
 // size never share any.
 __global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
+    pdl_wait();
     __shared__ double shd[8 * kUbWarps];
     __shared__ int64_t shi[kUbWarps + 1];
     __shared__ uint32_t hist[kUbWarps * 256];
@@ -871,6 +873,7 @@ __global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
 
 // A persistent grid over the groups: each CTA takes groups g, g + gridDim.x, ...
 __global__ void __launch_bounds__(kUbThreads) k_ub_group(UbArgs a) {
+    pdl_wait();
     __shared__ uint64_t sk[kUbSmemElems];
     __shared__ int32_t sv[kUbSmemElems];
     __shared__ double shd[8 * kUbWarps];
@@ -897,13 +900,13 @@ int unbind_groups(cwthf_ctx* ctx, const float* pos, const float* vel, const floa
     if (e != cudaSuccess) return cuda_status(e);
     const int blocks = ctx->sm_count * 8;
     CWTHF_LAUNCH(ctx, s, "k_ub_count",
-                 k_ub_bin<false><<<blocks, kBinThreads, 0, s>>>(mass, mass_unit, group, np, n_groups, d_groups, nullptr,
+                 pdl(k_ub_bin<false>, blocks, kBinThreads, 0, s)(mass, mass_unit, group, np, n_groups, d_groups, nullptr,
                                                                 cnt, nullptr, group_out, ctx->d_status));
     // in place: offsets, cnt[groups] = members
     int rc = d_groups ? scan_u32_dev(ctx, cnt, cnt, d_groups, n_groups, s) : scan_u32(ctx, cnt, cnt, n_groups, s);
     if (rc) return rc;
     CWTHF_LAUNCH(ctx, s, "k_ub_scatter",
-                 k_ub_bin<true><<<blocks, kBinThreads, 0, s>>>(nullptr, 1.0, group, np, n_groups, d_groups, cnt, cur,
+                 pdl(k_ub_bin<true>, blocks, kBinThreads, 0, s)(nullptr, 1.0, group, np, n_groups, d_groups, cnt, cur,
                                                                ctx->ub_mem, nullptr, ctx->d_status));
     if (n_groups > 0) {
         UbArgs a;
@@ -930,7 +933,7 @@ int unbind_groups(cwthf_ctx* ctx, const float* pos, const float* vel, const floa
         a.ctl = ctx->ub_bar;
         if ((e = cudaMemsetAsync(ctx->ub_bar, 0, kUbBarWords * 4, s)) != cudaSuccess) return cuda_status(e);
         const unsigned grid = unsigned(std::min<int64_t>(n_groups, int64_t(ctx->sm_count) * 4));
-        CWTHF_LAUNCH(ctx, s, "k_ub_group", k_ub_group<<<grid, kUbThreads, 0, s>>>(a));
+        CWTHF_LAUNCH(ctx, s, "k_ub_group", pdl(k_ub_group, grid, kUbThreads, 0, s)(a));
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e);
         // the larger groups: one cooperative launch
         UbGrid b;
