@@ -952,6 +952,7 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     const uint32_t* d_nseeds = ctx->n_seeds;  // seeds in use (clamped to slot_cap)
     int64_t slot_cap = cells / 8 + 8;
     int blocks = ctx->sm_count * 8;
+    const int sblocks = int(std::min<int64_t>(div_up(slot_cap, kThreads), blocks));  // slots
     cudaError_t e = cudaMemsetAsync(ctx->d_mtot, 0, 8, s);
     if (e != cudaSuccess) return cuda_status(e);
     if (!seeds_ready)  // after segment_impl the resolve pass has counted the cells already
@@ -970,10 +971,10 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     f.dens_th = p->dens_th;
     f.particle_th = p->particle_th;
     f.cat_cap = cat_cap;
-    CWTHF_LAUNCH(ctx, s, "k_keep", pdl(k_keep, blocks, kThreads, 0, s)(ctx->acc, d_nseeds, ctx->d_mtot, f, ctx->keep_off));
+    CWTHF_LAUNCH(ctx, s, "k_keep", pdl(k_keep, sblocks, kThreads, 0, s)(ctx->acc, d_nseeds, ctx->d_mtot, f, ctx->keep_off));
     if ((rc = scan_u32_dev(ctx, ctx->keep_off, ctx->keep_off, d_nseeds, slot_cap, s))) return rc;
     CWTHF_LAUNCH(ctx, s, "k_catalogue",
-                 pdl(k_catalogue, blocks, kThreads, 0, s)(ctx->acc, ctx->seed_list, d_nseeds, ctx->keep_off, cwt, f,
+                 pdl(k_catalogue, sblocks, kThreads, 0, s)(ctx->acc, ctx->seed_list, d_nseeds, ctx->keep_off, cwt, f,
                                                          cat, ctx->slot_halo + int64_t(scale) * slot_cap, n_halo,
                                                          ctx->d_status));
     if (scale == n_scales - 1) {  // halo ids of all scales at once

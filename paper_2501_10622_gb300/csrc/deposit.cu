@@ -391,12 +391,15 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     DepositGeom g = deposit_geom(ng);
     DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
     int64_t nkeys = g.ntiles * kDepClasses;
-    // Copies of the counters: 16 up to about 200^3, 8 up to about 640^3, one beyond (the
-    // 1024^3 box's hottest segments are short enough) and where particles are few.  They live in the
-    // first spectrum, which is free until the forward transform.
+    // Copies of the counters: 16, as long as there are at most 2^20 counters in all (halved beyond: 320^3 8,
+    // 512^3 2, one from 640^3 on) and particles are not few.  Every copy has a part of the segment of its
+    // own, and once these are written in too many places at a time their sectors leave the cache partly
+    // filled (2^25 particles on 512^3: scatter 583 us with one copy, 798 with eight).  They live in the first
+    // spectrum, which is free until the forward transform.
     Copies cp;
     cp.nkeys = uint32_t(nkeys);
-    cp.n = nkeys <= (1 << 15) ? 16 : (nkeys <= (1 << 20) ? 8 : 1);
+    cp.n = 16;
+    while (cp.n > 1 && int64_t(cp.n) * nkeys > (1 << 20)) cp.n /= 2;
     if (np < 16 * nkeys || size_t(cp.n) * size_t(nkeys) * 4 > spec_bytes(ctx->max_ng)) cp.n = 1;
     uint32_t* counters = cp.n > 1 ? reinterpret_cast<uint32_t*>(ctx->spec) : ctx->dep_count;
     cudaError_t e;
@@ -408,14 +411,16 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
                  pdl(k_dep_count, blocks, kCountThreads, 0, s)(a, counters, cp, ctx->d_mtot, ctx->d_status));
     if (cp.n > 1)
         CWTHF_LAUNCH(ctx, s, "k_dep_merge",
-                     pdl((cp.n == 16 ? k_dep_merge<16> : k_dep_merge<8>), kblocks, kCountThreads, 0, s)(
+                     pdl((cp.n == 16 ? k_dep_merge<16> : (cp.n == 8 ? k_dep_merge<8> : (cp.n == 4 ? k_dep_merge<4> : k_dep_merge<2>))),
+                         kblocks, kCountThreads, 0, s)(
                          counters, cp.nkeys, ctx->dep_count));
     int rc = scan_u32(ctx, ctx->dep_count, ctx->dep_off, nkeys, s);
     if (rc) return rc;
     uint32_t* cursors = cp.n > 1 ? counters : ctx->dep_cursor;
     if (cp.n > 1) {
         CWTHF_LAUNCH(ctx, s, "k_dep_starts",
-                     pdl((cp.n == 16 ? k_dep_starts<16> : k_dep_starts<8>), kblocks, kCountThreads, 0, s)(
+                     pdl((cp.n == 16 ? k_dep_starts<16> : (cp.n == 8 ? k_dep_starts<8> : (cp.n == 4 ? k_dep_starts<4> : k_dep_starts<2>))),
+                         kblocks, kCountThreads, 0, s)(
                          counters, cp.nkeys, ctx->dep_off));
     } else if ((e = cudaMemcpyAsync(ctx->dep_cursor, ctx->dep_off, size_t(nkeys) * 4, cudaMemcpyDeviceToDevice, s)) !=
                cudaSuccess) {
@@ -452,7 +457,7 @@ int deposit_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mas
                                                         ctx->d_status, tp));
     // the dense tiles' further parts (returns at once when there are none)
     CWTHF_LAUNCH(ctx, s, "k_dep_parts",
-                 pdl(parts, ctx->sm_count * kTileCtasPerSm, kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq,
+                 pdl(parts, int(std::min<int64_t>(8 * np / tp.split + 1, int64_t(ctx->sm_count) * kTileCtasPerSm)), kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq,
                                                                                ctx->d_mtot, grid, ctx->d_status, tp));
     if (mtot && (e = cudaMemcpyAsync(mtot, ctx->d_mtot, 8, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return cuda_status(e);
