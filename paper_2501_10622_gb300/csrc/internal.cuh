@@ -65,7 +65,7 @@ constexpr int64_t kUnbindGridMin = 1 << 16;
 // of medium and large groups, the next of either for the teams, and from
 // kUbTeamWords on four words per team (barrier, next group): the teams of
 // kUnbindTeam CTAs, then the bigger ones of kUnbindBigTeam.
-constexpr int kUnbindGridCtaCap = 1024, kUnbindTeam = 8, kUnbindBigTeam = 32;
+constexpr int kUnbindGridCtaCap = 1024, kUnbindTeam = 8, kUnbindBigTeam = 64;
 constexpr int kUbMedium = 2, kUbLarge = 3, kUbNext = 4, kUbNextBig = 5, kUbTeamWords = 8;
 constexpr size_t kUbBarWords =
     kUbTeamWords + 4 * (kUnbindGridCtaCap / kUnbindTeam + kUnbindGridCtaCap / kUnbindBigTeam);

@@ -1,5 +1,5 @@
 // unbind.cu -- the self-boundness check (Sec. 2.3; step 9 of the Sec. 2 step
-// list), one CTA per group, or the whole grid for a large group.
+// list), one CTA per group, or a team of CTAs or the whole grid for a large one.
 //
 // For every group g, following Sec. 2.3 in order:
 //   1. the centre is the centre of mass of the current members (mass-weighted
@@ -15,10 +15,10 @@
 //   5. a group that lost more than 40 % of its particles is discarded.
 // Each round: fixed-order block reductions (the sums do not depend on timing),
 // a sort of the radii (bitonic in shared memory for small groups, a stable
-// radix sort in the group's slice of global scratch for larger ones), chunked
+// radix sort in the group's slice of global scratch for the others), chunked
 // block scans for the shell sums, and a stable compaction of the members that
-// stay.  Groups above a size threshold are processed by the whole grid instead
-// (k_ub_grid, one group at a time), with the same steps over per-CTA chunks.
+// stay.  Larger groups are shared by teams of CTAs, the largest by the whole grid
+// one at a time (k_ub_grid), with the same steps over per-CTA chunks.
 #include <algorithm>
 #include <cmath>
 
@@ -29,15 +29,17 @@ namespace {
 
 constexpr int kUbThreads = 512;
 constexpr int kUbWarps = kUbThreads / 32;
-constexpr int kUbSmemElems = 2048;  // groups up to this size sort in shared memory
-// Groups up to this size take one CTA, larger ones a team of kUnbindTeam CTAs
-// (up to the whole-grid threshold): a CTA alone worked 10 ms on a group of
-// 60,000 members while the rest of the GPU had long finished.
-constexpr int kUbCtaMax = 4096;
+// Groups up to this size take one CTA (and sort in shared memory), larger ones
+// a team of kUnbindTeam CTAs (up to the whole-grid threshold): a CTA alone
+// worked 10 ms on a group of 60,000 members while the rest of the GPU had long
+// finished.
+constexpr int kUbCtaMax = 2048;
 // Groups above the whole-grid threshold but within these sizes take a team of
 // kUnbindBigTeam CTAs: several at a time, and with cheaper barriers, than one
-// after another with every CTA (six scales on 2^24 particles, 22 such groups:
-// the check's groups 53 ms with the grid for each, 38 ms with these teams).
+// after another with every CTA.  Six scales of the paper's box on 2^24
+// particles: groups of one CTA 63 ms and of the whole grid 29 ms before; 8.3 +
+// 30 ms with teams of 8 and 32 and one CTA up to 4096 members, 6.0 + 28 with 8
+// and 64 and up to 2048 (teams of 4, 16 or 32, or of 16, 96 or 128, are slower).
 constexpr int kUbBigMin = int(kUnbindGridMin), kUbBigMax = 1 << 20;
 __device__ __forceinline__ bool big_team_group(uint32_t n) { return n > uint32_t(kUbBigMin) && n <= uint32_t(kUbBigMax); }
 
@@ -228,87 +230,6 @@ __device__ void bitonic(K* k, int32_t* v, int P) {
         }
 }
 
-// Stable LSD radix sort (8-bit digits, bytes byte0 .. byte1 - 1 of the keys)
-// of the n pairs K[0..n), V[0..n), with K[n..2n), V[n..2n) as the other
-// buffer; the result ends in K[0..n), V[0..n).  Every warp owns a contiguous
-// chunk: per pass, per-warp digit counts (shared memory), their offsets
-// digit-major then warp by warp, and a scatter that keeps each warp's chunk in
-// order (lanes of one digit ranked by match_any).  A pass in which every key
-// has the same digit moves nothing and is skipped.  All threads of the block.
-__device__ void radix_sort_pairs(uint64_t* K, int32_t* V, int n, int byte0, int byte1, uint32_t* hist, int* skip) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int chunk = (n + nw - 1) / nw;
-    const int c0 = min(n, warp * chunk), c1 = min(n, c0 + chunk);
-    const uint32_t lt = (1u << lane) - 1u;
-    uint64_t *ka = K, *kb = K + n;
-    int32_t *va = V, *vb = V + n;
-    for (int pass = byte0; pass < byte1; pass++) {
-        const int sh = 8 * pass;
-        for (int i = threadIdx.x; i < nw * 256; i += blockDim.x) hist[i] = 0u;
-        if (threadIdx.x == 0) *skip = 0;
-        __syncthreads();
-        for (int k = c0 + lane; k < c1; k += 32) atomicAdd(&hist[warp * 256 + int((ka[k] >> sh) & 255u)], 1u);
-        __syncthreads();
-        // offsets: digit d's block starts after all smaller digits; within it, warp by warp
-        uint32_t tot = 0;
-        if (threadIdx.x < 256)
-            for (int w = 0; w < nw; w++) tot += hist[w * 256 + threadIdx.x];
-        if (threadIdx.x < 256 && tot == uint32_t(n)) *skip = 1;
-        // exclusive scan of the 256 digit totals (threads 0..255, 8 warps)
-        __shared__ uint32_t wsum[8];
-        uint32_t incl = tot;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (threadIdx.x < 256 && lane == 31) wsum[warp] = incl;
-        __syncthreads();
-        if (threadIdx.x < 256) {
-            uint32_t base = incl - tot;
-            for (int w = 0; w < warp; w++) base += wsum[w];
-            for (int w = 0; w < nw; w++) {
-                const uint32_t c = hist[w * 256 + threadIdx.x];
-                hist[w * 256 + threadIdx.x] = base;
-                base += c;
-            }
-        }
-        __syncthreads();
-        if (*skip) {  // block-uniform; the barrier keeps the next pass's reset behind every read
-            __syncthreads();
-            continue;
-        }
-        uint32_t* off = hist + warp * 256;
-        for (int k0 = c0; k0 < c1; k0 += 32) {
-            const int k = k0 + lane;
-            const bool valid = k < c1;
-            const int d = valid ? int((ka[k] >> sh) & 255u) : 256;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            if (valid) {
-                const uint32_t pos = off[d] + __popc(peers & lt);
-                kb[pos] = ka[k];
-                vb[pos] = va[k];
-            }
-            __syncwarp();
-            if (valid && lane == __ffs(peers) - 1) off[d] += __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        uint64_t* tk = ka;
-        ka = kb;
-        kb = tk;
-        int32_t* tv = va;
-        va = vb;
-        vb = tv;
-    }
-    if (ka != K) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            K[i] = ka[i];
-            V[i] = va[i];
-        }
-    }
-    __syncthreads();
-}
-
 // After a stable sort by the keys' upper halves: the pair at k, if it starts a
 // run of pairs with one upper half, sorts the run by the whole keys (a stable
 // insertion).  Runs are rare and short (the upper half holds 20 bits of a
@@ -339,43 +260,25 @@ __device__ __forceinline__ bool fix_run(uint64_t* K, int32_t* V, int n, int k) {
     return true;
 }
 
-// Sorts the group's first n pairs of (K, V): a bitonic sort in shared memory
-// when the padded length fits, else the radix sort in the group's slice of
-// global scratch (2n entries).  index: keys below 2^32; otherwise whole
-// 64-bit keys, by their upper halves and the short runs those leave (eight
-// digits' passes took most of a round).
-__device__ void sort_pairs(uint64_t* K, int32_t* V, int n, bool index, uint64_t* sk, int32_t* sv, uint32_t* hist,
-                           int* skip) {
+// Sorts the group's first n <= kUbCtaMax pairs of (K, V) in shared memory.
+__device__ void sort_pairs(uint64_t* K, int32_t* V, int n, uint64_t* sk, int32_t* sv) {
     int P = 1;
     while (P < n) P <<= 1;
-    if (P <= kUbSmemElems) {
-        for (int t = threadIdx.x; t < P; t += blockDim.x) {
-            sk[t] = t < n ? K[t] : ~0ull;
-            sv[t] = t < n ? V[t] : -1;
-        }
-        __syncthreads();
-        bitonic(sk, sv, P);
-        for (int t = threadIdx.x; t < n; t += blockDim.x) {
-            K[t] = sk[t];
-            V[t] = sv[t];
-        }
-        __syncthreads();
-    } else if (index) {
-        radix_sort_pairs(K, V, n, 0, 4, hist, skip);
-    } else {
-        radix_sort_pairs(K, V, n, 4, 8, hist, skip);
-        bool ok = true;
-        for (int t = threadIdx.x; t < n; t += blockDim.x) ok &= fix_run(K, V, n, t);
-        if (__syncthreads_or(!ok)) {
-            radix_sort_pairs(K, V, n, 0, 4, hist, skip);
-            radix_sort_pairs(K, V, n, 4, 8, hist, skip);
-        }
+    for (int t = threadIdx.x; t < P; t += blockDim.x) {
+        sk[t] = t < n ? K[t] : ~0ull;
+        sv[t] = t < n ? V[t] : -1;
     }
+    __syncthreads();
+    bitonic(sk, sv, P);
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        K[t] = sk[t];
+        V[t] = sv[t];
+    }
+    __syncthreads();
 }
 
 // One group (all of the CTA's threads).
-__device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* sv, double* shd, int64_t* shi,
-                             uint32_t* hist, int* skip) {
+__device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* sv, double* shd, int64_t* shi) {
     const uint32_t base = a.off[g];
     const int n0 = int(a.off[g + 1] - base);
     const int tid = threadIdx.x;
@@ -402,7 +305,7 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
         V[t] = X[t];
     }
     __syncthreads();
-    sort_pairs(K, V, n0, true, sk, sv, hist, skip);
+    sort_pairs(K, V, n0, sk, sv);
     for (int t = tid; t < n0; t += blockDim.x) X[t] = V[t];
     __syncthreads();
     const float* a0 = a.pos + 3 * size_t(X[0]);
@@ -442,7 +345,7 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
             V[t] = i;
         }
         __syncthreads();
-        sort_pairs(K, V, n, false, sk, sv, hist, skip);
+        sort_pairs(K, V, n, sk, sv);
         // 2-3. shell sums per member and the exclusions.  Thread t walks the
         // chunk [t ch, (t+1) ch): mass before the chunk and m/r after it come
         // from block scans of the chunk totals.  Massive members at the centre
@@ -552,9 +455,14 @@ __device__ __forceinline__ double part_prefix(const UbGrid& tm, int k, double* a
     return before;
 }
 
-// The stable LSD radix sort of radix_sort_pairs over the whole grid: the
-// digit offsets add the counts of all CTAs before this one.  Returns false on
-// a barrier timeout.
+// Stable LSD radix sort (8-bit digits, bytes byte0 .. byte1 - 1 of the keys) of
+// the n pairs K[0..n), V[0..n), with K[n..2n), V[n..2n) as the other buffer; the
+// result ends in K[0..n), V[0..n).  Every warp owns a contiguous chunk: per
+// pass, per-warp digit counts (shared memory), their offsets (all smaller
+// digits, the CTAs before this one, then warp by warp), and a scatter that keeps
+// each warp's chunk in order (lanes of one digit ranked by match_any).  A pass
+// in which every key has the same digit moves nothing and is skipped.  Returns
+// false on a barrier timeout.
 __device__ bool grid_radix(uint64_t* K, int32_t* V, int n, int byte0, int byte1, const UbGrid& b, uint32_t* hist,
                            uint32_t* dsum, uint32_t* dbase, int* skip, int& parity) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -874,15 +782,13 @@ __global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
 // A persistent grid over the groups: each CTA takes groups g, g + gridDim.x, ...
 __global__ void __launch_bounds__(kUbThreads) k_ub_group(UbArgs a) {
     pdl_wait();
-    __shared__ uint64_t sk[kUbSmemElems];
-    __shared__ int32_t sv[kUbSmemElems];
+    __shared__ uint64_t sk[kUbCtaMax];
+    __shared__ int32_t sv[kUbCtaMax];
     __shared__ double shd[8 * kUbWarps];
     __shared__ int64_t shi[kUbWarps + 1];
-    __shared__ uint32_t hist[kUbWarps * 256];
-    __shared__ int skip;
     const int64_t n_groups = a.d_groups ? int64_t(*a.d_groups) : a.n_groups;
     for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
-        unbind_group(a, g, sk, sv, shd, shi, hist, &skip);
+        unbind_group(a, g, sk, sv, shd, shi);
         __syncthreads();
     }
 }

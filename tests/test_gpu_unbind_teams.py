@@ -1,5 +1,5 @@
 """The self-boundness check's ways of sharing a group among CTAs: one CTA (up
-to 4096 members; sorted in shared memory up to 2048), a team of 8, a team of 32
+to 2048 members, sorted in shared memory), a team of 8, a team of 64
 (above 65,536), the whole grid.  Group sizes sit on the edges between them; the
 decisions must not depend on the way, nor on members at equal radii."""
 import numpy as np
