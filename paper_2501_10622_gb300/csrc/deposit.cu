@@ -409,22 +409,23 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     const int kblocks = int(std::min<int64_t>(div_up(nkeys, kCountThreads), int64_t(ctx->sm_count) * 8));
     CWTHF_LAUNCH(ctx, s, "k_dep_count",
                  pdl(k_dep_count, blocks, kCountThreads, 0, s)(a, counters, cp, ctx->d_mtot, ctx->d_status));
-    if (cp.n > 1)
-        CWTHF_LAUNCH(ctx, s, "k_dep_merge",
-                     pdl((cp.n == 16 ? k_dep_merge<16> : (cp.n == 8 ? k_dep_merge<8> : (cp.n == 4 ? k_dep_merge<4> : k_dep_merge<2>))),
-                         kblocks, kCountThreads, 0, s)(
-                         counters, cp.nkeys, ctx->dep_count));
-    int rc = scan_u32(ctx, ctx->dep_count, ctx->dep_off, nkeys, s);
-    if (rc) return rc;
+    // few counters (grids up to about 100^3): merge, scan and starts in one launch
     uint32_t* cursors = cp.n > 1 ? counters : ctx->dep_cursor;
-    if (cp.n > 1) {
-        CWTHF_LAUNCH(ctx, s, "k_dep_starts",
-                     pdl((cp.n == 16 ? k_dep_starts<16> : (cp.n == 8 ? k_dep_starts<8> : (cp.n == 4 ? k_dep_starts<4> : k_dep_starts<2>))),
-                         kblocks, kCountThreads, 0, s)(
-                         counters, cp.nkeys, ctx->dep_off));
-    } else if ((e = cudaMemcpyAsync(ctx->dep_cursor, ctx->dep_off, size_t(nkeys) * 4, cudaMemcpyDeviceToDevice, s)) !=
-               cudaSuccess) {
-        return cuda_status(e);
+    if (!scan_copies(ctx, counters, cp.n, cp.nkeys, ctx->dep_off, s)) {
+        auto merge = cp.n == 16 ? k_dep_merge<16> : (cp.n == 8 ? k_dep_merge<8> : (cp.n == 4 ? k_dep_merge<4> : k_dep_merge<2>));
+        auto starts = cp.n == 16 ? k_dep_starts<16> : (cp.n == 8 ? k_dep_starts<8> : (cp.n == 4 ? k_dep_starts<4> : k_dep_starts<2>));
+        if (cp.n > 1)
+            CWTHF_LAUNCH(ctx, s, "k_dep_merge",
+                         pdl(merge, kblocks, kCountThreads, 0, s)(counters, cp.nkeys, ctx->dep_count));
+        int rc = scan_u32(ctx, ctx->dep_count, ctx->dep_off, nkeys, s);
+        if (rc) return rc;
+        if (cp.n > 1) {
+            CWTHF_LAUNCH(ctx, s, "k_dep_starts",
+                         pdl(starts, kblocks, kCountThreads, 0, s)(counters, cp.nkeys, ctx->dep_off));
+        } else if ((e = cudaMemcpyAsync(ctx->dep_cursor, ctx->dep_off, size_t(nkeys) * 4, cudaMemcpyDeviceToDevice,
+                                        s)) != cudaSuccess) {
+            return cuda_status(e);
+        }
     }
     // (the same blocks as the counting pass: a particle's copy is its block's)
     CWTHF_LAUNCH(ctx, s, "k_dep_scatter",

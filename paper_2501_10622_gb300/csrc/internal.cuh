@@ -58,7 +58,7 @@ constexpr int kJumpWords = kMaxJumpRounds + 4;
 constexpr int kDefaultChaseLimit = 64;
 
 // Groups of the self-boundness check with more members than this are
-// processed by the whole grid, one at a time; smaller ones by one CTA each.
+// processed by the whole grid, one at a time, or by big teams of CTAs.
 constexpr int64_t kUnbindGridMin = 1 << 16;
 // Most CTAs of the launch for groups of several CTAs (its per-CTA scratch is
 // sized for them); its control words: the whole grid's barrier (2), the counts
@@ -159,7 +159,7 @@ struct cwthf_ctx {
     cwthf::HaloAcc* acc = nullptr;    // [ng^3 / 8 + 1]
     uint32_t* keep_off = nullptr;     // [ng^3 / 8 + 2] kept-halo prefix
     int32_t* slot_halo = nullptr;     // [max_scales][ng^3 / 8 + 8] seed of each kept slot, -1 otherwise
-    int32_t* part_slot = nullptr;     // [max_scales][max_np] record slots (-1: none), then [max_np][1|2|4k] halo ids
+    int32_t* part_slot = nullptr;     // [max_scales][max_np] record slots (-1: none), then (several scales) [max_np][2|4k] halo ids
     int* jump_changed = nullptr;      // [kJumpWords] segmentation control words
     uint32_t* scan_tmp = nullptr;     // block sums of the device scan
     size_t scan_tmp_cap = 0;          // words
@@ -180,7 +180,7 @@ struct cwthf_ctx {
     uint32_t* dep_nparts = nullptr;          // [1] parts listed
     double* ub_part = nullptr;       // [ub_grid_blocks][16] per-CTA partial sums of the whole-grid path
     uint32_t* ub_hist = nullptr;     // [2][ub_grid_blocks][256] per-CTA digit counts of its radix sort
-    unsigned* ub_bar = nullptr;      // [kUbBarWords] its barriers and group counts
+    unsigned* ub_bar = nullptr;      // [kUbBarWords] barriers and group counts
     int ub_grid_blocks = 0;          // CTAs of the whole-grid path's cooperative launch
 
     // cwthf_find internals
@@ -477,6 +477,9 @@ int scan_u32_dev(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, const uint32
                  cudaStream_t s);
 // Same over the words' bit counts (in and out do not alias).
 int scan_popc(cwthf_ctx* ctx, const uint32_t* bits, uint32_t* out, int64_t n, cudaStream_t s);
+// Offsets of nkeys counters kept in copies (merge, scan and start of every copy
+// in one launch); false, with nothing queued, unless they are few.
+bool scan_copies(cwthf_ctx* ctx, uint32_t* counters, uint32_t copies, uint32_t nkeys, uint32_t* out, cudaStream_t s);
 size_t scan_tmp_words(int64_t n_cap);
 
 // ---- stages -------------------------------------------------------------------

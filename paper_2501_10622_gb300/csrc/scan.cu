@@ -161,6 +161,34 @@ __global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const uint32_t* in
     if (threadIdx.x == 0) out[len] = carry;
 }
 
+// Offsets of few counters kept in N copies: out[k] = the sum of all copies of
+// the counters before k, and every copy's counter becomes its start (out[k] plus
+// the copies before it).  One block, one key per thread and step.
+template <int N>
+__global__ void __launch_bounds__(kScanOneThreads) k_scan_copies(uint32_t* counters, uint32_t nkeys, uint32_t* out) {
+    pdl_wait();
+    uint32_t carry = 0;
+    for (uint32_t base = 0; base < nkeys; base += kScanOneThreads) {
+        const uint32_t k = base + threadIdx.x;
+        uint32_t n[N], local = 0, tot;
+#pragma unroll
+        for (int c = 0; c < N; c++) n[c] = k < nkeys ? counters[size_t(c) * nkeys + k] : 0u;
+#pragma unroll
+        for (int c = 0; c < N; c++) local += n[c];
+        uint32_t ex = block_excl_scan<kScanOneThreads>(local, &tot) + carry;
+        if (k < nkeys) {
+            out[k] = ex;
+#pragma unroll
+            for (int c = 0; c < N; c++) {
+                counters[size_t(c) * nkeys + k] = ex;
+                ex += n[c];
+            }
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) out[nkeys] = carry;
+}
+
 template <bool kPopc>
 int scan_generic(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n_cap, const uint32_t* d_n,
                  cudaStream_t s) {
@@ -193,6 +221,12 @@ int scan_u32_dev(cwthf_ctx* ctx, const uint32_t* in, uint32_t* out, const uint32
 
 int scan_popc(cwthf_ctx* ctx, const uint32_t* bits, uint32_t* out, int64_t n, cudaStream_t s) {
     return scan_generic<true>(ctx, bits, out, n, nullptr, s);
+}
+
+bool scan_copies(cwthf_ctx* ctx, uint32_t* counters, uint32_t copies, uint32_t nkeys, uint32_t* out, cudaStream_t s) {
+    if (copies != 16 || nkeys > 4 * kScanOneThreads) return false;
+    CWTHF_LAUNCH(ctx, s, "k_scan_copies", pdl(k_scan_copies<16>, 1, kScanOneThreads, 0, s)(counters, nkeys, out));
+    return true;
 }
 
 // The three launches on caller-provided block-sum storage (no context).
