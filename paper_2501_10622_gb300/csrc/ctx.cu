@@ -90,8 +90,7 @@ void for_each_buffer(cwthf_ctx* c, int max_ng, int64_t max_np, int max_scales, u
     f(reinterpret_cast<void**>(&c->keep_off), size_t(z.slots + 2) * 4);
     f(reinterpret_cast<void**>(&c->slot_halo), size_t(z.slots) * 4 * size_t(std::max(max_scales, 1)));
     // record slots of every scale (scale-major), then (several scales) the
-    // records' halo ids in groups of 2 or 4k scales; one scale's ids replace
-    // its slots in place
+    // records' halo ids in groups of 2 or 4k scales
     const size_t ms = size_t(std::max(max_scales, 1));
     const size_t groups = ms == 1 ? 0 : (ms == 2 ? 2 : (ms + 3) & ~size_t(3));
     f(reinterpret_cast<void**>(&c->part_slot), (size_t(z.np) * ms + 4) * 4 + size_t(z.np) * 4 * groups);
@@ -110,7 +109,7 @@ void for_each_buffer(cwthf_ctx* c, int max_ng, int64_t max_np, int max_scales, u
         f(reinterpret_cast<void**>(&c->ub_it), size_t(z.slots + 1) * 4);
         f(reinterpret_cast<void**>(&c->ub_keep), size_t(z.slots + 2) * 4);
         f(reinterpret_cast<void**>(&c->ub_ngroups), 16);
-        // the whole-grid path for large groups: per-CTA partial sums and digit counts, barrier
+        // groups of several CTAs: per-CTA partial sums and digit counts, barriers
         f(reinterpret_cast<void**>(&c->ub_part), size_t(kUnbindGridCtaCap) * 16 * 8);
         f(reinterpret_cast<void**>(&c->ub_hist), size_t(kUnbindGridCtaCap) * 2 * 256 * 4);
         f(reinterpret_cast<void**>(&c->ub_bar), kUbBarWords * 4);

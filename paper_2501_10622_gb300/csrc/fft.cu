@@ -391,8 +391,15 @@ bool pass_plan(cwthf_ctx* ctx, int ng, int which, PassPlan& p) {
         std::lock_guard<std::mutex> g(ctx->table_mu);
         for (const auto& o : ctx->fft_plans)
             if (o.ng == ng && o.which == which) {
+                const int len = which == 0 ? ng : ng / 2;
                 p.ct = nullptr;
-                return plan_from(which == 0 ? ng : ng / 2, which, o.C, o.rad, o.nst, p.p);
+                if (!plan_from(len, which, o.C, o.rad, o.nst, p.p)) return false;
+                // the built-in plan's own radices and width: its compile-time instance
+                const PassPlan& b = which == 0 ? size_plans(ng).yz : size_plans(ng).x;
+                bool same = size_plans(ng).ok && !b.p.Lb && b.p.C == o.C && b.p.nst == o.nst;
+                for (int i = 0; i < o.nst && same; i++) same = b.p.rad[i] == o.rad[i];
+                if (same) p = b;
+                return true;
             }
     }
     const SizePlans& s = size_plans(ng);
