@@ -13,7 +13,7 @@ struct DepArgs {
     double mass_unit;
     uint32_t scale_m;  // quantisation scale s = scale_m * 2^scale_e (scale_m < 2^29)
     int scale_e;
-    unsigned long long inv_m;  // 1 / mass_unit = inv_m 2^inv_e up to 2^-40.9 of it (inv_m <= 2^40)
+    unsigned long long inv_m;  // 1 / mass_unit = inv_m 2^inv_e, to 2^-40 of it (2^39 <= inv_m <= 2^40)
     int inv_e;
     int64_t modulus;   // ng * 2^10
     int64_t np;
@@ -113,12 +113,13 @@ __device__ __forceinline__ bool quantise(float x, uint32_t sm, int se, int64_t m
 }
 
 // Integer mass of particle i: 1 when masses are equal, else rint(m / mass_unit)
-// (round half to even).  The fp64 quotient is formed only where it decides:
-// m times the reciprocal's leading 40 bits, as an integer product, is within
-// 2^-9 of it (quotients below 2^31), so a fraction that far from one half
-// rounds the same way.  (fp64 units are scarce: the division alone took over
-// half of a binning pass's time with masses, 0.22 ms for 2^23 particles.)  Returns CWTHF_OK, CWTHF_E_BAD_INPUT (negative / NaN)
-// or CWTHF_E_OVERFLOW (>= 2^31).
+// (round half to even).  The fp64 quotient is formed only where it decides: m
+// times the reciprocal's leading 40 bits, as an integer product, differs from
+// the rounded quotient by at most 2^31 (2^-40 + 2 2^-53) < 2^-9 + 2^-20
+// (quotients below 2^31), so a fraction 5 2^-11 or more from one half rounds the
+// same way.  (fp64 units are scarce: the division alone took over half of a
+// binning pass's time with masses, 0.22 ms for 2^23 particles.)  Returns
+// CWTHF_OK, CWTHF_E_BAD_INPUT (negative / NaN) or CWTHF_E_OVERFLOW (>= 2^31).
 __device__ __forceinline__ int mass_quantum(const DepArgs& a, int64_t i, uint32_t& mq) {
     mq = 0;
     if (!a.mass) { mq = 1; return CWTHF_OK; }
@@ -126,10 +127,10 @@ __device__ __forceinline__ int mass_quantum(const DepArgs& a, int64_t i, uint32_
     const uint32_t b = __float_as_uint(m);
     const uint32_t sh = uint32_t(150 - a.inv_e - int(b >> 23));  // m / mass_unit = P 2^-sh
     if (b - 0x00800000u < 0x7f000000u && sh - 12u < 52u) {       // positive, normal, finite; 12 <= sh < 64
-        const unsigned long long P = (unsigned long long)((b & 0x7fffffu) | 0x800000u) * a.inv_m; 
+        const unsigned long long P = (unsigned long long)((b & 0x7fffffu) | 0x800000u) * a.inv_m;
         const unsigned long long n = P >> sh;
         const int f = int((P >> (sh - 11u)) & 2047u) - 1024;  // fraction minus one half, in 2^-11
-        if (n < 0x7ffffff0ull && (f >= 4 || f < -4)) {
+        if (n < 0x7ffffff0ull && (f >= 5 || f < -5)) {
             mq = uint32_t(n) + (f > 0 ? 1u : 0u);
             return CWTHF_OK;
         }
