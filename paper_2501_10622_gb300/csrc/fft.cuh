@@ -724,17 +724,27 @@ __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_fwd(XArgs 
     // the grid (mass_unit is applied with the wavelet).
     constexpr float kUnit = 9.3132257461547852e-10f;  // 2^-30, exact
     constexpr int kRowVec = (F::kMaxLen + 31) / 32;  // a row's int64 pairs per lane
+    const bool vec = (reinterpret_cast<uintptr_t>(grid) & 15u) == 0;  // (rows are an even number of cells)
     for (int r = warp; r < C; r += nwarp) {
         int64_t row = int64_t(blockIdx.x) * C + r;
         longlong2 v[kRowVec];
         long long sum = 0;
-        const longlong2* src = reinterpret_cast<const longlong2*>(grid + row * a.ng);
+        const int64_t* src = grid + row * a.ng;
+        if (vec) {
 #pragma unroll
-        for (int i = 0; i < kRowVec; i++) {
-            int k = lane + 32 * i;
-            v[i] = (row < a.rows && k < M) ? src[k] : make_longlong2(0, 0);
-            sum += v[i].x + v[i].y;
+            for (int i = 0; i < kRowVec; i++) {
+                int k = lane + 32 * i;
+                v[i] = (row < a.rows && k < M) ? reinterpret_cast<const longlong2*>(src)[k] : make_longlong2(0, 0);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kRowVec; i++) {
+                int k = lane + 32 * i;
+                v[i] = (row < a.rows && k < M) ? make_longlong2(src[2 * k], src[2 * k + 1]) : make_longlong2(0, 0);
+            }
         }
+#pragma unroll
+        for (int i = 0; i < kRowVec; i++) sum += v[i].x + v[i].y;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         const long long q0 = sum >= 0 ? (long long)row_mean((unsigned long long)sum, unsigned(a.ng), a.inv_ng) : sum / a.ng;
@@ -840,13 +850,20 @@ __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_inv(XArgs 
     }
     __syncthreads();
     F::dft(p, tile, addr, tw, 0u);
+    const bool vec = (reinterpret_cast<uintptr_t>(cwt) & 7u) == 0;
     for (int r = warp; r < C; r += nwarp) {
         int64_t row = int64_t(blockIdx.x) * C + r;
         if (row >= a.rows) continue;
-        float2* out = reinterpret_cast<float2*>(cwt + row * a.ng);
+        float* out = cwt + row * a.ng;
         for (int n = lane; n < M; n += 32) {
             float2 z = tile[addr(n, r)];
-            out[n] = make_float2(z.x, -z.y);  // conj back; z[n] = x[2n] + i x[2n+1]
+            z.y = -z.y;  // conj back; z[n] = x[2n] + i x[2n+1]
+            if (vec) {
+                reinterpret_cast<float2*>(out)[n] = z;
+            } else {
+                out[2 * n] = z.x;
+                out[2 * n + 1] = z.y;
+            }
         }
     }
 }
