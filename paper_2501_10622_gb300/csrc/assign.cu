@@ -27,10 +27,10 @@ using u64 = unsigned long long;
 // global atomic per distinct label of every warp took 139 us at 256^3, 92
 // us now.)
 constexpr int kCellsPerThread = 16, kCountCells = kThreads * kCellsPerThread;
-__global__ void __launch_bounds__(kThreads) k_count_cells(const int32_t* __restrict__ label, int64_t cells,
-                                                         const uint32_t* __restrict__ bits,
-                                                         const uint32_t* __restrict__ prefix,
-                                                         const uint32_t* __restrict__ n_slots, HaloAcc* acc,
+__global__ void __launch_bounds__(kThreads) k_count_cells(const int32_t* label, int64_t cells,
+                                                         const uint32_t* bits,
+                                                         const uint32_t* prefix,
+                                                         const uint32_t* n_slots, HaloAcc* acc,
                                                          int* status) {
     pdl_wait();
     __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab];
@@ -133,13 +133,13 @@ __device__ __forceinline__ u64 sext(uint32_t v) { return u64((long long)int32_t(
 __device__ __forceinline__ u64 sext(int32_t v) { return u64((long long)v); }
 
 template <bool kMass>
-__global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_sums(DepArgs a, FastDiv divn, const uint32_t* __restrict__ total_ptr,
-                                                       const unsigned long long* __restrict__ rec,
-                                                       const uint32_t* __restrict__ rec_mq,
-                                                       const int32_t* __restrict__ label,
-                                                       const uint32_t* __restrict__ bits,
-                                                       const uint32_t* __restrict__ prefix,
-                                                       const uint32_t* __restrict__ n_slots, HaloAcc* acc,
+__global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_sums(DepArgs a, FastDiv divn, const uint32_t* total_ptr,
+                                                       const unsigned long long* rec,
+                                                       const uint32_t* rec_mq,
+                                                       const int32_t* label,
+                                                       const uint32_t* bits,
+                                                       const uint32_t* prefix,
+                                                       const uint32_t* n_slots, HaloAcc* acc,
                                                        int32_t* __restrict__ rec_slot, int slot_stride,
                                                        u64* __restrict__ mtot, int skip_marked, int* status) {
     pdl_wait();
@@ -345,8 +345,8 @@ struct FilterArgs {
 };
 
 // keep flag per slot (1 / 0), scanned afterwards into output positions.
-__global__ void __launch_bounds__(kThreads) k_keep(const HaloAcc* __restrict__ acc, const uint32_t* __restrict__ n_seeds,
-                                                  const u64* __restrict__ mtot, FilterArgs f,
+__global__ void __launch_bounds__(kThreads) k_keep(const HaloAcc* acc, const uint32_t* n_seeds,
+                                                  const u64* mtot, FilterArgs f,
                                                   uint32_t* __restrict__ keep) {
     pdl_wait();
     uint32_t ns = *n_seeds;
@@ -366,10 +366,10 @@ __global__ void __launch_bounds__(kThreads) k_keep(const HaloAcc* __restrict__ a
 // Catalogue entries of the kept slots, and each slot's halo (-1: not kept).
 // Kept slots are few (about 2 % at 1024^3) and dear (fp64 divides), so a warp
 // gathers them from its slots and forms 32 entries at a time.
-__global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* __restrict__ acc,
-                                                       const int32_t* __restrict__ seed_list,
-                                                       const uint32_t* __restrict__ n_seeds,
-                                                       const uint32_t* __restrict__ keep_off, const float* cwt,
+__global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* acc,
+                                                       const int32_t* seed_list,
+                                                       const uint32_t* n_seeds,
+                                                       const uint32_t* keep_off, const float* cwt,
                                                        FilterArgs f, cwthf_halo* __restrict__ cat,
                                                        int32_t* __restrict__ slot_halo,
                                                        int64_t* __restrict__ n_halo, int* status) {
@@ -466,8 +466,8 @@ struct IdGroup<4> {
 // tile, so the slot lookups are coherent.
 template <int RS>
 __global__ void __launch_bounds__(kThreads) k_rec_halo(const int32_t* rec_slot, int64_t np,
-                                                      const uint32_t* __restrict__ total_ptr, int n_scales,
-                                                      const int32_t* __restrict__ slot_halo, int64_t slot_stride,
+                                                      const uint32_t* total_ptr, int n_scales,
+                                                      const int32_t* slot_halo, int64_t slot_stride,
                                                       typename IdGroup<RS>::T* groups) {
     pdl_wait();
     constexpr int G = RS < 4 ? RS : 4;  // ids per stored group
@@ -492,9 +492,9 @@ __global__ void __launch_bounds__(kThreads) k_rec_halo(const int32_t* rec_slot, 
 // per particle and group of its record's ids.  Several particles per thread
 // keep independent gathers in flight.
 template <int RS>
-__global__ void __launch_bounds__(kThreads) k_finalize(const uint32_t* __restrict__ part_rec, int64_t np,
-                                                      const uint32_t* __restrict__ total_ptr,
-                                                      const typename IdGroup<RS>::T* __restrict__ groups,
+__global__ void __launch_bounds__(kThreads) k_finalize(const uint32_t* part_rec, int64_t np,
+                                                      const uint32_t* total_ptr,
+                                                      const typename IdGroup<RS>::T* groups,
                                                       int n_scales, int32_t* __restrict__ halo_id) {
     pdl_wait();
     constexpr int kIlp = 8;
@@ -531,10 +531,10 @@ __global__ void __launch_bounds__(kThreads) k_finalize(const uint32_t* __restric
 // turns record slots into ids first only pays when a record's ids of several
 // scales share a gather; for one scale it read and wrote every record to save
 // a lookup in the slots' table, which is in cache).
-__global__ void __launch_bounds__(kThreads) k_finalize_one(const uint32_t* __restrict__ part_rec, int64_t np,
-                                                          const uint32_t* __restrict__ total_ptr,
-                                                          const int32_t* __restrict__ rec_slot,
-                                                          const int32_t* __restrict__ slot_halo,
+__global__ void __launch_bounds__(kThreads) k_finalize_one(const uint32_t* part_rec, int64_t np,
+                                                          const uint32_t* total_ptr,
+                                                          const int32_t* rec_slot,
+                                                          const int32_t* slot_halo,
                                                           int32_t* __restrict__ halo_id) {
     pdl_wait();
     constexpr int kIlp = 8;
@@ -575,9 +575,9 @@ void launch_ids(cwthf_ctx* ctx, cudaStream_t s, int blocks, int pblocks, int64_t
 // Records of particles that already hold a halo id are marked in bit 63, so
 // that this scale's group sums skip them (Sec. 2 step 6: only particles
 // without a halo id are assigned).
-__global__ void __launch_bounds__(kThreads) k_ms_mark(const int32_t* __restrict__ halo_id,
-                                                     const uint32_t* __restrict__ part_rec, int64_t np,
-                                                     const uint32_t* __restrict__ total_ptr,
+__global__ void __launch_bounds__(kThreads) k_ms_mark(const int32_t* halo_id,
+                                                     const uint32_t* part_rec, int64_t np,
+                                                     const uint32_t* total_ptr,
                                                      unsigned long long* __restrict__ rec) {
     pdl_wait();
     const int64_t total = *total_ptr;
@@ -590,9 +590,9 @@ __global__ void __launch_bounds__(kThreads) k_ms_mark(const int32_t* __restrict_
 
 // Each particle's group slot at this scale (-1: in no group), kept until the
 // scale's halos are decided one iteration later.
-__global__ void __launch_bounds__(kThreads) k_ms_pslot(const uint32_t* __restrict__ part_rec, int64_t np,
-                                                      const uint32_t* __restrict__ total_ptr,
-                                                      const int32_t* __restrict__ rec_slot, int32_t* __restrict__ pslot) {
+__global__ void __launch_bounds__(kThreads) k_ms_pslot(const uint32_t* part_rec, int64_t np,
+                                                      const uint32_t* total_ptr,
+                                                      const int32_t* rec_slot, int32_t* __restrict__ pslot) {
     pdl_wait();
     const int64_t total = *total_ptr;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -663,11 +663,11 @@ __device__ bool ms_cross_scale(const float* __restrict__ C, int ng, int64_t s, c
 
 // Keep flag per group (slot): particle and density thresholds (same operands
 // as the single-scale path) and the cross-scale check.
-__global__ void __launch_bounds__(kThreads) k_ms_keep(const HaloAcc* __restrict__ acc,
-                                                     const int32_t* __restrict__ seed_list,
-                                                     const uint32_t* __restrict__ n_seeds,
-                                                     const u64* __restrict__ mtot, FilterArgs f,
-                                                     const float* __restrict__ C, const float* __restrict__ Cn,
+__global__ void __launch_bounds__(kThreads) k_ms_keep(const HaloAcc* acc,
+                                                     const int32_t* seed_list,
+                                                     const uint32_t* n_seeds,
+                                                     const u64* mtot, FilterArgs f,
+                                                     const float* C, const float* Cn,
                                                      int ngn, uint32_t* __restrict__ keep) {
     pdl_wait();
     const uint32_t ns = *n_seeds;
@@ -686,12 +686,12 @@ __global__ void __launch_bounds__(kThreads) k_ms_keep(const HaloAcc* __restrict_
 
 // Kept groups become halos base + rank (base: halos of the earlier scales, read
 // from *n_halo); catalogue entries, and each slot's halo id (-1: not kept).
-__global__ void __launch_bounds__(kThreads) k_ms_catalogue(const HaloAcc* __restrict__ acc,
-                                                          const int32_t* __restrict__ seed_list,
-                                                          const uint32_t* __restrict__ n_seeds,
-                                                          const uint32_t* __restrict__ keep_off, FilterArgs f,
-                                                          const float* __restrict__ C, const float* __restrict__ Cn,
-                                                          int ngn, int scale, const int64_t* __restrict__ n_halo,
+__global__ void __launch_bounds__(kThreads) k_ms_catalogue(const HaloAcc* acc,
+                                                          const int32_t* seed_list,
+                                                          const uint32_t* n_seeds,
+                                                          const uint32_t* keep_off, FilterArgs f,
+                                                          const float* C, const float* Cn,
+                                                          int ngn, int scale, const int64_t* n_halo,
                                                           cwthf_ms_halo* __restrict__ cat,
                                                           int32_t* __restrict__ slot_halo) {
     pdl_wait();
@@ -730,7 +730,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_catalogue(const HaloAcc* __rest
 }
 
 // The number of kept groups (keep_off[n_seeds]) as the check's group count.
-__global__ void k_ms_ub_count(const uint32_t* __restrict__ keep_off, const uint32_t* __restrict__ n_seeds,
+__global__ void k_ms_ub_count(const uint32_t* keep_off, const uint32_t* n_seeds,
                               uint32_t* __restrict__ n_groups) {
     pdl_wait();
     *n_groups = keep_off[*n_seeds];
@@ -739,9 +739,9 @@ __global__ void k_ms_ub_count(const uint32_t* __restrict__ keep_off, const uint3
 // The self-boundness check inside the loop (Sec. 2 step 9, Sec. 2.3): the
 // group of each candidate particle of a kept group (its rank among the kept
 // groups), or -1.
-__global__ void __launch_bounds__(kThreads) k_ms_ub_group(const int32_t* __restrict__ pslot,
-                                                         const int32_t* __restrict__ halo_id, int64_t np,
-                                                         const uint32_t* __restrict__ keep_off,
+__global__ void __launch_bounds__(kThreads) k_ms_ub_group(const int32_t* pslot,
+                                                         const int32_t* halo_id, int64_t np,
+                                                         const uint32_t* keep_off,
                                                          int32_t* __restrict__ grp) {
     pdl_wait();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -759,9 +759,9 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_group(const int32_t* __restr
 // Kept groups that the check did not discard stay (flag per slot, scanned
 // into their ranks afterwards); their particle count, mass and first moment
 // are cleared, to be summed again over the members that stay.
-__global__ void __launch_bounds__(kThreads) k_ms_ub_keep(const uint32_t* __restrict__ n_seeds,
-                                                        const uint32_t* __restrict__ keep_off,
-                                                        const int64_t* __restrict__ n_kept, HaloAcc* acc,
+__global__ void __launch_bounds__(kThreads) k_ms_ub_keep(const uint32_t* n_seeds,
+                                                        const uint32_t* keep_off,
+                                                        const int64_t* n_kept, HaloAcc* acc,
                                                         uint32_t* __restrict__ keep2) {
     pdl_wait();
     const uint32_t ns = *n_seeds;
@@ -785,9 +785,9 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_keep(const uint32_t* __restr
 // groups' accumulators (1.47 ms per scale for 2^24 particles); a CTA first
 // folds kUbSumItems particles per thread in a shared table.
 constexpr int kUbSumItems = 8;
-__global__ void __launch_bounds__(kThreads) k_ms_ub_sums(DepArgs a, const int32_t* __restrict__ pslot,
-                                                        const int32_t* __restrict__ bound,
-                                                        const int32_t* __restrict__ seed_list, HaloAcc* acc) {
+__global__ void __launch_bounds__(kThreads) k_ms_ub_sums(DepArgs a, const int32_t* pslot,
+                                                        const int32_t* bound,
+                                                        const int32_t* seed_list, HaloAcc* acc) {
     pdl_wait();
     __shared__ uint32_t tkey[kTab], tcnt[kTab], tused[kTab], t_lo[4][kTab], t_hi[4][kTab];  // mass, moments
     __shared__ uint32_t n_used;
@@ -853,9 +853,9 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_sums(DepArgs a, const int32_
 
 // Particles without a halo id whose group was kept take the halo's id (with
 // the self-boundness check: only the members that stayed).
-__global__ void __launch_bounds__(kThreads) k_ms_ids(const int32_t* __restrict__ pslot, int64_t np,
-                                                    const int32_t* __restrict__ slot_halo,
-                                                    const int32_t* __restrict__ bound, int32_t* __restrict__ halo_id) {
+__global__ void __launch_bounds__(kThreads) k_ms_ids(const int32_t* pslot, int64_t np,
+                                                    const int32_t* slot_halo,
+                                                    const int32_t* bound, int32_t* __restrict__ halo_id) {
     pdl_wait();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_ids(const int32_t* __restrict__
 
 // The running halo count after a scale: n_halo += kept groups; more halos
 // than cat_cap is reported as CWTHF_E_CAPACITY (the count is still exact).
-__global__ void k_ms_advance(const uint32_t* __restrict__ keep_off, const uint32_t* __restrict__ n_seeds,
+__global__ void k_ms_advance(const uint32_t* keep_off, const uint32_t* n_seeds,
                              int64_t* __restrict__ n_halo, int64_t cat_cap, int* status) {
     pdl_wait();
     const int64_t n = *n_halo + int64_t(keep_off[*n_seeds]);

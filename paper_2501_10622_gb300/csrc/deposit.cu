@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kCountThreads) k_dep_merge(uint32_t* __restric
 }
 template <int N>
 __global__ void __launch_bounds__(kCountThreads) k_dep_starts(uint32_t* __restrict__ counters, uint32_t nkeys,
-                                                             const uint32_t* __restrict__ off) {
+                                                             const uint32_t* off) {
     pdl_wait();
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nkeys; k += gridDim.x * blockDim.x) {
         const uint32_t o = off[k];
@@ -214,10 +214,10 @@ struct TileParts {
 };
 
 template <bool kParts, bool kMass>
-__global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepArgs a, const uint32_t* __restrict__ off,
-                                                          const unsigned long long* __restrict__ rec,
-                                                          const uint32_t* __restrict__ rec_mq,
-                                                          const unsigned long long* __restrict__ mtot,
+__global__ void __launch_bounds__(kTileThreads, kTileCtasPerSm) k_dep_tile(DepArgs a, const uint32_t* off,
+                                                          const unsigned long long* rec,
+                                                          const uint32_t* rec_mq,
+                                                          const unsigned long long* mtot,
                                                           int64_t* __restrict__ grid, int* status, TileParts tp) {
     pdl_wait();
     constexpr int kCells = kDepTX * kDepTY * kDepTZ;

@@ -703,7 +703,7 @@ __device__ __forceinline__ unsigned long long row_mean(unsigned long long s, uns
 // Bound by DRAM and the latency of a tile's phases (1024^3: 12.9 GB in 3.0 ms);
 // 64-bit conversions and a 64-bit divide per row took another 6 %.
 template <class F>
-__global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_fwd(XArgs a, const int64_t* __restrict__ grid,
+__global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_fwd(XArgs a, const int64_t* grid,
                                                                           float2* __restrict__ spec) {
     pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -794,7 +794,7 @@ __global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_fwd(XArgs 
 }
 
 template <class F>
-__global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_inv(XArgs a, const float2* __restrict__ spec,
+__global__ void __launch_bounds__(F::kThreads, F::kMinBlocks) k_fft_x_inv(XArgs a, const float2* spec,
                                                                           float* __restrict__ cwt) {
     pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];

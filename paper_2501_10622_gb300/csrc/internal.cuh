@@ -229,7 +229,11 @@ struct cwthf_ctx {
 namespace cwthf {
 
 // First statement of every kernel (see PdlLaunch): waits for the kernel before
-// it in the stream, then allows the next one's blocks to be scheduled.
+// it in the stream, then allows the next one's blocks to be scheduled.  What
+// that kernel wrote changes while this one is resident, so no kernel declares
+// an input `const ... __restrict__`: the compiler may take such data as constant
+// from the kernel's first instruction to its last (loads moved above the wait,
+// or through a path that expects no writes).
 __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

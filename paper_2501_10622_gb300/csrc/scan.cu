@@ -58,7 +58,7 @@ __device__ __forceinline__ uint32_t scan_value(uint32_t w) {
 }
 
 template <bool kPopc>
-__global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t* __restrict__ in, int64_t n,
+__global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t* in, int64_t n,
                                                              const uint32_t* d_n, uint32_t* __restrict__ sums) {
     pdl_wait();
     int64_t len = scan_len(n, d_n);
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* sums, int6
 
 template <bool kPopc>
 __global__ void __launch_bounds__(kScanThreads) k_scan_add(const uint32_t* in, int64_t n, const uint32_t* d_n,
-                                                           const uint32_t* __restrict__ sums, int64_t nblocks_cap,
+                                                           const uint32_t* sums, int64_t nblocks_cap,
                                                            uint32_t* out) {
     pdl_wait();
     int64_t len = scan_len(n, d_n);

@@ -426,7 +426,7 @@ __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, flo
     }
 }
 
-__global__ void __launch_bounds__(kSegThreads, 4) k_seg_tile(const float* __restrict__ C, int ng, float cwt_min,
+__global__ void __launch_bounds__(kSegThreads, 4) k_seg_tile(const float* C, int ng, float cwt_min,
                                                              int32_t* __restrict__ label,
                                                              uint32_t* __restrict__ seed_bits,
                                                              uint32_t* __restrict__ seed_cells,
@@ -513,7 +513,7 @@ __device__ __forceinline__ void resolve_batch(int32_t* __restrict__ label, bool 
 }
 
 __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __restrict__ label, int ng,
-                                                                 const uint32_t* __restrict__ ballots,
+                                                                 const uint32_t* ballots,
                                                                  uint32_t* __restrict__ seed_cells,
                                                                  int* __restrict__ changed,
                                                                  unsigned* __restrict__ next_rows, int limit,
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kResolveThreads) k_seg_resolve(int32_t* __rest
 // the last round is reported as CWTHF_E_NOT_CONVERGED (the labels are then
 // unspecified, and flagged values are skipped by the recount).
 __global__ void __launch_bounds__(256) k_seg_fallback(int32_t* __restrict__ label, int64_t cells, int* changed,
-                                                      int rounds, const uint32_t* __restrict__ bits,
+                                                      int rounds, const uint32_t* bits,
                                                       uint32_t* __restrict__ seed_cells, unsigned* bar, int* status) {
     pdl_wait();
     if (*reinterpret_cast<volatile int*>(&changed[0]) == 0) return;  // the same answer in every CTA
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(256) k_seg_fallback(int32_t* __restrict__ labe
 // slot -> seed cell, in increasing cell order.  *n_slots = number of seeds,
 // clamped to slot_cap (more seeds than that can only come from an inconsistent
 // label grid, reported as bad input).
-__global__ void k_seed_list(const uint32_t* __restrict__ bits, const uint32_t* __restrict__ prefix, int64_t nwords,
+__global__ void k_seed_list(const uint32_t* bits, const uint32_t* prefix, int64_t nwords,
                             int64_t slot_cap, int32_t* __restrict__ seed_list, uint32_t* __restrict__ n_slots,
                             int* status) {
     pdl_wait();
@@ -672,8 +672,8 @@ __global__ void k_seed_list(const uint32_t* __restrict__ bits, const uint32_t* _
 // loop over the bitmap, each seed's gather and 48 bytes of
 // stores waited for the seed before it in the same word (0.68 ms per scale at
 // 1024^3, 0.14 + 0.40 now).
-__global__ void k_seed_acc(const int32_t* __restrict__ seed_list, const uint32_t* __restrict__ seed_cells,
-                           HaloAcc* __restrict__ acc, const uint32_t* __restrict__ n_slots) {
+__global__ void k_seed_acc(const int32_t* seed_list, const uint32_t* seed_cells,
+                           HaloAcc* __restrict__ acc, const uint32_t* n_slots) {
     pdl_wait();
     // an accumulator is three 16-byte pieces, all zero but the count in the last one's upper half; one
     // thread per piece, so that a warp's stores are contiguous
@@ -687,20 +687,27 @@ __global__ void k_seed_acc(const int32_t* __restrict__ seed_list, const uint32_t
 }
 
 // Seeds from a label grid: the cells labelled with their own index.
-__global__ void k_seeds_from_labels(const int32_t* __restrict__ label, int64_t cells, uint32_t* __restrict__ bits,
+__global__ void k_seeds_from_labels(const int32_t* label, int64_t cells, uint32_t* __restrict__ bits,
                                     int* status) {
     pdl_wait();
-    int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < cells; c += stride) {
-        int32_t l = label[c];
-        if (l < -1 || l >= cells) set_status(status, CWTHF_E_BAD_INPUT);
-        if (l == c) atomicOr(&bits[c >> 5], 1u << (c & 31));
+    constexpr int kIlp = 4;  // labels in flight (one at a time: 256^3 37 us, 28 with four)
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t c0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c0 < cells; c0 += kIlp * stride) {
+        int32_t l[kIlp];
+#pragma unroll
+        for (int u = 0; u < kIlp; u++) l[u] = c0 + u * stride < cells ? label[c0 + u * stride] : -1;
+#pragma unroll
+        for (int u = 0; u < kIlp; u++) {
+            const int64_t c = c0 + u * stride;
+            if (l[u] < -1 || l[u] >= cells) set_status(status, CWTHF_E_BAD_INPUT);
+            if (l[u] == c) atomicOr(&bits[c >> 5], 1u << (c & 31));
+        }
     }
 }
 
 // Seeds of the last segmentation and their segments' cell counts.
-__global__ void k_segment_sizes(const int32_t* __restrict__ seed_list, const HaloAcc* __restrict__ acc,
-                                const uint32_t* __restrict__ n_slots, int64_t cap, int32_t* __restrict__ seeds,
+__global__ void k_segment_sizes(const int32_t* seed_list, const HaloAcc* acc,
+                                const uint32_t* n_slots, int64_t cap, int32_t* __restrict__ seeds,
                                 int64_t* __restrict__ n_cells, int64_t* __restrict__ n_out) {
     pdl_wait();
     const int64_t ns = *n_slots;

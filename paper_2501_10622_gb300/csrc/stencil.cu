@@ -46,7 +46,7 @@ __host__ __device__ constexpr int x_pitch_r(int ng, int RC) { return (ng + 2 * R
 // x pass: one warp per row, staged in shared memory with RC wrapped cells on
 // each side; each lane forms A and B for four neighbouring columns.
 template <int RC>
-__global__ void __launch_bounds__(32 * kXWarps) k_sten_x_reg(const int64_t* __restrict__ grid, int ng, StencilTaps t,
+__global__ void __launch_bounds__(32 * kXWarps) k_sten_x_reg(const int64_t* grid, int ng, StencilTaps t,
                                                              float* __restrict__ A, float* __restrict__ B) {
     pdl_wait();
     extern __shared__ __align__(16) float rows[];  // [kXWarps][pitch]
@@ -114,8 +114,8 @@ constexpr int kLineThreads = 256;
 constexpr int kOut = kLine / (kLineThreads / 32);  // 8
 
 template <bool kZ, int RC>
-__global__ void __launch_bounds__(kLineThreads) k_sten_yz_reg(const float* __restrict__ in0,
-                                                             const float* __restrict__ in1, int ng, StencilTaps t,
+__global__ void __launch_bounds__(kLineThreads) k_sten_yz_reg(const float* in0,
+                                                             const float* in1, int ng, StencilTaps t,
                                                              float scale, float* __restrict__ out0,
                                                              float* __restrict__ out1) {
     pdl_wait();
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kLineThreads) k_sten_yz_reg(const float* __res
 // x pass: one warp per row of the grid.  The row (with R wrapped cells on each
 // side) is staged in shared memory; each lane then forms A and B for the
 // columns lane, lane + 32, ...
-__global__ void __launch_bounds__(32 * kXWarps) k_sten_x(const int64_t* __restrict__ grid, int ng, StencilTaps t,
+__global__ void __launch_bounds__(32 * kXWarps) k_sten_x(const int64_t* grid, int ng, StencilTaps t,
                                                          float* __restrict__ A, float* __restrict__ B) {
     pdl_wait();
     extern __shared__ float rows[];  // [kXWarps][ng + 2R]
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(32 * kXWarps) k_sten_x(const int64_t* __restri
 // y and z passes: as above, each output's taps read from shared memory.
 
 template <bool kZ>
-__global__ void __launch_bounds__(kLineThreads) k_sten_yz(const float* __restrict__ in0, const float* __restrict__ in1,
+__global__ void __launch_bounds__(kLineThreads) k_sten_yz(const float* in0, const float* in1,
                                                          int ng, StencilTaps t, float scale,
                                                          float* __restrict__ out0, float* __restrict__ out1) {
     pdl_wait();

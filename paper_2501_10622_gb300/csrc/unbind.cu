@@ -52,10 +52,10 @@ __device__ __forceinline__ bool big_team_group(uint32_t n) { return n > uint32_t
 // counter (2^24 particles: 0.60 ms per pass with an atomic each).
 constexpr int kBinThreads = 256, kBinItems = 8;
 template <bool kScatter>
-__global__ void __launch_bounds__(kBinThreads) k_ub_bin(const float* __restrict__ mass, double mass_unit,
-                                                        const int32_t* __restrict__ group, int64_t np,
-                                                        int64_t n_groups, const uint32_t* __restrict__ d_groups,
-                                                        const uint32_t* __restrict__ off,
+__global__ void __launch_bounds__(kBinThreads) k_ub_bin(const float* mass, double mass_unit,
+                                                        const int32_t* group, int64_t np,
+                                                        int64_t n_groups, const uint32_t* d_groups,
+                                                        const uint32_t* off,
                                                         uint32_t* __restrict__ counter, int32_t* __restrict__ mem,
                                                         int32_t* __restrict__ group_out, int* status) {
     pdl_wait();
