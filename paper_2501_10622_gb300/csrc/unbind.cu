@@ -23,6 +23,7 @@
 #include <cmath>
 
 #include "internal.cuh"
+#include "unbind_teams.cuh"
 
 namespace cwthf {
 namespace {
@@ -754,7 +755,7 @@ __global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
         if (!unbind_group_grid(a, b, g, shd, shi, hist, dsum, dbase, &skip, parity)) return;
     }
     for (int big = 1; big >= 0; big--) {
-        const int size = big ? kUnbindBigTeam : kUnbindTeam;
+        const int size = ub_team_ctas(big ? kUnbindBigTeam : kUnbindTeam, int(gridDim.x));
         const int team = int(blockIdx.x) / size, first = team * size;
         if (first + size > int(gridDim.x)) continue;  // a rest too small for a team
         UbGrid tm;
