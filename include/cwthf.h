@@ -400,9 +400,9 @@ CWTHF_API int cwthf_set_fft_plan(cwthf_ctx *ctx, int ng, int which, int C, const
  *       CWTHF_E_INDEX), else 0.
  *   CWTHF_DEBUG_UNBIND_GRID_MIN  1..2^31-1 (default 65536): groups of the
  *       self-boundness check with more members than this are processed by the
- *       whole grid, one at a time, or (65,537 .. 2^20 members) by a team of
- *       CTAs; smaller ones by one CTA or a smaller team.  All give the same
- *       decisions up to rounding.
+ *       whole grid, one at a time, or (65,537 .. 2^20 members) by teams of 128
+ *       or 64 CTAs; smaller ones by one CTA or a team of up to eight.  All give
+ *       the same decisions up to rounding.
  * cwthf_debug_set returns CWTHF_E_INVALID_ARG for an unknown key or a value
  * out of range; settings persist for the context's lifetime. */
 #define CWTHF_DEBUG_JUMP_ROUNDS 1

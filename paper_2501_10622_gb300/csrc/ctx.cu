@@ -110,8 +110,8 @@ void for_each_buffer(cwthf_ctx* c, int max_ng, int64_t max_np, int max_scales, u
         f(reinterpret_cast<void**>(&c->ub_keep), size_t(z.slots + 2) * 4);
         f(reinterpret_cast<void**>(&c->ub_ngroups), 16);
         // groups of several CTAs: per-CTA partial sums and digit counts, barriers
-        f(reinterpret_cast<void**>(&c->ub_part), size_t(kUnbindGridCtaCap) * 16 * 8);
-        f(reinterpret_cast<void**>(&c->ub_hist), size_t(kUnbindGridCtaCap) * 2 * 256 * 4);
+        f(reinterpret_cast<void**>(&c->ub_part), size_t(kUbCtaCap) * 16 * 8);
+        f(reinterpret_cast<void**>(&c->ub_hist), size_t(kUbCtaCap) * 2 * 256 * 4);
         f(reinterpret_cast<void**>(&c->ub_bar), kUbBarWords * 4);
     }
     f(reinterpret_cast<void**>(&c->scan_tmp), z.scan_words * 4);
@@ -209,7 +209,7 @@ int cwthf_create_ex(int device, int max_ng, int64_t max_np, int max_scales, unsi
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         (c->fallback_blocks = fallback_blocks(c->sm_count)) <= 0 ||
         ((flags & CWTHF_CREATE_UNBIND) &&
-         (c->ub_grid_blocks = std::min(unbind_grid_blocks(c->sm_count), kUnbindGridCtaCap)) <= 0)) {
+         (c->ub_grid_blocks = std::min(unbind_grid_blocks(c->sm_count), kUbCtaCap)) <= 0)) {
         delete c;
         return CWTHF_E_CUDA;
     }

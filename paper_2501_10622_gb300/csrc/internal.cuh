@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/cwthf.h"
+#include "unbind_teams.cuh"
 
 namespace cwthf {
 
@@ -59,16 +60,14 @@ constexpr int kDefaultChaseLimit = 64;
 
 // Groups of the self-boundness check with more members than this are
 // processed by the whole grid, one at a time, or by big teams of CTAs.
-constexpr int64_t kUnbindGridMin = 1 << 16;
-// Most CTAs of the launch for groups of several CTAs (its per-CTA scratch is
-// sized for them); its control words: the whole grid's barrier (2), the counts
-// of medium and large groups, the next of either for the teams, and from
-// kUbTeamWords on four words per team (barrier, next group): the teams of
-// kUnbindTeam CTAs, then the bigger ones of kUnbindBigTeam.
-constexpr int kUnbindGridCtaCap = 1024, kUnbindTeam = 8, kUnbindBigTeam = 64;
-constexpr int kUbMedium = 2, kUbLarge = 3, kUbNext = 4, kUbNextBig = 5, kUbTeamWords = 8;
-constexpr size_t kUbBarWords =
-    kUbTeamWords + 4 * (kUnbindGridCtaCap / kUnbindTeam + kUnbindGridCtaCap / kUnbindBigTeam);
+constexpr int64_t kUnbindGridMin = kUbBigMin;
+// Control words of the launch for groups of several CTAs: the counts of medium
+// and large groups, the members of all medium and of all big ones (64 bits
+// each), the next group of every way of sharing, and from kUbTeamWords on four
+// words per team (barrier, next group).
+constexpr int kUbMedium = 0, kUbLarge = 1, kUbMembers = 2, kUbBigMembers = 4, kUbNext = 6, kUbTeamWords = 16;
+static_assert(kUbNext + kUbWays <= kUbTeamWords, "control words");
+constexpr size_t kUbBarWords = kUbTeamWords + 4 * size_t(ub_first_team(kUbWays));
 
 // A bounded device wait gives up after this many polls.
 constexpr long long kSpinLimit = 1ll << 20;

@@ -23,26 +23,13 @@
 #include <cmath>
 
 #include "internal.cuh"
-#include "unbind_teams.cuh"
 
 namespace cwthf {
 namespace {
 
+using u64 = unsigned long long;
 constexpr int kUbThreads = 512;
 constexpr int kUbWarps = kUbThreads / 32;
-// Groups up to this size take one CTA (and sort in shared memory), larger ones
-// a team of kUnbindTeam CTAs (up to the whole-grid threshold): a CTA alone
-// worked 10 ms on a group of 60,000 members while the rest of the GPU had long
-// finished.
-constexpr int kUbCtaMax = 2048;
-// Groups above the whole-grid threshold but within these sizes take a team of
-// kUnbindBigTeam CTAs: several at a time, and with cheaper barriers, than one
-// after another with every CTA.  Six scales of the paper's box on 2^24
-// particles: groups of one CTA 63 ms and of the whole grid 29 ms before; 8.3 +
-// 30 ms with teams of 8 and 32 and one CTA up to 4096 members, 6.0 + 28 with 8
-// and 64 and up to 2048 (teams of 4, 16 or 32, or of 16, 96 or 128, are slower).
-constexpr int kUbBigMin = int(kUnbindGridMin), kUbBigMax = 1 << 20;
-__device__ __forceinline__ bool big_team_group(uint32_t n) { return n > uint32_t(kUbBigMin) && n <= uint32_t(kUbBigMax); }
 
 // Counting sort of the particles by group, in two passes of one form: count
 // (kScatter false, which also clears group_out and checks the masses), then,
@@ -133,9 +120,9 @@ struct UbArgs {
                           // pairs and the radix sort's other buffer)
     int32_t* val;         // [2 np] sort values (the same layout)
     int max_iter;
-    int64_t grid_min;            // larger groups are left to the whole-grid path
-    uint32_t* list;              // [list_cap] groups of the team path from the front, of the whole-grid path
-    int64_t list_cap;            // from the back
+    int64_t grid_min;            // groups above it are large
+    uint32_t* list;              // [list_cap] medium groups from the front, large ones from the back
+    int64_t list_cap;
     unsigned* ctl;               // control words (kUbMedium, ...)
     int64_t n_groups;            // groups (or read from d_groups when given)
     const uint32_t* d_groups;
@@ -285,8 +272,13 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
     const int tid = threadIdx.x;
     if (int64_t(n0) > a.grid_min || n0 > kUbCtaMax) {  // left to the whole grid, or to a team of CTAs
         if (tid == 0) {
-            if (int64_t(n0) > a.grid_min) a.list[a.list_cap - 1 - int64_t(atomicAdd(a.ctl + kUbLarge, 1u))] = uint32_t(g);
-            else a.list[atomicAdd(a.ctl + kUbMedium, 1u)] = uint32_t(g);
+            if (int64_t(n0) > a.grid_min) {
+                a.list[a.list_cap - 1 - int64_t(atomicAdd(a.ctl + kUbLarge, 1u))] = uint32_t(g);
+                if (ub_big(n0)) atomicAdd(reinterpret_cast<u64*>(a.ctl + kUbBigMembers), u64(n0));
+            } else {
+                a.list[atomicAdd(a.ctl + kUbMedium, 1u)] = uint32_t(g);
+                atomicAdd(reinterpret_cast<u64*>(a.ctl + kUbMembers), u64(n0));
+            }
         }
         return;
     }
@@ -414,9 +406,8 @@ __device__ void unbind_group(const UbArgs& a, int64_t g, uint64_t* sk, int32_t* 
 
 // ---- several CTAs per group ---------------------------------------------------
 //
-// The largest groups one at a time with every CTA of the grid, then large ones
-// with teams of kUnbindBigTeam CTAs and medium ones with teams of kUnbindTeam,
-// each team taking the next group when it is done.
+// Each group is shared by a team of CTAs, or by all of them (unbind_teams.cuh
+// has the rule); a team takes the next group of its size when it is done.
 // The same steps as unbind_group, with each CTA owning a contiguous chunk of
 // the group's members and grid barriers between the phases.  Partial sums go
 // through per-CTA slots and are combined in CTA order by every CTA, so the
@@ -434,7 +425,11 @@ struct UbGrid {      // the grid, or one team of it
     int size, rank;  // CTAs that work together, this CTA's place among them
 };
 
-__device__ __forceinline__ bool team_sync(const UbGrid& b) { return grid_sync(b.bar, b.status, unsigned(b.size)); }
+__device__ __forceinline__ bool team_sync(const UbGrid& b) {
+    if (b.size > 1) return grid_sync(b.bar, b.status, unsigned(b.size));
+    __syncthreads();
+    return true;
+}
 
 // [b, e) of the CTA's chunk of n members
 __device__ __forceinline__ void cta_chunk(const UbGrid& tm, int n, int& b, int& e) {
@@ -561,7 +556,7 @@ __device__ bool grid_radix(uint64_t* K, int32_t* V, int n, int byte0, int byte1,
     return true;
 }
 
-// One group with every CTA of the grid.  Returns false on a barrier timeout.
+// One group with every CTA of a team.  Returns false on a barrier timeout.
 __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, double* shd, int64_t* shi,
                                   uint32_t* hist, uint32_t* dsum, uint32_t* dbase, int* skip, int& parity) {
     __shared__ double bc[8];
@@ -733,11 +728,9 @@ __device__ bool unbind_group_grid(const UbArgs& a, const UbGrid& b, int64_t g, d
     return team_sync(b);
 }
 
-// The listed groups above a.grid_min, one after another with the whole grid
-// (those of a big team's size left out), then the teams' groups (a cooperative
-// launch: every CTA resident).  A barrier that runs out ends the kernel with
-// CWTHF_E_TIMEOUT.  A team's scratch is that of its CTAs, so teams of either
-// size never share any.
+// The listed groups, way by way (a cooperative launch: every CTA resident).  A
+// barrier that runs out ends the kernel with CWTHF_E_TIMEOUT.  A team's scratch
+// is that of its CTAs, so teams never share any.
 __global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
     pdl_wait();
     __shared__ double shd[8 * kUbWarps];
@@ -745,37 +738,57 @@ __global__ void __launch_bounds__(kUbThreads, 2) k_ub_grid(UbArgs a, UbGrid b) {
     __shared__ uint32_t hist[kUbWarps * 256];
     __shared__ uint32_t dsum[256], dbase[256];
     __shared__ int skip;
-    b.size = int(gridDim.x);
-    b.rank = int(blockIdx.x);
-    const unsigned n_large = a.ctl[kUbLarge], n_medium = a.ctl[kUbMedium];  // counted by k_ub_group
-    int parity = 0;
-    for (unsigned i = 0; i < n_large; i++) {
-        const uint32_t g = a.list[a.list_cap - 1 - int64_t(i)];
-        if (big_team_group(a.off[g + 1] - a.off[g])) continue;
-        if (!unbind_group_grid(a, b, g, shd, shi, hist, dsum, dbase, &skip, parity)) return;
-    }
-    for (int big = 1; big >= 0; big--) {
-        const int size = ub_team_ctas(big ? kUnbindBigTeam : kUnbindTeam, int(gridDim.x));
+    __shared__ unsigned ways;
+    const int ctas = int(gridDim.x);
+    // counted by k_ub_group
+    const unsigned n_large = a.ctl[kUbLarge], n_medium = a.ctl[kUbMedium];
+    auto group = [&](bool from_large, unsigned i) { return a.list[from_large ? a.list_cap - 1 - int64_t(i) : int64_t(i)]; };
+    auto way_of = [&](bool from_large, unsigned i) {
+        const uint32_t g = group(from_large, i);
+        const long long n = (long long)(a.off[g + 1] - a.off[g]);
+        if (from_large && !ub_big(n)) return kUbWhole;
+        const u64 total = *reinterpret_cast<const u64*>(a.ctl + (from_large ? kUbBigMembers : kUbMembers));
+        return from_large ? ub_big_way(n, (long long)total, ctas) : ub_medium_way(n, (long long)total, ctas);
+    };
+    // the ways that occur (the same in every CTA)
+    if (threadIdx.x == 0) ways = 0u;
+    __syncthreads();
+    unsigned mine = 0;
+    for (unsigned i = threadIdx.x; i < n_large; i += blockDim.x) mine |= 1u << way_of(true, i);
+    for (unsigned i = threadIdx.x; i < n_medium; i += blockDim.x) mine |= 1u << way_of(false, i);
+    if (mine) atomicOr(&ways, mine);
+    __syncthreads();
+    for (int way = 0; way < kUbWays; way++) {
+        if (!(ways & (1u << way))) continue;
+        const bool from_large = way < kUbMediumWays;
+        const int size = ub_team_ctas(ub_team_size(way), ctas);
         const int team = int(blockIdx.x) / size, first = team * size;
-        if (first + size > int(gridDim.x)) continue;  // a rest too small for a team
+        if (first + size > ctas) continue;  // a rest too small for a team
         UbGrid tm;
         tm.part = b.part + size_t(first) * kUbPart;
         tm.hist = b.hist + size_t(first) * 2 * 256;
-        unsigned* words = b.bar + kUbTeamWords + 4 * (team + (big ? kUnbindGridCtaCap / kUnbindTeam : 0));
-        tm.bar = words;
+        tm.bar = b.bar + kUbTeamWords + 4 * (ub_first_team(way) + team);
         tm.status = b.status;
         tm.size = size;
         tm.rank = int(blockIdx.x) - first;
-        parity = 0;
+        int parity = 0;
+        // The last teams pick first, over some 8 us: a launch's first eight CTAs sit on four SMs, two by two, the
+        // others alone until every SM has one.  (One group of 40,000 members: 5.5 ms on CTAs 0 to 7, 3.2 ms on the
+        // last eight; one of 2^20: 10.6 ms on CTAs 0 to 127, 7.6 ms on the next 128.)
+        const int teams = ctas / size;
+        if (tm.rank == 0 && threadIdx.x == 0) __nanosleep(8192u * unsigned(teams - 1 - team) / unsigned(teams));
         for (;;) {
-            if (tm.rank == 0 && threadIdx.x == 0) __stcg(words + 2, atomicAdd(a.ctl + (big ? kUbNextBig : kUbNext), 1u));
+            const unsigned n = from_large ? n_large : n_medium;
+            if (tm.rank == 0 && threadIdx.x == 0) {  // the next group of this way
+                unsigned i = atomicAdd(a.ctl + kUbNext + way, 1u);
+                while (i < n && way_of(from_large, i) != way) i = atomicAdd(a.ctl + kUbNext + way, 1u);
+                __stcg(tm.bar + 2, i);
+            }
             if (!team_sync(tm)) return;
-            const unsigned i = __ldcg(words + 2);
+            const unsigned i = __ldcg(tm.bar + 2);
             if (!team_sync(tm)) return;  // every CTA has read the number before the next one is written
-            if (i >= (big ? n_large : n_medium)) break;  // the same in the whole team
-            const uint32_t g = big ? a.list[a.list_cap - 1 - int64_t(i)] : a.list[i];
-            if (big && !big_team_group(a.off[g + 1] - a.off[g])) continue;  // done by the whole grid
-            if (!unbind_group_grid(a, tm, g, shd, shi, hist, dsum, dbase, &skip, parity)) return;
+            if (i >= n) break;           // the same in the whole team
+            if (!unbind_group_grid(a, tm, group(from_large, i), shd, shi, hist, dsum, dbase, &skip, parity)) return;
         }
     }
 }
