@@ -384,8 +384,8 @@ bool plan_from(int L, int which, int C, const int* rad, int nst, Plan& p) {
     return box;
 }
 
-// The plan a pass of this context uses: the caller's (run-time kernels), else
-// the built-in one.
+// The plan a pass of this context uses: the caller's (on the run-time kernels,
+// unless it is the built-in one), else the built-in one.
 bool pass_plan(cwthf_ctx* ctx, int ng, int which, PassPlan& p) {
     {
         std::lock_guard<std::mutex> g(ctx->table_mu);

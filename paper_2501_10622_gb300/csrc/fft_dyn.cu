@@ -1,8 +1,8 @@
 // fft_dyn.cu -- the run-time FFT pass kernels, for the plans a caller sets
 // (cwthf_set_fft_plan: any radix order and tile width).  One butterfly per
 // thread and stage, each radix's stage a function of its own; the built-in
-// plans run compile-time instances instead (fft_ct.cuh), which take a third
-// to a tenth of the time.
+// plans, also when a caller sets one, run compile-time instances instead
+// (fft_ct.cuh), which take a third to a tenth of the time.
 #include "fft.cuh"
 
 namespace cwthf {
