@@ -464,10 +464,12 @@ struct CtFft {
     static constexpr int kThreads = T_, kMinBlocks = kShape.blocks;
     static constexpr bool kBlue = kBlue_;
     static constexpr int kMaxLen = kBlue_ ? (L_ + 1) / 2 : L_;  // the longest pass
-    // the x passes' row loops take the length as a literal only here: with a literal the
-    // compiler merges their branches for some lengths and not for others and then contracts
-    // the products differently, so the last bit would depend on the length's parity
-    static constexpr bool kLiteral = !kBlue_ && (L_ == 256 || L_ == 512);
+    // The x passes' row loops take the length as a literal for powers of two from 256 on, else at
+    // run time.  The compiler contracts their products in another order with a literal, for some
+    // lengths, so either choice is one of a length's last bits, on which near ties of the
+    // segmentation hang; each length keeps the choice its results were made with.  In time: 1024^3
+    // 10.52 ms with the literal, 11.07 without; 512^3 1.25 and 1.24; 640^3 (and others) the same.
+    static constexpr bool kLiteral = !kBlue_ && L_ >= 256 && (L_ & (L_ - 1)) == 0;
     static_assert(N_ >= 1 && R0 * R1 * R2 == L_, "radices multiply to the length");
     static_assert(!kBlue_ || N_ >= 2, "a Bluestein plan has two or three stages");
     static __device__ __forceinline__ int cols(const Plan&) { return C_; }
