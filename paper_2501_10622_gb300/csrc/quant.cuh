@@ -112,12 +112,24 @@ __device__ __forceinline__ bool quantise(float x, uint32_t sm, int se, int64_t m
     return quantise_any(x, sm, se, modulus, q);
 }
 
+// Whether rint(RN(m / u)) is n + 1 rather than n, for a quotient within 2^-8 of
+// h = n + 1/2 (RN: rounded to fp64, as the division rounds).  RN(m / u) is h
+// itself for quotients within half a unit of h's last place, 2^(k - 53) with
+// 2^k <= h, of it, and a half rounds to even.  m - h u is a multiple of half of
+// u's last place, fewer than 2^47 of them, so the fused product is exact.
+__device__ __forceinline__ bool half_rounds_up(float m, double u, uint32_t n) {
+    const double r = __fma_rn(-(double(n) + 0.5), u, double(m));
+    const double lim = __dmul_rn(u, __hiloint2double((1023 + (31 - __clz(n)) - 53) << 20, 0));
+    return (n & 1u) ? r >= -lim : r > lim;
+}
+
 // Integer mass of particle i: 1 when masses are equal, else rint(m / mass_unit)
 // (round half to even).  The fp64 quotient is formed only where it decides: m
 // times the reciprocal's leading 40 bits, as an integer product, differs from
 // the rounded quotient by at most 2^31 (2^-40 + 2 2^-53) < 2^-9 + 2^-20
 // (quotients below 2^31), so a fraction 5 2^-11 or more from one half rounds the
-// same way.  (fp64 units are scarce: the division alone took over half of a
+// same way; a fraction nearer to one half is decided by the sign of m - (n + 1/2)
+// mass_unit.  (fp64 units are scarce: the division alone took over half of a
 // binning pass's time with masses, 0.22 ms for 2^23 particles.)  Returns
 // CWTHF_OK, CWTHF_E_BAD_INPUT (negative / NaN) or CWTHF_E_OVERFLOW (>= 2^31).
 __device__ __forceinline__ int mass_quantum(const DepArgs& a, int64_t i, uint32_t& mq) {
@@ -130,8 +142,9 @@ __device__ __forceinline__ int mass_quantum(const DepArgs& a, int64_t i, uint32_
         const unsigned long long P = (unsigned long long)((b & 0x7fffffu) | 0x800000u) * a.inv_m;
         const unsigned long long n = P >> sh;
         const int f = int((P >> (sh - 11u)) & 2047u) - 1024;  // fraction minus one half, in 2^-11
-        if (n < 0x7ffffff0ull && (f >= 5 || f < -5)) {
-            mq = uint32_t(n) + (f > 0 ? 1u : 0u);
+        if (n < 0x7ffffff0ull) {
+            const bool up = f >= 5 || f < -5 ? f > 0 : half_rounds_up(m, a.mass_unit, uint32_t(n));
+            mq = uint32_t(n) + (up ? 1u : 0u);
             return CWTHF_OK;
         }
     }

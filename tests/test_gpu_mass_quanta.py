@@ -53,3 +53,20 @@ def test_quanta_about_halves(ctx, unit, top):
     want = np.rint(mass.astype(np.float64) / unit)
     assert want.sum() < 2 ** 33
     np.testing.assert_array_equal(_quanta(ctx, mass, unit), want.astype(np.int64))
+
+
+def test_quotients_that_round_to_a_half(ctx):
+    # units such that the fp64 quotient is a half, or a few units of its last place beside one, while the mass is
+    # not that many units exactly
+    rng = np.random.default_rng(3)
+    halves = 0
+    for k in range(400):
+        mass = np.float32(rng.uniform(0.5, 4.0) * 2.0 ** rng.integers(-3, 28))
+        h = np.floor(rng.uniform(0.0, 2.0 ** rng.integers(0, 31))) + 0.5
+        unit = float(mass) / h
+        for _ in range(abs(k % 5 - 2)):
+            unit = float(np.nextafter(unit, 0.0 if k % 5 < 2 else np.inf))
+        q = float(mass) / unit
+        halves += q == h
+        assert _quanta(ctx, np.array([mass]), unit)[0] == np.rint(q), (float(mass), unit.hex())
+    assert 50 < halves < 350  # both kinds occur
