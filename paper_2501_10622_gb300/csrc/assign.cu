@@ -133,7 +133,8 @@ __device__ __forceinline__ u64 sext(uint32_t v) { return u64((long long)int32_t(
 __device__ __forceinline__ u64 sext(int32_t v) { return u64((long long)v); }
 
 template <bool kMass>
-__global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_sums(DepArgs a, FastDiv divn, const uint32_t* total_ptr,
+__global__ void __launch_bounds__(kHsThreads, hs_ctas_per_sm<kMass>()) k_halo_sums(DepArgs a, FastDiv divn,
+                                                       const uint32_t* total_ptr,
                                                        const unsigned long long* rec,
                                                        const uint32_t* rec_mq,
                                                        const int32_t* label,
@@ -325,16 +326,17 @@ void launch_halo_sums(cwthf_ctx* ctx, cudaStream_t s, int64_t np, const DepArgs&
     int* st = ctx->d_status;
     const FastDiv dn = make_fastdiv(uint32_t(a.ng));
     const int64_t chunks = div_up(std::max<int64_t>(np, 1), kChunk);
+    auto blocks = [&](int per_sm) { return int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * per_sm)); };
     if (a.mass)
         CWTHF_LAUNCH(ctx, s, "k_halo_sums",
-                     pdl(k_halo_sums<true>, int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * hs_ctas_per_sm<true>())),
-                                         kHsThreads, 0, s)(a, dn, total, rec, rec_mq, label, bits, prefix, n_slots,
-                                                             acc, rec_slot, slot_stride, mtot, skip_marked, st));
+                     pdl(k_halo_sums<true>, blocks(hs_ctas_per_sm<true>()), kHsThreads, 0, s)(
+                         a, dn, total, rec, rec_mq, label, bits, prefix, n_slots, acc, rec_slot, slot_stride, mtot,
+                         skip_marked, st));
     else
         CWTHF_LAUNCH(ctx, s, "k_halo_sums",
-                     pdl(k_halo_sums<false>, int(std::min<int64_t>(chunks, int64_t(ctx->sm_count) * hs_ctas_per_sm<false>())),
-                                          kHsThreads, 0, s)(a, dn, total, rec, rec_mq, label, bits, prefix, n_slots,
-                                                              acc, rec_slot, slot_stride, mtot, skip_marked, st));
+                     pdl(k_halo_sums<false>, blocks(hs_ctas_per_sm<false>()), kHsThreads, 0, s)(
+                         a, dn, total, rec, rec_mq, label, bits, prefix, n_slots, acc, rec_slot, slot_stride, mtot,
+                         skip_marked, st));
 }
 
 struct FilterArgs {
@@ -434,14 +436,9 @@ __global__ void __launch_bounds__(kThreads) k_catalogue(const HaloAcc* acc,
 // Each scale's pass stores its record slots contiguously (rec_slot[scale * np
 // + r]: whole sectors written, none read back).  After the last scale the halo
 // ids are regrouped per record, RS ids per record (two scales: 8-byte groups;
-// more: 16-byte groups of four scales), so that the final pass
-// reads a particle's ids with one vector gather per four scales.
-__host__ __device__ __forceinline__ int slot_group_stride(int n_scales) {
-    return n_scales <= 2 ? n_scales : (n_scales + 3) & ~3;
-}
-__host__ __device__ __forceinline__ int64_t slot_groups_offset(int n_scales, int64_t np) {
-    return n_scales == 1 ? 0 : (int64_t(n_scales) * np + 3) & ~int64_t(3);
-}
+// more: 16-byte groups of four scales), so that the final pass reads a
+// particle's ids with one vector gather per four scales.  (One scale: no groups.)
+inline int64_t slot_groups_offset(int n_scales, int64_t np) { return (int64_t(n_scales) * np + 3) & ~int64_t(3); }
 
 template <int RS>
 struct IdGroup;
@@ -957,8 +954,8 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
     if (e != cudaSuccess) return cuda_status(e);
     if (!seeds_ready)  // after segment_impl the resolve pass has counted the cells already
         CWTHF_LAUNCH(ctx, s, "k_count_cells",
-                     pdl(k_count_cells, int(std::min<int64_t>(div_up(cells, kCountCells), blocks)), kThreads, 0, s)(label, cells, ctx->seed_bits, ctx->seed_prefix,
-                                                               d_nseeds, ctx->acc, ctx->d_status));
+                     pdl(k_count_cells, int(std::min<int64_t>(div_up(cells, kCountCells), blocks)), kThreads, 0, s)(
+                         label, cells, ctx->seed_bits, ctx->seed_prefix, d_nseeds, ctx->acc, ctx->d_status));
     DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
     const int64_t total_key = deposit_geom(ng).ntiles * kDepClasses;  // dep_off[total_key] = records binned
     int pblocks = int(std::min<int64_t>(div_up(std::max<int64_t>(np, 1), kThreads), int64_t(ctx->sm_count) * 16));
@@ -978,13 +975,12 @@ int assign_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mass
                                                          cat, ctx->slot_halo + int64_t(scale) * slot_cap, n_halo,
                                                          ctx->d_status));
     if (scale == n_scales - 1) {  // halo ids of all scales at once
-        const int rs = slot_group_stride(n_scales);
         const uint32_t* total = ctx->dep_off + total_key;
-        if (rs == 1)
+        if (n_scales == 1)
             CWTHF_LAUNCH(ctx, s, "k_finalize",
                          pdl(k_finalize_one, pblocks, kThreads, 0, s)(ctx->part_rec, np, total, ctx->part_slot,
                                                                      ctx->slot_halo, halo_id));
-        else if (rs == 2) launch_ids<2>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
+        else if (n_scales == 2) launch_ids<2>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
         else launch_ids<4>(ctx, s, blocks, pblocks, np, total, n_scales, slot_cap, halo_id);
     }
     return cuda_status(cudaGetLastError());

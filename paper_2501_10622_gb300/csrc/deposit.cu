@@ -67,10 +67,9 @@ __device__ __forceinline__ PartBin bin_particle(const DepArgs& a, int64_t i) {
 // The counters may come in several copies (a power of two), block b using copy
 // b mod copies in both passes: a clump's core sends a few per cent, or tens of
 // per cent, of all particles into one segment, and their atomics queue up at
-// one address (about 1 ns each): 144^3 grid, 8 particles per cell, count 495 ->
-// 249 us, scatter 604 -> 384 us; six scales of the paper's box 5.9 -> 3.1 ms.
-// copy_of: this block's copy of an array of
-// nkeys counters.
+// one address (about 1 ns each).  144^3 grid, 8 particles per cell: count 495 ->
+// 249 us, scatter 604 -> 384 us.  copy_of: this block's copy of an array of nkeys
+// counters.
 struct Copies {
     uint32_t n, nkeys;
 };
@@ -392,7 +391,7 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     DepArgs a = make_dep_args(pos, mass, mass_unit, np, L, ng);
     int64_t nkeys = g.ntiles * kDepClasses;
     // Copies of the counters: 16, as long as there are at most 2^20 counters in all (halved beyond: 320^3 8,
-    // 512^3 2, one from 640^3 on) and particles are not few.  Every copy has a part of the segment of its
+    // 512^3 2, larger grids one) and particles are not few.  Every copy has a part of the segment of its
     // own, and once these are written in too many places at a time their sectors leave the cache partly
     // filled (2^25 particles on 512^3: scatter 583 us with one copy, 798 with eight).  They live in the first
     // spectrum, which is free until the forward transform.
@@ -412,8 +411,10 @@ int bin_particles(cwthf_ctx* ctx, const float* pos, const float* mass, double ma
     // few counters (grids up to about 100^3): merge, scan and starts in one launch
     uint32_t* cursors = cp.n > 1 ? counters : ctx->dep_cursor;
     if (!scan_copies(ctx, counters, cp.n, cp.nkeys, ctx->dep_off, s)) {
-        auto merge = cp.n == 16 ? k_dep_merge<16> : (cp.n == 8 ? k_dep_merge<8> : (cp.n == 4 ? k_dep_merge<4> : k_dep_merge<2>));
-        auto starts = cp.n == 16 ? k_dep_starts<16> : (cp.n == 8 ? k_dep_starts<8> : (cp.n == 4 ? k_dep_starts<4> : k_dep_starts<2>));
+        auto merge = cp.n == 16 ? k_dep_merge<16>
+                                : (cp.n == 8 ? k_dep_merge<8> : (cp.n == 4 ? k_dep_merge<4> : k_dep_merge<2>));
+        auto starts = cp.n == 16 ? k_dep_starts<16>
+                                 : (cp.n == 8 ? k_dep_starts<8> : (cp.n == 4 ? k_dep_starts<4> : k_dep_starts<2>));
         if (cp.n > 1)
             CWTHF_LAUNCH(ctx, s, "k_dep_merge",
                          pdl(merge, kblocks, kCountThreads, 0, s)(counters, cp.nkeys, ctx->dep_count));
@@ -457,9 +458,10 @@ int deposit_impl(cwthf_ctx* ctx, const float* pos, const float* mass, double mas
                  pdl(tiles, tblocks, kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid,
                                                         ctx->d_status, tp));
     // the dense tiles' further parts (returns at once when there are none)
+    const int pblocks = int(std::min<int64_t>(8 * np / tp.split + 1, int64_t(ctx->sm_count) * kTileCtasPerSm));
     CWTHF_LAUNCH(ctx, s, "k_dep_parts",
-                 pdl(parts, int(std::min<int64_t>(8 * np / tp.split + 1, int64_t(ctx->sm_count) * kTileCtasPerSm)), kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq,
-                                                                               ctx->d_mtot, grid, ctx->d_status, tp));
+                 pdl(parts, pblocks, kTileThreads, 0, s)(a, ctx->dep_off, ctx->dep_rec, ctx->dep_mq, ctx->d_mtot, grid,
+                                                        ctx->d_status, tp));
     if (mtot && (e = cudaMemcpyAsync(mtot, ctx->d_mtot, 8, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return cuda_status(e);
     return cuda_status(cudaGetLastError());
@@ -489,7 +491,8 @@ int deposit_into_scratch(const DepositScratch& sc, const float* pos, const float
     whole.count = nullptr;
     whole.cap = 0;
     whole.split = kTileSplit;
-    pdl((mass ? k_dep_tile<false, true> : k_dep_tile<false, false>), tblocks, kTileThreads, 0, s)(a, sc.off, sc.rec, sc.mq, sc.mtot, grid, sc.status, whole);
+    const auto tiles = mass ? k_dep_tile<false, true> : k_dep_tile<false, false>;
+    pdl(tiles, tblocks, kTileThreads, 0, s)(a, sc.off, sc.rec, sc.mq, sc.mtot, grid, sc.status, whole);
     return cuda_status(cudaGetLastError());
 }
 

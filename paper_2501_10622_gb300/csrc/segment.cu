@@ -51,7 +51,8 @@ constexpr int kTileSeedCap = (kChTX / 2) * (kChTY / 2) * (kChTZ / 2);
 constexpr int kCountSeeds = 1024;
 constexpr int kSegLines = (kChTY + 2) * (kChTZ + 2);  // rows of the box, with their global indices
 static_assert(kSBytes + 2 * kTileSeedCap + 4 * kCountSeeds < 60000, "16-bit addresses");
-constexpr int kSegSmem = kSBytes + 2 * kTileSeedCap + 4 * (kCountSeeds + 1) + 4 * (kSegLines + 1);  // (a row for "no seed")
+constexpr int kSegSmem =  // (a row for "no seed")
+    kSBytes + 2 * kTileSeedCap + 4 * (kCountSeeds + 1) + 4 * (kSegLines + 1);
 
 // o / kSRow for offsets o <= kSNone
 constexpr uint32_t kYMul = 30841;
@@ -108,17 +109,18 @@ __device__ __forceinline__ void best2(float m1, int q1, float m2, int q2, bool t
 // kernel that decoded them to 32-bit pointers): 250 instructions per cell,
 // 3.34 + 4.52 ms per scale at 1024^3 and 0.26 + 0.26 ms at 384^3, against
 // 4.47 and 0.27 ms here (of which the parents take half, the chains a fifth,
-// the labels the rest).  16-bit
-// pointers in a box with a halo need no decoding and no test for neighbours
-// outside the tile, and leave room for four blocks per SM.  Two rows per warp
-// rather than four: the halo rows' x windows cost 4 instructions per cell more,
-// but half the code and 64 registers per thread keep 32 warps on an SM
-// (1024^3: 7.16 ms with four rows, 128 registers and 16 warps).
+// the labels the rest).  16-bit pointers in a box with a halo need no decoding
+// and no test for neighbours outside the tile, and leave room for four blocks
+// per SM.  Two rows per warp rather than four: the halo rows' x windows cost 4
+// instructions per cell more, but half the code and 64 registers per thread
+// keep 32 warps on an SM (1024^3: 7.16 ms with four rows, 128 registers and 16
+// warps).
 template <bool kInner>
 __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, float cwt_min, int32_t* __restrict__ label,
                                          uint32_t* __restrict__ seed_bits, uint32_t* __restrict__ seed_cells,
                                          uint32_t* __restrict__ ballots, int* status, uint32_t sb, uint32_t* n_seeds) {
-    const uint32_t seeds = sb + kSBytes, cnt = seeds + 2 * kTileSeedCap, line = cnt + 4 * (kCountSeeds + 1), none = sb + kSNone;
+    const uint32_t seeds = sb + kSBytes, cnt = seeds + 2 * kTileSeedCap, line = cnt + 4 * (kCountSeeds + 1);
+    const uint32_t none = sb + kSNone;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ntx = (N + kChTX - 1) / kChTX, nty = (N + kChTY - 1) / kChTY;
@@ -395,7 +397,11 @@ __device__ __forceinline__ void seg_tile(const float* __restrict__ C, int N, flo
         // transposed over the warp: word w (lane w) gets bit w of every lane
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) {
-            const uint32_t low = d == 16 ? 0x0000ffffu : (d == 8 ? 0x00ff00ffu : (d == 4 ? 0x0f0f0f0fu : (d == 2 ? 0x33333333u : 0x55555555u)));
+            const uint32_t low = d == 16 ? 0x0000ffffu
+                               : d == 8  ? 0x00ff00ffu
+                               : d == 4  ? 0x0f0f0f0fu
+                               : d == 2  ? 0x33333333u
+                                         : 0x55555555u;
             const uint32_t other = __shfl_xor_sync(full, flags, d);
             flags = (lane & d) ? ((flags & ~low) | ((other & ~low) >> d)) : ((flags & low) | ((other & low) << d));
         }
@@ -669,9 +675,8 @@ __global__ void k_seed_list(const uint32_t* bits, const uint32_t* prefix, int64_
 
 // Clears the slots' accumulators; the cell count starts from the tile pass's
 // count at the seed's cell when given.  With the clearing inside the list's
-// loop over the bitmap, each seed's gather and 48 bytes of
-// stores waited for the seed before it in the same word (0.68 ms per scale at
-// 1024^3, 0.14 + 0.40 now).
+// loop over the bitmap, each seed's gather and 48 bytes of stores waited for the
+// seed before it in the same word (0.68 ms per scale at 1024^3, 0.14 + 0.40 now).
 __global__ void k_seed_acc(const int32_t* seed_list, const uint32_t* seed_cells,
                            HaloAcc* __restrict__ acc, const uint32_t* n_slots) {
     pdl_wait();
@@ -733,7 +738,8 @@ int seeds_rank(cwthf_ctx* ctx, int ng, const uint32_t* seed_cells, cudaStream_t 
     int64_t cells = int64_t(ng) * ng * ng;
     int64_t nwords = (cells + 31) / 32;
     const int blocks = int(std::min<int64_t>(div_up(nwords, 256), int64_t(ctx->sm_count) * 8));
-    const int sblocks = int(std::min<int64_t>(div_up(3 * cells / 8, 256), int64_t(ctx->sm_count) * 8));  // at most a seed per 8 cells
+    // (at most a seed per 8 cells)
+    const int sblocks = int(std::min<int64_t>(div_up(3 * cells / 8, 256), int64_t(ctx->sm_count) * 8));
     int rc = scan_popc(ctx, ctx->seed_bits, ctx->seed_prefix, nwords, s);
     if (rc) return rc;
     CWTHF_LAUNCH(ctx, s, "k_seed_list",
@@ -749,7 +755,8 @@ int seeds_from_labels(cwthf_ctx* ctx, const int32_t* label, int ng, cudaStream_t
     int64_t nwords = (cells + 31) / 32;
     cudaError_t e = cudaMemsetAsync(ctx->seed_bits, 0, size_t(nwords) * 4, s);
     if (e != cudaSuccess) return cuda_status(e);
-    CWTHF_LAUNCH(ctx, s, "k_seeds_from_labels", pdl(k_seeds_from_labels, ctx->sm_count * 8, 256, 0, s)(label, cells, ctx->seed_bits, ctx->d_status));
+    CWTHF_LAUNCH(ctx, s, "k_seeds_from_labels",
+                 pdl(k_seeds_from_labels, ctx->sm_count * 8, 256, 0, s)(label, cells, ctx->seed_bits, ctx->d_status));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e);
     return seeds_rank(ctx, ng, nullptr, s);
 }
@@ -769,7 +776,8 @@ int launch_fallback(cwthf_ctx* ctx, int32_t* label, int64_t cells, cudaStream_t 
     unsigned* bar = reinterpret_cast<unsigned*>(changed + kJumpBarrier);
     int rounds = ctx->dbg_jump_rounds;
     // fewer CTAs for small grids: a cooperative launch waits until all of its CTAs fit beside what runs on
-    // other streams, and nearly always has nothing to do (a batch of 24 finds on 8 streams 2.94 -> 2.52 ms, with the launches sized by their work beside it)
+    // other streams, and nearly always has nothing to do (a batch of 24 finds on 8 streams 2.94 -> 2.52 ms,
+    // together with the launches sized by their work)
     const unsigned blocks = unsigned(std::min<int64_t>(ctx->fallback_blocks, cells / 16384 + 1));
     void* args[] = {&label, &cells, &changed, &rounds, &ctx->seed_bits, &ctx->seed_cells, &bar, &ctx->d_status};
     cudaError_t e;
@@ -799,13 +807,15 @@ int segment_impl(cwthf_ctx* ctx, const float* cwt, int ng, float cwt_min, int32_
     int blocks = ctx->sm_count * 8;
     int* changed = ctx->jump_changed;  // see kJumpWords
     // rows per turn: four tiles' where there are many turns per CTA (the barriers around a turn's table flush
-    // were the pass's largest stall with one tile: 2.14 ms per scale at 1024^3, 1.93 with four), two rows where tiles are too few to fill the
-    // GPU (64^3: 38 us with 16 whole tiles, 27 us)
+    // were the pass's largest stall with one tile: 2.14 ms per scale at 1024^3, 1.93 with four), two rows where
+    // tiles are too few to fill the GPU (64^3: 38 us with 16 whole tiles, 27 us)
     const int rows = ntiles < 2 * ctx->sm_count ? 2 : (ntiles < 16 * blocks ? kChTY : 4 * kChTY);
+    const int rblocks = int(std::min<int64_t>(blocks, ntiles * kChTY / rows));
     CWTHF_LAUNCH(ctx, s, "k_seg_resolve",
-                 pdl(k_seg_resolve, int(std::min<int64_t>(blocks, ntiles * kChTY / rows)), kResolveThreads, 0, s)(label, ng, ballots, ctx->seed_cells, changed,
-                                                                   reinterpret_cast<unsigned*>(changed + kJumpTileCounter),
-                                                                   ctx->dbg_chase_limit, rows, ctx->d_status));
+                 pdl(k_seg_resolve, rblocks, kResolveThreads, 0, s)(
+                     label, ng, ballots, ctx->seed_cells, changed,
+                     reinterpret_cast<unsigned*>(changed + kJumpTileCounter), ctx->dbg_chase_limit, rows,
+                     ctx->d_status));
     // pointer doubling and a recount for whatever the bounded walks left
     // (normally nothing: the kernel then returns at once)
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e);

@@ -13,7 +13,8 @@ CSRC = Path(pkg.__file__).parent / "csrc"
 def _run(tmp_path, body):
     """The lines that `body`, a main's statements, prints."""
     src = tmp_path / "t.cpp"
-    src.write_text('#include <cstdio>\n#include "unbind_teams.cuh"\nusing namespace cwthf;\nint main() {\n' + body + "\n}\n")
+    src.write_text('#include <cstdio>\n#include "unbind_teams.cuh"\nusing namespace cwthf;\n'
+                   "int main() {\n" + body + "\n}\n")
     subprocess.run(["g++", "-std=c++17", "-I", str(CSRC), str(src), "-o", str(tmp_path / "t")], check=True)
     return subprocess.run([str(tmp_path / "t")], check=True, capture_output=True, text=True).stdout.split("\n")[:-1]
 
