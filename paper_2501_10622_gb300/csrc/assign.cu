@@ -569,6 +569,9 @@ void launch_ids(cwthf_ctx* ctx, cudaStream_t s, int blocks, int pblocks, int64_t
 
 // ---- the multi-scale loop (Sec. 2, Fig. 1; App. B; Sec. 2.4) -----------------
 
+// Particles in flight per thread of the passes that follow an index per particle.
+constexpr int kMsIlp = 4;
+
 // Records of particles that already hold a halo id are marked in bit 63, so
 // that this scale's group sums skip them (Sec. 2 step 6: only particles
 // without a halo id are assigned).
@@ -579,9 +582,19 @@ __global__ void __launch_bounds__(kThreads) k_ms_mark(const int32_t* halo_id,
     pdl_wait();
     const int64_t total = *total_ptr;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
-        const uint32_t r = part_rec[i];
-        if (halo_id[i] >= 0 && int64_t(r) < total) rec[r] |= 1ull << 63;
+    for (int64_t i0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i0 < np; i0 += kMsIlp * stride) {
+        uint32_t r[kMsIlp];
+        unsigned long long v[kMsIlp];
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++) {
+            const int64_t i = i0 + u * stride;
+            r[u] = i < np && halo_id[i] >= 0 ? part_rec[i] : 0xffffffffu;
+        }
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++) v[u] = int64_t(r[u]) < total ? rec[r[u]] : 0ull;
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++)
+            if (int64_t(r[u]) < total) rec[r[u]] = v[u] | (1ull << 63);
     }
 }
 
@@ -593,9 +606,17 @@ __global__ void __launch_bounds__(kThreads) k_ms_pslot(const uint32_t* part_rec,
     pdl_wait();
     const int64_t total = *total_ptr;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
-        const uint32_t r = part_rec[i];
-        pslot[i] = int64_t(r) < total ? rec_slot[r] : -1;
+    for (int64_t i0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i0 < np; i0 += kMsIlp * stride) {
+        int32_t v[kMsIlp];
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++) {
+            const int64_t i = i0 + u * stride;
+            const uint32_t r = i < np ? part_rec[i] : 0xffffffffu;
+            v[u] = int64_t(r) < total ? rec_slot[r] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++)
+            if (i0 + u * stride < np) pslot[i0 + u * stride] = v[u];
     }
 }
 
@@ -742,14 +763,23 @@ __global__ void __launch_bounds__(kThreads) k_ms_ub_group(const int32_t* pslot,
                                                          int32_t* __restrict__ grp) {
     pdl_wait();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np; i += stride) {
-        const int32_t sl = pslot[i];
-        int32_t g = -1;
-        if (sl >= 0 && halo_id[i] < 0) {
-            const uint32_t r = keep_off[sl];
-            if (keep_off[sl + 1] != r) g = int32_t(r);
+    for (int64_t i0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i0 < np; i0 += kMsIlp * stride) {
+        int32_t sl[kMsIlp], id[kMsIlp], g[kMsIlp];
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++) {
+            const int64_t i = i0 + u * stride;
+            sl[u] = i < np ? pslot[i] : -1;
+            id[u] = i < np ? halo_id[i] : -1;
         }
-        grp[i] = g;
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++) {
+            const bool in = sl[u] >= 0 && id[u] < 0;
+            const uint32_t r = in ? keep_off[sl[u]] : 0u, e = in ? keep_off[sl[u] + 1] : 0u;
+            g[u] = e != r ? int32_t(r) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kMsIlp; u++)
+            if (i0 + u * stride < np) grp[i0 + u * stride] = g[u];
     }
 }
 
